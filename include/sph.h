@@ -67,7 +67,8 @@ extern "C" {
 
 /* ---- flags (sph_params.flags) ----------------------------------------------------- */
 #define SPH_FLAG_GRAPH     1u  /* sph_step runs each advection step as one CUDA graph whose
-                                  acoustic-substep loop is a device-side conditional WHILE node */
+                                  acoustic-substep loop is a device-side conditional WHILE node
+                                  (small handles: see sph_step) */
 #define SPH_FLAG_KEEP_ACC  2u  /* keep the last dv/dt of every particle for sph_get_acceleration */
 #define SPH_FLAG_FROZEN_GEOMETRY 4u  /* keep each pair's vector r_i - r_j and (dW/dr)/r from the
                                       * configuration update (after sph_advection_step's density
@@ -82,7 +83,9 @@ extern "C" {
                                       * pressure relaxation, density relaxation) separated by
                                       * grid-wide barriers whose waits are bounded (a timeout ends
                                       * the launch with SPH_E_TIMEOUT). Results are bit-identical
-                                      * to the per-launch loop. Ignored with
+                                      * to the per-launch loop. On a handle that sph_step runs
+                                      * in one launch a step, one launch runs all steps of a
+                                      * call. Ignored with
                                       * SPH_FLAG_FROZEN_GEOMETRY, SPH_FLAG_HALF_PAIR,
                                       * SPH_FLAG_DEBUG_BOUNDS or kernel
                                       * timing on; takes precedence over SPH_FLAG_GRAPH. */
@@ -241,7 +244,12 @@ int sph_acoustic_substep(sph_handle* h, int32_t* done_out, double* dt_out, void*
 /* n_advection_steps complete dual-criteria steps: build cells, advection step,
  * substeps until Dt_ad is covered. With SPH_FLAG_GRAPH each step is one CUDA
  * graph launch (the substep loop is a device-side WHILE node); otherwise the
- * host drives the loop, synchronising once per substep. Synchronous. */
+ * host drives the loop, synchronising once per substep. A handle of one small tank (2D:
+ * up to 704 particles an SM, 107,008 on GB300; 3D: 192, 29,184) without a solid, frozen
+ * geometry, half-pair evaluation, kernel timing or bounds checks runs each advection step as
+ * one cooperative launch instead, whatever the flags and the launch configuration; the
+ * results are identical bit for bit, and a call stops at the first step that fails.
+ * Synchronous. */
 int sph_step(sph_handle* h, int32_t n_advection_steps, void* stream);
 
 /* FP64 diagnostics, one sph_diag per instance into out[0..n_instances) (host). */
@@ -307,12 +315,12 @@ int sph_set_gravity(sph_handle* h, int32_t instance, const double* g, void* stre
 /* Launch configuration of the two acoustic-substep kernels: cfg[0] threads per particle
  * and cfg[1] block size of the pressure relaxation, cfg[2], cfg[3] the same for the
  * density relaxation. Threads per particle 1, 2 or 4 (the lanes of a particle split its
- * neighbour row and add their sums in a fixed order); block 128, 256 or 512; or, on a
+ * neighbour row, its terms being added in row order); block 128, 256 or 512; or, on a
  * handle of one tank, threads per particle 1 with block 896, the row-task form: one
  * resident block of 28 warps an SM, each warp taking the next 32 particles of one
  * search-cell row (the cells along x at fixed y, z) from its block's queue, the blocks
- * advancing through the cell order side by side; it computes each particle as the other
- * one-thread-per-particle variants do, so their results are identical bit for bit. Set
+ * advancing through the cell order side by side. The results of all variants are identical
+ * bit for bit. Set
  * returns SPH_E_INVALID for other values. Handles created with SPH_FLAG_FROZEN_GEOMETRY
  * run one thread per particle in 128-thread blocks whatever the configuration says. */
 int sph_get_launch_config(const sph_handle* h, int32_t* cfg);

@@ -212,6 +212,7 @@ Inst make_inst(const sph_params& p) {
   I.nu = p.nu;
   I.cfl_ad = p.cfl_ad;
   I.cfl_ac = p.cfl_ac;
+  I.dt_min = 1e-12 * p.h / p.c0;
   I.dq_d = dq;
   I.rho0_d = p.rho0;
   return I;
@@ -358,6 +359,20 @@ void enqueue_substep(sph_handle* h, cudaStream_t s, bool use_cond, int64_t* n) {
   else sph::launch_density_relaxation(h->b, s, n);
   sph_fsi_after_density(h, s, n);
   if (h->timing && !use_cond) cudaEventRecord(h->ev[2], s);
+}
+
+// Whether sph_step runs whole advection steps in one launch (sph_fused_step.cuh): one tank,
+// the ordinary pair evaluation, nothing that needs the host or other kernels between the
+// phases, and a size where that is the faster form. A further step took, per launch (graph
+// loop) and in one launch: 2D dam break 132 / 55 us at 3,200 particles, 143 / 104 at 20,000,
+// 184 / 158 at 100,352; Taylor-Green 122 / 85 us at 57,600 but 169 / 178 at 160,000; 3D dam
+// break 301 / 106 us at 2,662, 275 / 153 at 16,000, 247 / 238 at 27,648 but 291 / 332 at
+// 54,000. So the line lies where every SM's block is full: 704 particles an SM in 2D, and in
+// 3D, with four times the neighbours, 192.
+bool fused_step_fits(const sph_handle* h) {
+  const Buffers& b = h->b;
+  if (!b.step_ctl || b.geo || b.hrev || h->solid || b.dt_cap || h->timing || debug_bounds(h)) return false;
+  return b.n <= (int64_t)(b.dim == 2 ? 704 : 192) * b.n_sm && b.n_cells <= 4000000;
 }
 
 int build_graph(sph_handle* h) {
@@ -651,8 +666,11 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
     DALLOC(h, b.row_cnt, (size_t)b.n_rows);
     DALLOC(h, b.row_off, (size_t)b.n_rows + 1);
     DALLOC(h, b.row_tmp, sph::scan_tmp_elems(b.n_rows));
+    DALLOC(h, b.step_ctl, 1);
+    CK(h, cudaMemset(b.step_ctl, 0, sizeof(sph::StepCtl)));
   }
   b.rows_valid = &h->rows_valid;
+  b.counts_zero = &h->counts_zero;
   {
     int dev = 0;
     CK(h, cudaGetDevice(&dev));
@@ -866,6 +884,28 @@ int sph_acoustic_substep(sph_handle* h, int32_t* done_out, double* dt_out, void*
 int sph_step(sph_handle* h, int32_t n_advection_steps, void* stream) {
   if (!h || n_advection_steps < 0) return SPH_E_INVALID;
   cudaStream_t s = (cudaStream_t)stream;
+  if (n_advection_steps > 0 && fused_step_fits(h)) {
+    // one cooperative launch a step (with SPH_FLAG_PERSISTENT: one for all of them)
+    if (h->step_ctl_dirty) CK(h, cudaMemsetAsync(h->b.step_ctl, 0, sizeof(sph::StepCtl), s));
+    h->step_ctl_dirty = false;
+    const int per = (h->flags & SPH_FLAG_PERSISTENT) ? n_advection_steps : 1;
+    cudaError_t e = cudaSuccess;
+    int done = 0;
+    for (; done < n_advection_steps && e == cudaSuccess; done += per) e = sph::launch_fused_steps(h->b, per, s);
+    if (e == cudaSuccess) {
+      h->launches += n_advection_steps / per;
+      h->rows_valid = false;                     // the row pieces follow the new order
+      h->cells_valid = true;
+      const int r = sync_status(h, s);
+      if (r != SPH_OK) {                         // a failed launch may leave its counters behind
+        h->step_ctl_dirty = true;
+        h->counts_zero = false;
+      }
+      return r;
+    }
+    cudaGetLastError();                          // no room for a cooperative launch: the general paths
+    if (done > per) return cuda_fail(h, e, "advection step launch");
+  }
   if ((h->flags & SPH_FLAG_PERSISTENT) && !h->timing && !debug_bounds(h) && !h->b.geo && !h->b.hrev && !h->solid) {
     // each advection step: the configuration update and the advection step's kernels, then
     // one cooperative launch for all of its substeps
@@ -889,6 +929,7 @@ int sph_step(sph_handle* h, int32_t n_advection_steps, void* stream) {
     CK(h, cudaMemcpyAsync(h->hglob, h->b.glob, sizeof(Global), cudaMemcpyDeviceToHost, s));
     CK(h, cudaStreamSynchronize(s));
     long long sub0 = h->hglob->substeps;
+    h->counts_zero = false;                      // the graph's sort leaves its counts
     for (int k = 0; k < n_advection_steps; ++k) CK(h, cudaGraphLaunch(h->gexec, s));
     int r = sync_status(h, s);
     h->graph_kernels += (int64_t)n_advection_steps * h->graph_fixed +

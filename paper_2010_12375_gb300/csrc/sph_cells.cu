@@ -14,7 +14,7 @@
 //             sphere's chord), about 42 % of the candidates of a 3^D scan of 2h cells
 #include <cstdio>
 
-#include "sph_kernels.h"
+#include "sph_cells.cuh"
 
 namespace sph {
 
@@ -27,11 +27,6 @@ constexpr int kScanTile = kScanThreads * kScanItems;
 
 inline unsigned grid_for(int64_t n, int block = kBlock) {
   return (unsigned)((n + block - 1) / block);
-}
-
-__device__ __forceinline__ void raise_error(Global* g, int bit, long long idx) {
-  int old = atomicOr(&g->err, bit);
-  if (old == 0) g->bad_index = idx;
 }
 
 // ---------------------------------------------------------------- scan ---------------
@@ -138,21 +133,8 @@ __global__ void k_hash(int64_t n, const int4* __restrict__ P, const int* __restr
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const Inst& I = inst[inst_of ? inst_of[i] : 0];
-  int4 p = P[i];
-  int q[3] = {p.x, p.y, p.z};
-  long long c = 0, stride = 1;
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    int ca = q[a] >> I.sbits;                       // search cell: half a cell per axis
-    if (ca < 0 || ca >= I.scell[a]) {
-      raise_error(g, ERR_DOMAIN, i);
-      ca = ca < 0 ? 0 : I.scell[a] - 1;
-    }
-    c += (long long)ca * stride;
-    stride *= I.scell[a];
-  }
-  c += I.cell_base;
-  cell[i] = (uint32_t)c;
+  const uint32_t c = hash_cell<D>(I, P[i], i, g);
+  cell[i] = c;
   rank[i] = atomicAdd(&count[c], 1u);
 }
 
@@ -212,136 +194,6 @@ __global__ void k_copy_back(int64_t n, const int4* __restrict__ Pin, const float
 }
 
 // ---------------------------------------------------------------- neighbours ---------
-__device__ __forceinline__ int wrap_cell(int c, int n) { return c < 0 ? c + n : (c >= n ? c - n : c); }
-
-// Distance (quanta) from a point at offset o inside its search cell (width S) to the
-// slab of the cell d rows away; exact integers below 2^23, so exact in FP32.
-__device__ __forceinline__ float slab_gap(int d, float o, float S) {
-  return d > 0 ? (float)d * S - o : (d < 0 ? o + (float)(-d - 1) * S + 1.0f : 0.0f);
-}
-
-// Flattened search cell of a particle (clamped to its tank's grid).
-template <int D>
-__device__ __forceinline__ long long search_cell(const Inst& I, const int4& p) {
-  const int sb = I.sbits;
-  const int cx = min(max(p.x >> sb, 0), I.scell[0] - 1);
-  const int cy = min(max(p.y >> sb, 0), I.scell[1] - 1);
-  const int cz = D == 3 ? min(max(p.z >> sb, 0), I.scell[2] - 1) : 0;
-  return I.cell_base + ((long long)cz * I.scell[1] + cy) * I.scell[0] + cx;
-}
-
-// Visit the search-cell runs that can hold a neighbour of the particle at p: for every
-// row (dy, dz) in [-2, 2]^(D-1) whose slab lies closer than 2h, the x cells that meet the
-// sphere's chord in that slab. Within a row the cells of a run are one contiguous slot
-// range; a periodic x axis splits a run that crosses the edge into two. The row test and
-// the chord are evaluated in FP32 against R2 (1 + 2^-20), a margin above every rounding
-// error of the squares, so they only ever err towards visiting more: a particle j in a
-// skipped row or cell has sum (q_i - q_j)^2 >= R2 and is not a neighbour.
-template <int D, bool PER, typename F>
-__device__ __forceinline__ void for_neighbour_runs(const Inst& I, const int4& p,
-                                                   const uint32_t* __restrict__ start, F&& visit) {
-  const int sb = I.sbits;
-  const float S = (float)(1 << sb);
-  const int nx = I.scell[0], ny = I.scell[1], nz = D == 3 ? I.scell[2] : 1;
-  const int cy = min(max(p.y >> sb, 0), ny - 1);
-  const int cz = D == 3 ? min(max(p.z >> sb, 0), nz - 1) : 0;
-  const float oy = (float)(p.y - (cy << sb));
-  const float oz = D == 3 ? (float)(p.z - (cz << sb)) : 0.0f;
-  const float R2m = (float)I.R2 * (1.0f + 9.5367431640625e-07f);
-  const long long base = I.cell_base;
-  for (int dz = (D == 3 ? -2 : 0); dz <= (D == 3 ? 2 : 0); ++dz) {
-    int z = 0;
-    float gz2 = 0.0f;
-    if (D == 3) {
-      const int zu = cz + dz;
-      if (PER && I.period[2]) z = wrap_cell(zu, nz);
-      else if (zu < 0 || zu >= nz) continue;
-      else z = zu;
-      const float gz = fmaxf(slab_gap(dz, oz, S), 0.0f);
-      gz2 = gz * gz;
-      if (gz2 >= R2m) continue;
-    }
-    for (int dy = -2; dy <= 2; ++dy) {
-      const int yu = cy + dy;
-      int y;
-      if (PER && I.period[1]) y = wrap_cell(yu, ny);
-      else if (yu < 0 || yu >= ny) continue;
-      else y = yu;
-      const float gy = fmaxf(slab_gap(dy, oy, S), 0.0f);
-      const float rem = R2m - gz2 - gy * gy;
-      if (rem <= 0.0f) continue;
-      // |dx| of a neighbour is below sqrt(rem); rsqrt-based root within 2 quanta
-      const long long xr = (long long)(rem * rsqrtf(rem)) + 2;
-      int xa = (int)(((long long)p.x - xr) >> sb), xb = (int)(((long long)p.x + xr) >> sb);
-      const long long row = base + ((long long)z * ny + y) * nx;
-      if (PER && I.period[0]) {
-        if (xa < 0) {
-          visit(start[row + xa + nx], start[row + nx]);
-          xa = 0;
-        }
-        if (xb >= nx) {
-          visit(start[row + xa], start[row + nx]);
-          visit(start[row], start[row + xb - nx + 1]);
-          continue;
-        }
-      } else {
-        xa = max(xa, 0);
-        xb = min(xb, nx - 1);
-        if (xa > xb) continue;
-      }
-      visit(start[row + xa], start[row + xb + 1]);
-    }
-  }
-}
-
-// Appends neighbour indices to one particle's quad-interleaved row (slot s of particle i
-// at ((s >> 2) n + i) 4 + (s & 3)) with a running pointer instead of a product per slot.
-struct RowWriter {
-  int* p;
-  int64_t stride;   // 4n ints between consecutive quads of one particle
-  int sub, count, cap;
-  __device__ __forceinline__ RowWriter(int* nbr, int64_t n, int64_t i, int slot0, int cap_)
-      : p(nbr + ((int64_t)(slot0 >> 2) * n + i) * 4), stride(4 * n), sub(slot0 & 3), count(0), cap(cap_ - slot0) {}
-  __device__ __forceinline__ void push(int j, bool& overflow) {
-    if (count < cap) {
-      p[sub] = j;
-      if (++sub == 4) {
-        sub = 0;
-        p += stride;
-      }
-    } else {
-      overflow = true;
-    }
-    ++count;
-  }
-};
-
-// Candidate test: the squared distance in FP32 from exactly converted integer
-// differences (error < 3 ulp); only inside a +-2^-20 band around the threshold is
-// the exact integer test needed, so the decision is always the integer one.
-// Two candidates at once in the lanes of packed FP32 instructions. The exact test sits
-// behind a warp vote: a warp takes it only when one of its candidates falls in the band
-// (measured 0.1 ms faster per build at 8M than selecting between the two tests).
-template <int D, bool PER>
-__device__ __forceinline__ void within_fast2(const int4& p, const int4& a, const int4& b, const Inst& I,
-                                             float lo, float hi, bool& in_a, bool& in_b) {
-  const float2 M = f2(-kMagic);
-  const float2 dx = add2(make_float2(biased_diff<PER>(p.x, a.x, I.period[0]), biased_diff<PER>(p.x, b.x, I.period[0])), M);
-  const float2 dy = add2(make_float2(biased_diff<PER>(p.y, a.y, I.period[1]), biased_diff<PER>(p.y, b.y, I.period[1])), M);
-  float2 d2 = fma2(dx, dx, mul2(dy, dy));
-  if (D == 3) {
-    const float2 dz = add2(make_float2(biased_diff<PER>(p.z, a.z, I.period[2]), biased_diff<PER>(p.z, b.z, I.period[2])), M);
-    d2 = fma2(dz, dz, d2);
-  }
-  in_a = d2.x < lo;
-  in_b = d2.y < lo;
-  const bool ea = !in_a && d2.x < hi, eb = !in_b && d2.y < hi;
-  if (__any_sync(__activemask(), ea || eb)) {
-    if (ea) in_a = within<D>(p, a, I);
-    if (eb) in_b = within<D>(p, b, I);
-  }
-}
-
 template <int D, bool PER>
 __global__ void __launch_bounds__(kBlock)
 k_neighbours(int64_t n, const int4* __restrict__ P, const int* __restrict__ inst_of,
@@ -515,6 +367,7 @@ __global__ void k_row_fill(const Inst I, int64_t n_rows, const uint32_t* __restr
 
 void launch_hash(const Buffers& b, cudaStream_t s, int64_t* launches) {
   cudaMemsetAsync(b.count, 0, sizeof(uint32_t) * b.n_cells, s);
+  if (b.counts_zero) *b.counts_zero = false;
   if (b.n == 0) return;
   if (b.dim == 2)
     k_hash<2><<<grid_for(b.n), kBlock, 0, s>>>(b.n, b.PS, b.inst_of, b.inst, b.cell, b.count, b.rank, b.glob);

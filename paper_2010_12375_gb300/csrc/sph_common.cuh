@@ -54,6 +54,7 @@ struct Inst {
   long long fluid_begin, fluid_end;
   long long wall_begin, wall_end;
   double h_d, c0_d, u_ref, nu, cfl_ad, cfl_ac;
+  double dt_min;                 // 1e-12 h / c0: a smaller acoustic step is an error
   double lo[3];                  // cell-grid origin
   double dq_d;                   // position quantum in double precision
   double rho0_d;

@@ -1,0 +1,9 @@
+// The one-launch step of 3D tanks without a periodic axis (sph_fused_step.cuh); a translation unit
+// of its own so that the four compile in parallel.
+#include "sph_fused_step.cuh"
+
+namespace sph {
+cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s) {
+  return launch_d<3, false>(b, n_steps, clear_counts, s);
+}
+}  // namespace sph

@@ -39,6 +39,8 @@ struct sph_handle {
   int64_t timed[2] = {0, 0};
   bool cells_valid = false;
   bool rows_valid = false;         // row pieces match the current cell order (row-task form)
+  bool counts_zero = false;        // the cell counts are all zero (left so by the one-launch step)
+  bool step_ctl_dirty = false;     // a one-launch step failed: clear its control block first
   float4* grad = nullptr;          // [3][n] gradient sums of sph_gradient_diagnostics (lazily)
   sph_solid* solid = nullptr;      // attached elastic solid (sph_solid_create), or NULL
 };

@@ -25,6 +25,16 @@ struct GridBarrier {
   int active[2];       // per substep (alternating): some tank needs another substep
 };
 
+// Barrier, time-step control and scan sums of the one-launch step (device memory).
+constexpr int kStepMaxGrid = 1024;
+struct StepCtl {
+  unsigned count;            // arrivals of the barriers so far (zero between launches)
+  unsigned exits;            // blocks that have left the launch
+  unsigned vm[2];            // bits of max |v|^2 of a substep (alternating)
+  int stop;                  // an earlier step of the launch failed
+  unsigned sums[kStepMaxGrid];   // particles in each block's cells
+};
+
 // Device buffers of one handle. Fluid arrays are indexed in cell-sorted order.
 struct Buffers {
   LaunchCfg cfg;
@@ -63,6 +73,7 @@ struct Buffers {
   uint32_t* nbc = nullptr;        // [n] fluid count | wall count << 16
   float4* geo = nullptr;          // [cap][n] frozen r_i - r_j and (dW/dr)/r per slot (or NULL)
   GridBarrier* pbar = nullptr;    // [1] persistent substep loop
+  StepCtl* step_ctl = nullptr;    // [1] one-launch step (NULL: handle of several tanks)
   double* dt_cap = nullptr;       // [n_inst] cap on the acoustic step (0 = none), or NULL
   // half-pair evaluation (or NULL): per-slot shares [cap][n], per-particle partial sums [n],
   // reverse slots [cap][n] (slot of j in i's row for each slot of j's row holding i < j)
@@ -77,6 +88,7 @@ struct Buffers {
   uint32_t* row_tmp = nullptr;    // scan scratch
   int64_t n_rows = 0, row_task_cap = 0;
   bool* rows_valid = nullptr;     // host flag: the pieces match the current cell order
+  bool* counts_zero = nullptr;    // host flag: count is all zero (left so by the one-launch step)
   int n_sm = 0;                   // SMs of the device (grid of the row-task form)
 };
 
@@ -125,6 +137,20 @@ void launch_density_relaxation(const Buffers& b, cudaStream_t s, int64_t* launch
 // every acoustic substep of the current advection step for every tank in one cooperative
 // launch (not with the frozen-geometry reading); *grid_out receives the blocks launched
 cudaError_t launch_substeps_persistent(const Buffers& b, cudaStream_t s, int* grid_out);
+// n_steps whole advection steps of a handle of one tank in one cooperative launch (not with
+// the frozen-geometry or half-pair evaluation, nor a solid)
+// (clear_counts: the cell counts are not all zero yet)
+cudaError_t launch_fused_2d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
+cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);   // a periodic axis
+cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
+cudaError_t launch_fused_3dp(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
+inline cudaError_t launch_fused_steps(const Buffers& b, int n_steps, cudaStream_t s) {
+  auto f = b.dim == 2 ? (b.any_periodic ? launch_fused_2dp : launch_fused_2d)
+                      : (b.any_periodic ? launch_fused_3dp : launch_fused_3d);
+  const cudaError_t e = f(b, n_steps, *b.counts_zero ? 0 : 1, s);
+  if (e == cudaSuccess) *b.counts_zero = true;   // a launch leaves the cell counts zero
+  return e;
+}
 // half-pair evaluation: the reverse-slot map of the current table (after each build), and
 // one relaxation (pressure or density) as its two passes
 void launch_reverse_slots(const Buffers& b, cudaStream_t s, int64_t* launches);

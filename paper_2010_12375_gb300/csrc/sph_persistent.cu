@@ -71,8 +71,8 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
       if (dtd == 0.0) valid = false;
       const Inst& I = UNI ? Ip : inst[k];
       bool writer;
-      const float v2 = pr_particle<D, PER, 1, false, TV, const int4*, const float4*>(
-          I, i, 0, valid, dtd, nullptr, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
+      const float v2 = pr_particle<D, PER, false, TV, const int4*, const float4*>(
+          I, i, valid, dtd, nullptr, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
       warp_vmax(v2, writer, k, ctrl);
     }
     if (!grid_barrier(bar, g)) return;
@@ -84,7 +84,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
       if (dtd == 0.0) valid = false;
       if (!valid) continue;
       const Inst& I = UNI ? Ip : inst[k];
-      dr_particle<D, PER, 1, false, const int4*, const float4*>(I, i, 0, true, dtd, nullptr, n, PH, VH, PS, VS,
+      dr_particle<D, PER, false, const int4*, const float4*>(I, i, true, dtd, nullptr, n, PH, VH, PS, VS,
                                                                mass, nbr, nbc, WP, WN, g);
     }
     if (!grid_barrier(bar, g)) return;

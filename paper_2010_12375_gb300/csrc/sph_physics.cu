@@ -17,6 +17,7 @@
 #include <cmath>
 
 #include "sph_ctrl.cuh"
+#include "sph_density.cuh"
 #include "sph_kernels.h"
 
 namespace sph {
@@ -221,20 +222,10 @@ __global__ void k_reset_vmax(int n_inst, Ctrl* ctrl) {
   for (int k = threadIdx.x; k < n_inst; k += blockDim.x) ctrl[k].vmax2 = 0u;
 }
 
-// Eq. dt-advection: Dt_ad = CFL_ad min(h / max(|v|max, U_ref), h^2 / nu).
+// Eq. dt-advection for every tank (sph_ctrl.cuh).
 __global__ void k_dt_advection(int n_inst, const Inst* __restrict__ inst, Ctrl* ctrl, Global* g) {
   for (int k = threadIdx.x; k < n_inst; k += blockDim.x) {
-    const Inst& I = inst[k];
-    Ctrl& C = ctrl[k];
-    double vmax = sqrt((double)__uint_as_float(C.vmax2));
-    double dt = I.h_d / fmax(vmax, I.u_ref);
-    if (I.nu > 0.0) dt = fmin(dt, I.h_d * I.h_d / I.nu);
-    C.dt_ad = I.cfl_ad * dt;
-    C.tau = 0.0;
-    C.done = 0;
-    C.dt = 0.0;
-    C.sub_in_step = 0;
-    C.adv_steps += 1;
+    dt_advection_one(inst[k], ctrl[k]);
   }
   if (threadIdx.x == 0) g->active = 1;
 }
@@ -253,30 +244,6 @@ __global__ void k_dt_acoustic(int n_inst, const Inst* __restrict__ inst, Ctrl* c
 }
 
 // ---------------------------------------------------------------- density -------------
-// W of two pairs at once from their packed squared distances; lanes with mask 0 add 0.
-__device__ __forceinline__ float2 kernel_W2(float2 r2, float inv_h, float w_a) {
-  const float2 q = mul2(mul2(r2, rsqrt2(fma2(r2, f2(1.0f), f2(1e-30f)))), f2(inv_h));
-  const float2 t = max2(fma2(q, f2(-0.5f), f2(1.0f)), 0.0f);
-  const float2 t2 = mul2(t, t);
-  return mul2(mul2(f2(w_a), mul2(t2, t2)), fma2(q, f2(2.0f), f2(1.0f)));
-}
-
-template <int D, bool PER>
-__device__ __forceinline__ float2 pair_r2(const int4& p, const int4& a, const int4& b, const Inst& I) {
-  const float2 M = f2(-kMagic), DQ = f2(I.dq);
-  const float2 dx = mul2(add2(make_float2(biased_diff<PER>(p.x, a.x, I.period[0]), biased_diff<PER>(p.x, b.x, I.period[0])), M), DQ);
-  const float2 dy = mul2(add2(make_float2(biased_diff<PER>(p.y, a.y, I.period[1]), biased_diff<PER>(p.y, b.y, I.period[1])), M), DQ);
-  float2 r2 = fma2(dx, dx, mul2(dy, dy));
-  if (D == 3) {
-    const float2 dz = mul2(add2(make_float2(biased_diff<PER>(p.z, a.z, I.period[2]), biased_diff<PER>(p.z, b.z, I.period[2])), M), DQ);
-    r2 = fma2(dz, dz, r2);
-  }
-  return r2;
-}
-
-// Eq. eqrhosum / Eq. eqrhosumnosurface: rho = rho0 sum W / sum W0 (with max(rho*, .) for a
-// free surface), sum over self, fluid and wall neighbours. The Kahan sum starts from
-// W(0) - sumW0 so it holds the deviation rho/rho0 - 1 with its own relative precision.
 template <int D, bool PER>
 __global__ void __launch_bounds__(kBlock)
 k_density(int64_t n, int4* P, const int* __restrict__ inst_of, const Inst* __restrict__ inst,
@@ -285,37 +252,7 @@ k_density(int64_t n, int4* P, const int* __restrict__ inst_of, const Inst* __res
   if (i >= n) return;
   const Inst& I = inst[inst_index(inst_of, i)];
   const int4 pi = P[i];
-  const uint32_t c = nbc[i];
-  const int nf = (int)(c & 0xffffu), nw = (int)(c >> 16);
-  float2 s = make_float2(I.sig_hi, 0.0f), nc = f2(0.0f);
-  kahan2(s, nc, make_float2(I.sig_lo, 0.0f), f2(1.0f));
-  const int4* __restrict__ nb4 = reinterpret_cast<const int4*>(nbr);
-  const int nq = (nf + 3) >> 2;
-  int4 nxt = nq ? nb4[i] : make_int4(0, 0, 0, 0);
-  for (int q = 0; q < nq; ++q) {
-    const int4 cq = nxt;
-    if (q + 1 < nq) nxt = nb4[(int64_t)(q + 1) * n + i];   // next quad in flight
-    const int sl = q << 2;
-    const int j1 = sl + 1 < nf ? cq.y : cq.x, j2 = sl + 2 < nf ? cq.z : cq.x, j3 = sl + 3 < nf ? cq.w : cq.x;
-    const int4 a0 = P[cq.x], a1 = P[j1], a2 = P[j2], a3 = P[j3];
-    const float2 m01 = make_float2(1.0f, sl + 1 < nf ? 1.0f : 0.0f);
-    const float2 m23 = make_float2(sl + 2 < nf ? 1.0f : 0.0f, sl + 3 < nf ? 1.0f : 0.0f);
-    kahan2(s, nc, kernel_W2(pair_r2<D, PER>(pi, a0, a1, I), I.inv_h, I.w_a), m01);
-    kahan2(s, nc, kernel_W2(pair_r2<D, PER>(pi, a2, a3, I), I.inv_h, I.w_a), m23);
-  }
-  const int q0 = wall_slot0(nf) >> 2, nwq = (nw + 3) >> 2;
-  for (int q = 0; q < nwq; ++q) {
-    const int4 cq = nb4[(int64_t)(q0 + q) * n + i];
-    const int sl = q << 2;
-    const int w1 = sl + 1 < nw ? cq.y : cq.x, w2 = sl + 2 < nw ? cq.z : cq.x, w3 = sl + 3 < nw ? cq.w : cq.x;
-    const int4 a0 = WP[cq.x], a1 = WP[w1], a2 = WP[w2], a3 = WP[w3];
-    const float2 m01 = make_float2(1.0f, sl + 1 < nw ? 1.0f : 0.0f);
-    const float2 m23 = make_float2(sl + 2 < nw ? 1.0f : 0.0f, sl + 3 < nw ? 1.0f : 0.0f);
-    kahan2(s, nc, kernel_W2(pair_r2<D, PER>(pi, a0, a1, I), I.inv_h, I.w_a), m01);
-    kahan2(s, nc, kernel_W2(pair_r2<D, PER>(pi, a2, a3, I), I.inv_h, I.w_a), m23);
-  }
-  float dev = I.rho0_over_sigma0 * ((s.x + nc.x) + (s.y + nc.y));   // rho0 sumW/sumW0 - rho0
-  if (I.free_surface) dev = fmaxf(i2f(pi.w), dev);
+  const float dev = density_dev<D, PER, 1>(I, i, 0, pi, nbc[i], n, P, reinterpret_cast<const int4*>(nbr), WP, nullptr);
   reinterpret_cast<int*>(P + i)[3] = f2i(dev);        // only .w changes; others read .xyz
 }
 
@@ -328,34 +265,8 @@ k_viscous(int64_t n, const int4* __restrict__ P, const float4* __restrict__ V,
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const Inst& I = inst[inst_index(inst_of, i)];
-  const int4 pi = P[i];
-  const float4 vi = V[i];
-  float rho_i = I.rho0 + i2f(pi.w);
-  int nf = (int)(nbc[i] & 0xffffu);
-  float ax = 0.f, ay = 0.f, az = 0.f;
-  if (I.eta > 0.0f) {
-    for (int k = 0; k < nf; ++k) {
-      int j = nbr[slot_index(n, i, k)];
-      const int4 pj = P[j];
-      const float4 vj = V[j];
-      float dx = (float)wrap_diff(pi.x - pj.x, I.period[0]) * I.dq;
-      float dy = (float)wrap_diff(pi.y - pj.y, I.period[1]) * I.dq;
-      float r2 = dx * dx + dy * dy;
-      if (D == 3) {
-        float dz = (float)wrap_diff(pi.z - pj.z, I.period[2]) * I.dq;
-        r2 += dz * dz;
-      }
-      if (!(r2 < I.four_h2) || r2 == 0.0f) continue;
-      float fw = kernel_dW_over_r(sqrtf(r2), I);            // (dW/dr)/r
-      float mj = mass ? mass[j] : I.mass;
-      float f = mj / (I.rho0 + i2f(pj.w)) * fw;
-      ax += f * (vi.x - vj.x);
-      ay += f * (vi.y - vj.y);
-      if (D == 3) az += f * (vi.z - vj.z);
-    }
-  }
-  float s = 2.0f * I.eta / rho_i;
-  acc_prior[i] = make_float4(s * ax, s * ay, s * az, 0.0f);
+  acc_prior[i] = viscous_acc<D, 1>(I, i, 0, (int)(nbc[i] & 0xffffu), n, P, V, mass,
+                                   reinterpret_cast<const int4*>(nbr), nullptr);
 }
 
 }  // namespace

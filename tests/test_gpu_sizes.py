@@ -58,3 +58,101 @@ def test_weight_gradients_at_tile_edges(sph, nx, ny):
             assert rel_l2(got, dW[k]) < 1e-3, k        # the bound the weight gradients are held to
     sph.sph_learned_destroy(net)
     sim.close()
+
+
+def _fused_case(name):
+    """Tanks that sph_step runs in one launch a step, at the lane counts' edges (8, 4, 2, 1
+    lanes a particle by the particles an SM holds) and with each of the step's options."""
+    if name.startswith("2d"):
+        nx, ny = {"2d_one": (1, 1), "2d_three": (3, 1), "2d_9728": (128, 76), "2d_9729": (423, 23),
+                  "2d_19456": (152, 128), "2d_30600": (180, 170), "2d_visc": (37, 29)}[name]
+        prob = wk.dam_break(dim=2, H=ny * 0.02, L=nx * 0.02, dp=0.02, tank=max(nx, ny, 12) * 0.02 + 0.3)
+        if name == "2d_visc":
+            prob.nu = 0.01
+    elif name.startswith("tg"):
+        prob = wk.taylor_green({"tg_48": 48, "tg_230": 230}[name])
+    elif name == "box3d":
+        prob = wk.periodic_box(dim=3, n=12, seed=2)
+    else:
+        prob = wk.dam_break_3d({"3d_11": 11, "3d_17": 17, "3d_24": 24}[name])
+        prob.nu = 0.002 if name == "3d_17" else 0.0
+    if name in ("2d_three", "3d_11"):                # masses that differ: a per-particle array
+        prob.mass = prob.mass * np.random.default_rng(3).uniform(0.95, 1.05, prob.mass.shape)
+    return prob
+
+
+@pytest.mark.parametrize("case", ["2d_one", "2d_three", "2d_9728", "2d_9729", "2d_19456", "2d_30600", "2d_visc",
+                                  "tg_48", "tg_230", "box3d", "3d_11", "3d_17", "3d_24"])
+def test_one_launch_step_equals_the_per_launch_loop(sph, case):
+    # every sum of the one-launch step adds the same terms in the same order: state, table,
+    # acceleration, clock and substep count agree bit for bit (kernel timing keeps sph_step on
+    # the per-launch kernels), in the host, graph and all-steps-in-one-launch forms
+    prob = _fused_case(case)
+    rng = np.random.default_rng(7)
+    x = prob.pos + rng.uniform(-0.1, 0.1, prob.pos.shape) * prob.dp
+    v = prob.vel + rng.uniform(-0.2, 0.2, prob.vel.shape)
+    if np.any(prob.periodic[:prob.dim]):
+        x = np.mod(x, 1.0)
+    out = []
+    for flags, timing in ((0, True), (0, False), (sph.SPH_FLAG_GRAPH, False), (sph.SPH_FLAG_PERSISTENT, False)):
+        sim = sph.Simulation(prob, flags=flags | sph.SPH_FLAG_KEEP_ACC)
+        sim.set_state(x, v, prob.rho, t=0.0)
+        sph.sph_set_kernel_timing(sim.handle, timing)
+        before = sim.kernel_launches()
+        sim.step(3)
+        launches = sim.kernel_launches() - before
+        assert launches > 20 if timing else launches == (1 if flags == sph.SPH_FLAG_PERSISTENT else 3)
+        d = sim.diagnostics()
+        fc, wc, fi, wi = sim.neighbours()
+        rows = [np.concatenate([fi[i, :fc[i]], wi[i, :wc[i]]]) for i in range(0, sim.n, max(1, sim.n // 500))]
+        out.append((*sim.state(), sim.acceleration(), sim.permutation(), fc, wc, np.concatenate(rows),
+                    np.array([d["substeps"], d["t"], d["dt_ad"], d["advection_steps"]])))
+        sim.step(1)                                  # and on from there
+        out[-1] = out[-1] + sim.state()
+        sim.close()
+    for o_ in out[1:]:
+        for a, b in zip(out[0], o_):
+            np.testing.assert_array_equal(a, b)
+
+
+def test_one_launch_step_reports_errors_and_goes_on(sph):
+    # a row beyond the capacity and a particle outside the grid: the codes of the other loops,
+    # and the handle steps on after a new state
+    prob = wk.dam_break_2d(n_per_H=20)
+    sim = sph.Simulation(prob, capacity=8)
+    with pytest.raises(sph.SphError) as e:
+        sim.step(2)
+    assert e.value.code == sph.SPH_E_CAPACITY
+    sim.close()
+    ref, sim = sph.Simulation(prob), sph.Simulation(prob)
+    x = prob.pos.copy()
+    x[5, 0] = prob.hi[0] + 1.0
+    sim.set_state(x, prob.vel, prob.rho, t=0.0)
+    with pytest.raises(sph.SphError) as e:
+        sim.step(2)
+    assert e.value.code == sph.SPH_E_DOMAIN
+    sph.sph_clear_error(sim.handle)
+    for s in (ref, sim):
+        s.set_state(prob.pos, prob.vel, prob.rho, t=0.0)
+        s.step(3)
+    for a, b in zip(ref.state(), sim.state()):
+        np.testing.assert_array_equal(a, b)
+    ref.close()
+    sim.close()
+
+
+@pytest.mark.parametrize("case", ["3d_11", "2d_visc"])
+def test_threads_per_particle_change_no_bit(sph, case):
+    # the lanes of a particle add its terms in row order (kernel timing: per-launch kernels)
+    prob = _fused_case(case)
+    out = []
+    for cfg in ([1, 128, 1, 128], [2, 128, 4, 256], [4, 512, 2, 512]):
+        sim = sph.Simulation(prob)
+        sph.sph_set_launch_config(sim.handle, cfg)
+        sph.sph_set_kernel_timing(sim.handle, True)
+        sim.step(3)
+        out.append(sim.state())
+        sim.close()
+    for o_ in out[1:]:
+        for a, b in zip(out[0], o_):
+            np.testing.assert_array_equal(a, b)
