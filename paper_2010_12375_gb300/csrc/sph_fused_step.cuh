@@ -26,15 +26,15 @@
 // and 184 us in the graph loop's launches), of the 3D one 153 us at 16,000 (275 us).
 //
 // Memory ordering: a phase gathers what other blocks wrote in the one before, so everything
-// written here is read through plain coherent loads, and a barrier fences on both sides. A
-// block that waits longer than about a second at a barrier sets ERR_TIMEOUT and returns, and
-// the others then time out at the same barrier, so the launch always ends.
+// written here is read through plain coherent loads (sph_grid_sync.cuh has the barrier and
+// its bounded wait).
 #pragma once
 #include <algorithm>
 
 #include "sph_cells.cuh"
 #include "sph_ctrl.cuh"
 #include "sph_density.cuh"
+#include "sph_grid_sync.cuh"
 #define SPH_HAVE_RAISE_ERROR
 #include "sph_relax.cuh"
 
@@ -45,31 +45,6 @@ namespace {
 template <int LPP>
 constexpr int kStepThreads = LPP <= 2 ? 704 : 512;   // most work threads: 88 and 96 registers
 constexpr int kStepMaxWarps = 704 / 32 + 1;
-constexpr unsigned kStepSpinLimit = 1u << 21;    // polls of half a microsecond: about a second
-
-// Arrive and wait for every block. target counts the arrivals of the barriers so far (thread
-// 0's copy is the one used). False: a wait gave up, the caller returns.
-__device__ __forceinline__ bool step_barrier(StepCtl* c, unsigned& target, Global* g) {
-  __shared__ int ok;
-  __syncthreads();
-  target += gridDim.x;
-  if (threadIdx.x == 0) {
-    ok = 1;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;\n" ::"l"(&c->count) : "memory");
-    unsigned spins = 0, seen;
-    while (true) {
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n" : "=r"(seen) : "l"(&c->count) : "memory");
-      if ((int)(seen - target) >= 0) break;
-      if (++spins > kStepSpinLimit) {
-        atomicOr(&g->err, ERR_TIMEOUT);
-        ok = 0;
-        break;
-      }
-    }
-  }
-  __syncthreads();
-  return ok != 0;
-}
 
 // Sum of v over the block, and the exclusive prefix of this thread.
 __device__ __forceinline__ uint32_t block_scan(uint32_t v, uint32_t* warp_tot, uint32_t* total) {
@@ -313,7 +288,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
   if (threadIdx.x == 0) C = b.ctrl[0];
   if (clear_counts) {
     for (int64_t k = tid; k < b.n_cells; k += threads) b.count[k] = 0u;
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
   }
   for (int st = 0; st < n_steps; ++st) {
     // ---- cells: hash, scan, sort by (cell, id)
@@ -322,7 +297,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       b.cell[i] = cell;
       b.rank[i] = atomicAdd(&b.count[cell], 1u);
     }
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     uint32_t sum = 0, total;
     for (int64_t k = c0 + 4 * threadIdx.x; k < c1; k += 4 * blockDim.x) {
       const uint4 v = load4(b.count, k, c1);
@@ -333,7 +308,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       c->sums[blockIdx.x] = total;
       if (blockIdx.x == 0) c->stop = st > 0 && *(volatile int*)&g->err != 0;
     }
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     if (c->stop) break;                          // an earlier step failed
     uint32_t before = 0, run;
     for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) before += c->sums[k];
@@ -351,13 +326,13 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       run += total;
     }
     if (tid == 0) b.fstart[b.n_cells] = (uint32_t)n;
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     for (int64_t i = tid; i < n; i += threads) {
       const uint32_t d = b.fstart[b.cell[i]] + b.rank[i];
       b.key[d] = b.id[i];
       b.src[d] = (int)i;
     }
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     for (int64_t d = tid; d < n; d += threads) { // place in the cell: the mates with smaller ids
       const int s = b.src[d], key = b.key[d];
       const int4 p = b.PS[s];
@@ -370,7 +345,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       id_new[t] = key;
       if (b.mass) b.mass_tmp[t] = b.mass[s];
     }
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     // ---- neighbours and density, a block's share of the particles at a time; Dt_ad and the
     // first dt beside them
     if (control) {
@@ -402,7 +377,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       }
     }
     if (tid == 0) c->vm[0] = 0u;
-    if (!step_barrier(c, target, g)) return;
+    if (!grid_barrier(&c->count, target, g)) return;
     if (b.acc_prior) {   // read back by the lane that wrote it: no barrier
       for (int64_t i = first; i < n; i += step) {
         const float4 a = viscous_acc<D, LPP>(I, i, sub, (int)(b.nbc[i] & 0xffffu), n, (const int4*)b.PS,
@@ -435,7 +410,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       if ((threadIdx.x & 31) == 0 && m) atomicMax(&vmax_block, m);
       __syncthreads();
       if (threadIdx.x == 0 && vmax_block) atomicMax(&c->vm[it], vmax_block);
-      if (!step_barrier(c, target, g)) return;
+      if (!grid_barrier(&c->count, target, g)) return;
       if (dtd != 0.0) {
         for (int64_t i = first; i < n; i += step) {
           if (i != first || step < n) head.load<LPP>(i, sub, n, nb4, b.nbc);
@@ -448,7 +423,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
         C.vmax2 = __ldcg(&c->vm[it]);
         if (any) more = dt_acoustic_one(I, C, g, 0.0);
       }
-      if (!step_barrier(c, target, g)) return;
+      if (!grid_barrier(&c->count, target, g)) return;
       if (!any) break;
     }
     if (tid == 0) g->substeps += ran;

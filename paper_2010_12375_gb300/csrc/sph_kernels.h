@@ -20,8 +20,7 @@ struct LaunchCfg {
 
 // Grid-wide barrier and loop flags of the persistent substep loop (device memory).
 struct GridBarrier {
-  unsigned count;      // blocks arrived at the current barrier
-  unsigned gen;        // barriers completed
+  unsigned count;      // arrivals at the barriers of the launch so far
   int active[2];       // per substep (alternating): some tank needs another substep
 };
 

@@ -13,11 +13,9 @@
 // maximum (order-free).
 //
 // Memory ordering: a phase gathers what other blocks wrote in the previous one, so the
-// state arrays are read through plain (coherent) loads, never the read-only path, and the
-// barrier fences before arriving and after leaving. The barrier's wait is bounded: a block
-// that waits longer than about a second sets ERR_TIMEOUT and returns, and the others then
-// time out at their next barrier, so the launch always ends. The launch is cooperative,
-// which makes the runtime refuse a grid larger than can be resident at once.
+// state arrays are read through plain (coherent) loads, never the read-only path
+// (sph_grid_sync.cuh has the barrier and its bounded wait). The launch is cooperative, which
+// makes the runtime refuse a grid larger than can be resident at once.
 #include <algorithm>
 
 #include "sph_ctrl.cuh"
@@ -53,6 +51,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
                       const float4* __restrict__ WN, const float4* __restrict__ acc_prior,
                       float4* __restrict__ acc_keep) {
   const int64_t stride = (int64_t)gridDim.x * kPBlock;
+  unsigned target = 0;
   for (int it = 0;; ++it) {
     if (blockIdx.x == 0) {
       const int any = dt_acoustic_block(n_inst, inst, ctrl, g);
@@ -62,7 +61,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
         g->substeps += 1;
       }
     }
-    if (!grid_barrier(bar, g)) return;
+    if (!grid_barrier(&bar->count, target, g)) return;
     for (int64_t i0 = (int64_t)blockIdx.x * kPBlock; i0 < n; i0 += stride) {
       const int64_t i = i0 + threadIdx.x;
       bool valid = i < n;
@@ -75,7 +74,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
           I, i, valid, dtd, nullptr, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
       warp_vmax(v2, writer, k, ctrl);
     }
-    if (!grid_barrier(bar, g)) return;
+    if (!grid_barrier(&bar->count, target, g)) return;
     for (int64_t i0 = (int64_t)blockIdx.x * kPBlock; i0 < n; i0 += stride) {
       const int64_t i = i0 + threadIdx.x;
       bool valid = i < n;
@@ -87,7 +86,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
       dr_particle<D, PER, false, const int4*, const float4*>(I, i, true, dtd, nullptr, n, PH, VH, PS, VS,
                                                                mass, nbr, nbc, WP, WN, g);
     }
-    if (!grid_barrier(bar, g)) return;
+    if (!grid_barrier(&bar->count, target, g)) return;
     if (!__ldcg(&bar->active[it & 1])) break;
   }
 }
@@ -143,7 +142,7 @@ cudaError_t launch_persistent_d(const Buffers& b, cudaStream_t s, int* grid_out)
 
 cudaError_t launch_substeps_persistent(const Buffers& b, cudaStream_t s, int* grid_out) {
   *grid_out = 0;
-  cudaError_t e = cudaMemsetAsync(&b.pbar->count, 0, sizeof(unsigned), s);   // a clean start after a timeout
+  cudaError_t e = cudaMemsetAsync(&b.pbar->count, 0, sizeof(unsigned), s);   // the barrier counts from zero
   if (e != cudaSuccess) return e;
   if (b.dim == 2) return b.any_periodic ? launch_persistent_d<2, true>(b, s, grid_out)
                                         : launch_persistent_d<2, false>(b, s, grid_out);
