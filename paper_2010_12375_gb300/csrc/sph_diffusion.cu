@@ -21,7 +21,7 @@
 // the magic-number add, wrapped on periodic axes only for particles within the support of
 // a periodic face; and when all volumes and diffusivity factors of a tank are equal
 // (checked once per call by the pack kernel, read by the host, which then launches the
-// uniform instantiation; neighbours never cross tanks, so then V_j = V_i) the volume, the
+// uniform instantiation, or by the one-launch form itself; neighbours never cross tanks, so then V_j = V_i) the volume, the
 // factor and the kernel constants leave the pair loop. Otherwise V_j comes from the record
 // (2D) or a per-slot array (3D) and the factor pair from a per-slot array. Wall neighbours
 // are skipped: walls carry no species (zero flux). Pairs at zero distance add nothing.
@@ -39,9 +39,11 @@
 //
 // Between calls the species is kept by caller row, so the fluid solver may re-sort the
 // particles; each call gathers it into slot order, runs its steps and scatters it back.
+#include <algorithm>
 #include <cmath>
 #include <string>
 
+#include "sph_grid_sync.cuh"
 #include "sph_handle.h"
 
 namespace sph {
@@ -239,6 +241,16 @@ __device__ __forceinline__ float row_sum_any(int64_t n, int64_t i, int nf, const
   return row_sum<D, false, ISO, VJ, CORR, TEN>(n, i, nf, I, K, ri, ci, R, nb4, vol, sq, sqi, Bc, Bi, Lc, Li);
 }
 
+// The value a stage gives particle i from its weighted row sum: C^n + dt f, or in the second
+// stage its mean with C^n, read from the output record's own slot (written by no other thread).
+template <bool ISO>
+__device__ __forceinline__ float stage_value(const Inst& I, const DiffCoef& K, float dt, float ci, float sum, bool second,
+                                             const int4* Rout, int64_t i) {
+  const float rate = 2.0f * (ISO ? I.dwr_a * K.kappa : I.dwr_a) * sum;
+  const float next = fmaf(dt, rate, ci);
+  return second ? 0.5f * (i2f(Rout[i].w) + next) : next;
+}
+
 // Five blocks of 256 per SM (48 registers) for the isotropic uniform variants: the stage
 // is latency-bound and runs 8 % faster at 8M particles than with four; the anisotropic
 // variants keep four, since they would spill at 48 registers.
@@ -274,25 +286,16 @@ k_diffusion_stage(int64_t n, const int4* __restrict__ Rin, int4* __restrict__ Ro
   } else {
     sum = row_sum_any<D, PER, ISO, true, CORR, TEN>(n, i, nf, I, K, ri, ci, Rin, nb4, vol, sq, sqi, Bc, Bi, Lc, Li);
   }
-  const float rate = 2.0f * (ISO ? I.dwr_a * K.kappa : I.dwr_a) * sum;
-  const float next = fmaf(dt, rate, ci);
-  // stage 2 reads C^n from the output record's own slot (written by no other thread)
-  const float out = SECOND ? 0.5f * (i2f(Rout[i].w) + next) : next;
-  reinterpret_cast<int*>(Rout)[4 * i + 3] = f2i(out);
+  reinterpret_cast<int*>(Rout)[4 * i + 3] = f2i(stage_value<ISO>(I, K, dt, ci, sum, SECOND, Rout, i));
 }
 
 // Per call: records of both buffers from the fluid state and the species by caller row
 // (b.id[slot] = caller row), the per-slot volumes (3D) and the flag of unequal volumes
 // within a tank.
 template <int D>
-__global__ void k_species_pack(int64_t n, const int4* __restrict__ P, const int* __restrict__ id,
-                               const int* __restrict__ inst_of, const Inst* __restrict__ inst,
-                               const float* __restrict__ mass, const float* __restrict__ by_row,
-                               int4* __restrict__ R0, int4* __restrict__ R1, float* __restrict__ vol,
-                               const float* __restrict__ scale_by_row, float* __restrict__ sq,
-                               int* __restrict__ nonuniform) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+__device__ __forceinline__ void pack_slot(int64_t i, const int4* P, const int* id, const int* inst_of, const Inst* inst,
+                                          const float* mass, const float* by_row, int4* R0, int4* R1, float* vol,
+                                          const float* scale_by_row, float* sq, unsigned* nonuniform) {
   const Inst& I = inst[inst_of ? inst_of[i] : 0];
   const int4 p = P[i];
   const float v = __fdividef(mass ? mass[i] : I.mass, I.rho0 + i2f(p.w));      // m_i / rho_i
@@ -303,12 +306,25 @@ __global__ void k_species_pack(int64_t n, const int4* __restrict__ P, const int*
   if (D == 3) vol[i] = v;
   const int64_t f = I.fluid_begin;                                    // the tank's first slot
   const float vf = __fdividef(mass ? mass[f] : I.mass, I.rho0 + i2f(P[f].w));
-  if (vf != v) atomicOr(nonuniform, 1);
+  if (vf != v) atomicOr(nonuniform, 1u);
   if (scale_by_row) {                                                 // sqrt of s_i, R17
     const float q = sqrtf(scale_by_row[id[i]]);
     sq[i] = q;
-    if (sqrtf(scale_by_row[id[f]]) != q) atomicOr(nonuniform, 2);
+    if (sqrtf(scale_by_row[id[f]]) != q) atomicOr(nonuniform, 2u);
   }
+}
+
+template <int D>
+__global__ void k_species_pack(int64_t n, const int4* __restrict__ P, const int* __restrict__ id,
+                               const int* __restrict__ inst_of, const Inst* __restrict__ inst,
+                               const float* __restrict__ mass, const float* __restrict__ by_row,
+                               int4* __restrict__ R0, int4* __restrict__ R1, float* __restrict__ vol,
+                               const float* __restrict__ scale_by_row, float* __restrict__ sq,
+                               int* __restrict__ nonuniform) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n)
+    pack_slot<D>(i, P, id, inst_of, inst, mass, by_row, R0, R1, vol, scale_by_row, sq,
+                 reinterpret_cast<unsigned*>(nonuniform));
 }
 
 // Per slot: B0_i = (sum_j V_j (r_j - r_i) (x) grad_i W_ij)^-1 over the fluid part of row i
@@ -419,6 +435,140 @@ __global__ void k_species_pack_tensors(int64_t n, const int* __restrict__ id, co
     Lc[2 * i] = make_float4(q * l[0], q * l[1], q * l[2], q * l[3]);
     Lc[2 * i + 1] = make_float4(q * l[4], q * l[5], 0.0f, 0.0f);
   }
+}
+
+// ---- one launch a call ------------------------------------------------------------------
+// The plain form (no tensors, no correction) on few particles: pack, every step's two stages
+// and unpack as phases of one cooperative launch, the choice between the uniform and the
+// weighted sum made on the device. A call is then bound by its few dependent round trips:
+// a call of one step on a 200 x 200 sheet takes 16.5 us (32 us as four launches with a
+// synchronisation to choose the stage kernels). LPP lanes share a particle (lanes p,
+// p + 32 / LPP, ... of a warp, neighbouring lanes holding neighbouring particles) and its
+// terms are added in row order through shared memory, so the result is the stage kernels' bit
+// for bit.
+struct DiffSmall {
+  int64_t n;
+  int n_steps;
+  const int4* P;
+  const int* id;
+  const int* inst_of;
+  const Inst* inst;
+  const float* mass;
+  float* by_row;
+  int4* r0;
+  int4* r1;
+  float* vol;
+  const float* scale_by_row;
+  float* sq;
+  const int* nbr;
+  const uint32_t* nbc;
+  DiffCoef K;
+  float dt;
+  unsigned* ctl;             // [2] zero at launch: barrier arrivals, flag of unequal volumes or factors
+  Global* g;
+};
+constexpr int kSmallThreads = 512;
+
+template <int D, bool PER, bool ISO, int LPP>
+__global__ void __launch_bounds__(kSmallThreads, 2)
+k_diffusion_small(const DiffSmall a) {
+  __shared__ float4 terms_all[LPP > 1 ? kSmallThreads / 32 : 1][2 * 32];
+  float4* terms = terms_all[LPP > 1 ? threadIdx.x >> 5 : 0];
+  constexpr int kStride = 32 / LPP;
+  const int lane = threadIdx.x & 31, sub = LPP == 1 ? 0 : lane / kStride, p = lane & (kStride - 1);
+  const unsigned gm = LPP == 1 ? 0u : (LPP == 2 ? 0x00010001u : LPP == 4 ? 0x01010101u : 0x11111111u) << p;
+  const int64_t n = a.n, share = blockDim.x / LPP, step = (int64_t)gridDim.x * share,
+                first = (int64_t)blockIdx.x * share + (LPP == 1 ? threadIdx.x : (threadIdx.x >> 5) * kStride + p);
+  unsigned target = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    pack_slot<D>(i, a.P, a.id, a.inst_of, a.inst, a.mass, a.by_row, a.r0, a.r1, a.vol, a.scale_by_row, a.sq, a.ctl + 1);
+  if (!grid_barrier(a.ctl, target, a.g)) return;
+  const bool unif = *(volatile unsigned*)(a.ctl + 1) == 0u;
+  const int4* nb4 = reinterpret_cast<const int4*>(a.nbr);
+  // the stage's sum of particle i over its row, in lane 0 of the group
+  auto row = [&](int64_t i, const int4* R, const Inst& I, const int4& ri, float ci, float sqi) {
+    const int nf = (int)(a.nbc[i] & 0xffffu), nq = (nf + 3) >> 2;
+    float2 s = f2(0.0f);
+    int4 nxt = sub < nq ? nb4[(int64_t)sub * n + i] : make_int4(0, 0, 0, 0);
+    for (int q0 = 0; q0 < nq; q0 += LPP) {
+      const int q = q0 + sub;
+      if (LPP == 1 || q < nq) {
+        const int4 cq = nxt;
+        if (q + LPP < nq) nxt = nb4[(int64_t)(q + LPP) * n + i];
+        const int sl = q << 2;
+        const int j0 = cq.x, j1 = sl + 1 < nf ? cq.y : cq.x, j2 = sl + 2 < nf ? cq.z : cq.x, j3 = sl + 3 < nf ? cq.w : cq.x;
+        const int4 a0 = R[j0], a1 = R[j1], a2 = R[j2], a3 = R[j3];
+        float2 w01 = make_float2(1.0f, sl + 1 < nf ? 1.0f : 0.0f);
+        float2 w23 = make_float2(sl + 2 < nf ? 1.0f : 0.0f, sl + 3 < nf ? 1.0f : 0.0f);
+        if (!unif) {
+          if (D == 2) {
+            w01 = mul2(w01, make_float2(i2f(a0.z), i2f(a1.z)));
+            w23 = mul2(w23, make_float2(i2f(a2.z), i2f(a3.z)));
+          } else {
+            w01 = mul2(w01, make_float2(a.vol[j0], a.vol[j1]));
+            w23 = mul2(w23, make_float2(a.vol[j2], a.vol[j3]));
+          }
+          if (a.sq) {
+            const float2 m01 = mul2(add2(f2(sqi), make_float2(a.sq[j0], a.sq[j1])), f2(0.5f));
+            const float2 m23 = mul2(add2(f2(sqi), make_float2(a.sq[j2], a.sq[j3])), f2(0.5f));
+            w01 = mul2(w01, mul2(m01, m01));
+            w23 = mul2(w23, mul2(m23, m23));
+          }
+        }
+        const float2 t01 = diff_terms2<D, PER, ISO>(I, a.K, ri, ci, a0, a1);
+        const float2 t23 = diff_terms2<D, PER, ISO>(I, a.K, ri, ci, a2, a3);
+        if (LPP == 1) {
+          s = fma2(t01, w01, s);
+          s = fma2(t23, w23, s);
+        } else {
+          terms[lane] = make_float4(t01.x, t01.y, t23.x, t23.y);
+          terms[32 + lane] = make_float4(w01.x, w01.y, w23.x, w23.y);
+        }
+      }
+      if (LPP > 1) {
+        __syncwarp(gm);
+        if (sub == 0)
+          for (int k = 0; k < LPP && q0 + k < nq; ++k) {
+            const float4 t = terms[p + k * kStride], w = terms[32 + p + k * kStride];
+            s = fma2(make_float2(t.x, t.y), make_float2(w.x, w.y), s);
+            s = fma2(make_float2(t.z, t.w), make_float2(w.z, w.w), s);
+          }
+        __syncwarp(gm);
+      }
+    }
+    return s.x + s.y;
+  };
+  for (int st = 0; st < 2 * a.n_steps; ++st) {
+    const int4* Rin = st & 1 ? a.r1 : a.r0;
+    int4* Rout = st & 1 ? a.r0 : a.r1;
+    for (int64_t i = first; i < n; i += step) {
+      const Inst& I = a.inst[a.inst_of ? a.inst_of[i] : 0];
+      const int4 ri = Rin[i];
+      const float ci = i2f(ri.w), sqi = a.sq ? a.sq[i] : 1.0f;
+      float sum = row(i, Rin, I, ri, ci, sqi);
+      if (unif) sum = (D == 2 ? i2f(ri.z) : a.vol[i]) * (sqi * sqi) * sum;
+      const float out = stage_value<ISO>(I, a.K, a.dt, ci, sum, st & 1, Rout, i);
+      if (sub == 0) {
+        reinterpret_cast<int*>(Rout)[4 * i + 3] = f2i(out);
+        if (st == 2 * a.n_steps - 1) a.by_row[a.id[i]] = out;
+      }
+    }
+    if (st < 2 * a.n_steps - 1 && !grid_barrier(a.ctl, target, a.g)) return;
+  }
+}
+
+template <int D, bool PER, bool ISO>
+cudaError_t launch_small(const DiffSmall& a, int n_sm, cudaStream_t s) {
+  const int64_t per = (a.n + n_sm - 1) / n_sm;
+  const int lpp = per * 4 <= 2 * kSmallThreads ? 4 : per * 2 <= 2 * kSmallThreads ? 2 : 1;
+  const void* kern = lpp == 4 ? (const void*)k_diffusion_small<D, PER, ISO, 4>
+                              : lpp == 2 ? (const void*)k_diffusion_small<D, PER, ISO, 2>
+                                         : (const void*)k_diffusion_small<D, PER, ISO, 1>;
+  const int64_t lanes = a.n * lpp;
+  const int threads = (int)std::min<int64_t>(kSmallThreads, std::max<int64_t>(128, (lanes / (2 * n_sm) + 31) / 32 * 32));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((lanes + threads - 1) / threads, 2 * (int64_t)n_sm));
+  void* args[] = {const_cast<DiffSmall*>(&a)};
+  return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, 0, s);
 }
 
 // Flags a diffusivity factor that is not a positive finite number.
@@ -535,7 +685,8 @@ struct sph_species {
   int4* r0 = nullptr;          // [n] slot records carrying C^n
   int4* r1 = nullptr;          // [n] slot records carrying C*
   float* vol = nullptr;        // [n] slot volumes m/rho (3D)
-  int* nonuniform = nullptr;   // [1] bit 0: volumes differ within a tank; bit 1: factors do
+  int* nonuniform = nullptr;   // [2] bit 0: volumes differ within a tank; bit 1: factors do (the one-launch
+                               // form: its barrier's count, then these bits)
   float* scale_by_row = nullptr;  // [n] per-particle diffusivity factors s (NULL: all 1)
   float* sq = nullptr;         // [n] sqrt(s) per slot (with scale_by_row)
   double* stage = nullptr;     // [n] doubles for host copies
@@ -610,6 +761,17 @@ void inverse_from_cholesky(const double* L, int d, double* Dinv) {
     }
 }
 
+// Whether a call runs in one launch: while every particle has a lane of its own (1024 an SM),
+// where a one-step call and a further step took, as stage launches and in one launch, 32 + 12.6
+// and 16.5 + 9.9 us on a 2D sheet of 40,000, 75 + 54 and 45 + 39 us on a 3D block of 64,000;
+// beyond that for short calls, whose packing and synchronisation it saves (44 + 15.7 against
+// 26 + 18.0 us on 160,000 in 2D, 142 + 117 against 123 + 114 us on 216,000 in 3D, but 244 + 217
+// against 252 + 240 us on 512,000).
+bool small_diffusion(const sph::Buffers& b, int n_steps) {
+  const int64_t per = (b.n + b.n_sm - 1) / b.n_sm;
+  return per <= 2 * sph::kSmallThreads || (n_steps <= 4 && per <= (b.dim == 2 ? 4096 : 1400));
+}
+
 }  // namespace
 
 extern "C" {
@@ -643,7 +805,7 @@ int sph_species_create(sph_handle* h, const double* D, sph_species** out) {
         cudaMalloc(&sp->r0, sizeof(int4) * n) != cudaSuccess ||
         cudaMalloc(&sp->r1, sizeof(int4) * n) != cudaSuccess ||
         cudaMalloc(&sp->vol, sizeof(float) * n) != cudaSuccess ||
-        cudaMalloc(&sp->nonuniform, sizeof(int)) != cudaSuccess ||
+        cudaMalloc(&sp->nonuniform, 2 * sizeof(int)) != cudaSuccess ||
         cudaMalloc(&sp->gate, sizeof(float) * n) != cudaSuccess ||
         cudaMalloc(&sp->stage, sizeof(double) * n) != cudaSuccess) {
       cudaGetLastError();
@@ -883,8 +1045,24 @@ int sph_diffusion_step(sph_handle* h, sph_species* sp, double dt, int32_t n_step
   cudaStream_t s = (cudaStream_t)stream;
   const unsigned grid = sph::diff_grid(b.n);
   const float fdt = (float)dt;
-  if (cudaMemsetAsync(sp->nonuniform, 0, sizeof(int), s) != cudaSuccess)
+  if (cudaMemsetAsync(sp->nonuniform, 0, 2 * sizeof(int), s) != cudaSuccess)
     return sfail(sp, SPH_E_CUDA, "diffusion set-up failed");
+  if (!sp->Lrow && !sp->corrected && small_diffusion(b, n_steps)) {
+    const sph::DiffSmall a{b.n, n_steps, b.PS, b.id, b.inst_of, b.inst, b.mass, sp->by_row, sp->r0, sp->r1, sp->vol,
+                           sp->scale_by_row, sp->sq, b.nbr, b.nbc, sp->K, fdt,
+                           reinterpret_cast<unsigned*>(sp->nonuniform), b.glob};
+    using Launch = cudaError_t (*)(const sph::DiffSmall&, int, cudaStream_t);
+    const Launch f = b.dim == 2
+        ? (b.any_periodic ? (sp->iso ? sph::launch_small<2, true, true> : sph::launch_small<2, true, false>)
+                          : (sp->iso ? sph::launch_small<2, false, true> : sph::launch_small<2, false, false>))
+        : (b.any_periodic ? (sp->iso ? sph::launch_small<3, true, true> : sph::launch_small<3, true, false>)
+                          : (sp->iso ? sph::launch_small<3, false, true> : sph::launch_small<3, false, false>));
+    if (f(a, b.n_sm, s) == cudaSuccess) {
+      ++h->launches;
+      return SPH_OK;
+    }
+    cudaGetLastError();            // no room for a cooperative launch: a launch a phase
+  }
   auto pack = b.dim == 2 ? sph::k_species_pack<2> : sph::k_species_pack<3>;
   pack<<<grid, sph::kDiffBlock, 0, s>>>(b.n, b.PS, b.id, b.inst_of, b.inst, b.mass, sp->by_row, sp->r0,
                                         sp->r1, sp->vol, sp->scale_by_row, sp->sq, sp->nonuniform);

@@ -156,3 +156,36 @@ def test_threads_per_particle_change_no_bit(sph, case):
     for o_ in out[1:]:
         for a, b in zip(out[0], o_):
             np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("case", ["sheet", "sheet_masses", "box2d_aniso", "block3d", "block3d_scale"])
+def test_one_launch_diffusion_equals_the_stage_launches(sph, case):
+    # above one lane a particle a call of five steps runs as stage launches and a call of one
+    # step as one launch: five of the latter give the same bits
+    D = None
+    if case.startswith("sheet"):
+        prob = wk.diffusion_patch(400)
+    elif case == "box2d_aniso":
+        prob, D = wk.diffusion_band(n=400, ny=400), np.array([[2.0, 0.3], [0.3, 1.0]])
+    else:
+        prob = wk.diffusion_block_3d(55)
+    if case == "sheet_masses":
+        prob.mass = prob.mass * np.random.default_rng(1).uniform(0.9, 1.1, prob.mass.shape)
+    sim = sph.Simulation(prob)
+    sim.build_cells()
+    sp = sph.sph_species_create(sim.handle, prob.meta["D"] if D is None else D, prob.dim)
+    if case.endswith("scale"):
+        sph.sph_species_set_scale(sim.handle, sp, np.random.default_rng(2).uniform(0.5, 2.0, sim.n))
+    C0 = np.random.default_rng(3).uniform(0.0, 1.0, sim.n)
+    out = []
+    for calls, steps in ((1, 5), (5, 1)):
+        sph.sph_species_set(sim.handle, sp, C0)
+        l0 = sim.kernel_launches()
+        for _ in range(calls):
+            sph.sph_diffusion_step(sim.handle, sp, 0.5 * prob.meta["dt"], steps)
+        assert sim.kernel_launches() - l0 == (12 if calls == 1 else 5)
+        out.append(sph.sph_species_get(sim.handle, sp, sim.n))
+    np.testing.assert_array_equal(out[0], out[1])
+    assert not np.array_equal(out[0], C0.astype(np.float32))
+    sph.sph_species_destroy(sp)
+    sim.close()
