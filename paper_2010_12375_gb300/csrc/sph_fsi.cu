@@ -266,19 +266,22 @@ __device__ __forceinline__ float3 fsi_force(const FsiPair& P, float dev_i, float
 // over warps), since the near list's length is on the device.
 constexpr int kCoupleWarps = kFBlock / 32;
 
-// Bounding box (lo, hi) of the positions of each chunk of 32 consecutive entries of a list
-// (idx[k], or k itself when idx is NULL) of n entries, n on the device when n_dev is given.
+// Bounding boxes (lo, hi) of the positions of each chunk of 32 consecutive solid particles
+// (sbox) and of each chunk of the near fluid list (fbox; its length is on the device), and
+// |v|max cleared for its recomputation over the corrected velocities: one launch.
 __global__ void __launch_bounds__(kFBlock)
-k_chunk_boxes(int64_t n_host, const int* __restrict__ n_dev, const int* __restrict__ idx, const int4* __restrict__ X,
-              int4* __restrict__ box) {
-  const int64_t n = n_dev ? (int64_t)*n_dev : n_host;
+k_fsi_boxes(int64_t ns, const int4* __restrict__ X, int4* __restrict__ sbox, const int* __restrict__ n_near,
+            const int* __restrict__ near, const int4* __restrict__ PH, int4* __restrict__ fbox, Ctrl* ctrl) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctrl[0].vmax2 = 0u;
+  const int64_t nf = *n_near, sc = (ns + 31) / 32, fc = (nf + 31) / 32;
   const int lane = threadIdx.x & 31;
-  for (int64_t c = (int64_t)blockIdx.x * kCoupleWarps + (threadIdx.x >> 5); c * 32 < n;
-       c += (int64_t)gridDim.x * kCoupleWarps) {
-    const int64_t k = c * 32 + lane;
+  for (int64_t w = (int64_t)blockIdx.x * kCoupleWarps + (threadIdx.x >> 5); w < sc + fc;
+       w += (int64_t)gridDim.x * kCoupleWarps) {
+    const bool solid = w < sc;
+    const int64_t c = solid ? w : w - sc, k = c * 32 + lane;
     int lo[3] = {INT_MAX, INT_MAX, INT_MAX}, hi[3] = {INT_MIN, INT_MIN, INT_MIN};
-    if (k < n) {
-      const int4 q = X[idx ? (int64_t)idx[k] : k];
+    if (k < (solid ? ns : nf)) {
+      const int4 q = solid ? X[k] : PH[near[k]];
       lo[0] = hi[0] = q.x;
       lo[1] = hi[1] = q.y;
       lo[2] = hi[2] = q.z;
@@ -288,6 +291,7 @@ k_chunk_boxes(int64_t n_host, const int* __restrict__ n_dev, const int* __restri
       hi[a] = __reduce_max_sync(0xffffffffu, hi[a]);
     }
     if (lane == 0) {
+      int4* box = solid ? sbox : fbox;
       box[2 * c] = make_int4(lo[0], lo[1], lo[2], 0);
       box[2 * c + 1] = make_int4(hi[0], hi[1], hi[2], 0);
     }
@@ -327,94 +331,119 @@ __device__ __forceinline__ float csum_warp(float s, float e) {
   return s + e;
 }
 
+// Visits the chunks whose box comes within the support of q, in order: fetch(c) brings the
+// lane's particle of chunk c, and pair(record) takes it while the next chunk's records are
+// already on their way (a particle's walk is a chain of a few dependent fetches).
+template <int D, typename R, typename F, typename G>
+__device__ __forceinline__ void for_near_chunks(const int4& q, int64_t nch, const int4* __restrict__ box, long long R2,
+                                                F&& fetch, G&& pair) {
+  const int lane = threadIdx.x & 31;
+  bool have = false;
+  R cur;
+  for (int64_t c0 = 0; c0 < nch; c0 += 32) {
+    const int64_t c = c0 + lane;
+    unsigned hits = __ballot_sync(0xffffffffu, c < nch && box_within<D>(q, box[2 * c], box[2 * c + 1], R2));
+    for (; hits; hits &= hits - 1) {
+      const R next = fetch(c0 + __ffs(hits) - 1);
+      if (have) pair(cur);
+      cur = next;
+      have = true;
+    }
+  }
+  if (have) pair(cur);
+}
+
+// A solid particle as the coupling sums need it (in: it exists).
+struct SolidRec {
+  int4 q;
+  float4 n, vbar, abar;
+  bool in;
+};
+__device__ __forceinline__ SolidRec solid_rec(int64_t c, int64_t ns, const int4* __restrict__ X,
+                                              const float4* __restrict__ N, const float4* __restrict__ vbar,
+                                              const float4* __restrict__ abar) {
+  const int64_t a = min(c * 32 + (threadIdx.x & 31), ns - 1);
+  return SolidRec{X[a], N[a], vbar[a], abar[a], c * 32 + (threadIdx.x & 31) < ns};
+}
+
+// The two sides of the coupling force, independent of each other: the first fluid_blocks
+// blocks take the near fluid particles, the others the solid's (one launch).
 template <int D>
 __global__ void __launch_bounds__(kFBlock)
-k_fsi_fluid_pressure(const Inst I, const int* __restrict__ n_near_p, const int* __restrict__ near, const int4* __restrict__ PH,
-                     float4* __restrict__ VH, const float4* __restrict__ VS, const float* __restrict__ mass,
-                     const Ctrl* __restrict__ ctrl, int64_t ns, const int4* __restrict__ X,
-                     const float4* __restrict__ N, const float4* __restrict__ vbar, const float4* __restrict__ abar,
-                     const int4* __restrict__ sbox, float4* __restrict__ acc_keep) {
+k_fsi_force(const Inst I, const int* __restrict__ n_near_p, const int* __restrict__ near, const int4* __restrict__ PH,
+            float4* __restrict__ VH, const float4* __restrict__ VS, const float* __restrict__ mass,
+            const Ctrl* __restrict__ ctrl, int64_t ns, const int4* __restrict__ X, const float4* __restrict__ N,
+            const float4* __restrict__ vbar, const float4* __restrict__ abar, const int4* __restrict__ sbox,
+            const int4* __restrict__ fbox, float4* __restrict__ acc_keep, float4* __restrict__ force,
+            int fluid_blocks) {
   const double dtd = ctrl[0].dt;
   if (dtd == 0.0) return;
   const int lane = threadIdx.x & 31;
   const int n_near = *n_near_p;
-  const int64_t nch = (ns + 31) / 32;
-  for (int k = blockIdx.x * kCoupleWarps + (threadIdx.x >> 5); k < n_near; k += gridDim.x * kCoupleWarps) {
-    const int i = near[k];
-    const int4 qi = PH[i];
-    const float dev_i = i2f(qi.w);
-    const float m_i = mass ? mass[i] : I.mass;
-    const float4 vi = VS[i];
-    float s[3] = {0, 0, 0}, e[3] = {0, 0, 0};
-    for (int64_t c0 = 0; c0 < nch; c0 += 32) {
-      const int64_t c = c0 + lane;
-      unsigned hits = __ballot_sync(0xffffffffu, c < nch && box_within<D>(qi, sbox[2 * c], sbox[2 * c + 1], I.R2));
-      while (hits) {
-        const int64_t a = (c0 + __ffs(hits) - 1) * 32 + lane;
-        hits &= hits - 1;
-        if (a >= ns) continue;
-        const int4 qa = X[a];
-        const FsiPair P = fsi_geometry<D>(qi, qa, I);
-        if (!P.in) continue;
-        const float3 f = fsi_force(P, dev_i, m_i, vi, i2f(qa.w), N[a], vbar[a], abar[a], I);
-        csum_add(s[0], e[0], f.x / m_i);
-        csum_add(s[1], e[1], f.y / m_i);
-        if (D == 3) csum_add(s[2], e[2], f.z / m_i);
+  float s[3], e[3];
+  if ((int)blockIdx.x < fluid_blocks) {
+    for (int k = blockIdx.x * kCoupleWarps + (threadIdx.x >> 5); k < n_near; k += fluid_blocks * kCoupleWarps) {
+      const int i = near[k];
+      const int4 qi = PH[i];
+      const float dev_i = i2f(qi.w);
+      const float m_i = mass ? mass[i] : I.mass;
+      const float4 vi = VS[i];
+      for (int c = 0; c < 3; ++c) s[c] = e[c] = 0.f;
+      for_near_chunks<D, SolidRec>(qi, (ns + 31) / 32, sbox, I.R2,
+          [&](int64_t c) { return solid_rec(c, ns, X, N, vbar, abar); },
+          [&](const SolidRec& r) {
+            const FsiPair P = fsi_geometry<D>(qi, r.q, I);
+            if (!P.in || !r.in) return;
+            const float3 f = fsi_force(P, dev_i, m_i, vi, i2f(r.q.w), r.n, r.vbar, r.abar, I);
+            csum_add(s[0], e[0], f.x / m_i);
+            csum_add(s[1], e[1], f.y / m_i);
+            if (D == 3) csum_add(s[2], e[2], f.z / m_i);
+          });
+      const float ax = csum_warp(s[0], e[0]), ay = csum_warp(s[1], e[1]), az = D == 3 ? csum_warp(s[2], e[2]) : 0.f;
+      if (lane == 0) {
+        const float dt = (float)dtd;
+        float4 v = VH[i];
+        v.x += dt * ax;
+        v.y += dt * ay;
+        if (D == 3) v.z += dt * az;
+        VH[i] = v;
+        if (acc_keep) {
+          float4 acc = acc_keep[i];
+          acc.x += ax;
+          acc.y += ay;
+          acc.z += az;
+          acc_keep[i] = acc;
+        }
       }
     }
-    const float ax = csum_warp(s[0], e[0]), ay = csum_warp(s[1], e[1]), az = D == 3 ? csum_warp(s[2], e[2]) : 0.f;
-    if (lane == 0) {
-      const float dt = (float)dtd;
-      float4 v = VH[i];
-      v.x += dt * ax;
-      v.y += dt * ay;
-      if (D == 3) v.z += dt * az;
-      VH[i] = v;
-      if (acc_keep) {
-        float4 acc = acc_keep[i];
-        acc.x += ax;
-        acc.y += ay;
-        acc.z += az;
-        acc_keep[i] = acc;
-      }
-    }
+    return;
   }
-}
-
-template <int D>
-__global__ void __launch_bounds__(kFBlock)
-k_fsi_solid_force(const Inst I, const int* __restrict__ n_near_p, const int* __restrict__ near, const int4* __restrict__ PH,
-                  const float4* __restrict__ VS, const float* __restrict__ mass, const Ctrl* __restrict__ ctrl,
-                  int64_t ns, const int4* __restrict__ X, const float4* __restrict__ N,
-                  const float4* __restrict__ vbar, const float4* __restrict__ abar, const int4* __restrict__ fbox,
-                  float4* __restrict__ force) {
-  if (ctrl[0].dt == 0.0) return;
-  const int lane = threadIdx.x & 31;
-  const int n_near = *n_near_p;
-  const int nch = (n_near + 31) / 32;
-  for (int64_t a = (int64_t)blockIdx.x * kCoupleWarps + (threadIdx.x >> 5); a < ns; a += (int64_t)gridDim.x * kCoupleWarps) {
+  struct FluidRec {
+    int4 q;
+    float4 v;
+    float m;
+    bool in;
+  };
+  const int64_t w0 = (int64_t)(blockIdx.x - fluid_blocks) * kCoupleWarps + (threadIdx.x >> 5);
+  for (int64_t a = w0; a < ns; a += (int64_t)(gridDim.x - fluid_blocks) * kCoupleWarps) {
     const int4 qa = X[a];
     const float V_a = i2f(qa.w);
     const float4 n = N[a], vb = vbar[a], ab = abar[a];
-    float s[3] = {0, 0, 0}, e[3] = {0, 0, 0};
-    for (int c0 = 0; c0 < nch; c0 += 32) {
-      const int c = c0 + lane;
-      unsigned hits = __ballot_sync(0xffffffffu, c < nch && box_within<D>(qa, fbox[2 * c], fbox[2 * c + 1], I.R2));
-      while (hits) {
-        const int k = (c0 + __ffs(hits) - 1) * 32 + lane;
-        hits &= hits - 1;
-        if (k >= n_near) continue;
-        const int i = near[k];
-        const int4 qi = PH[i];
-        const FsiPair P = fsi_geometry<D>(qi, qa, I);
-        if (!P.in) continue;
-        const float m_i = mass ? mass[i] : I.mass;
-        const float3 f = fsi_force(P, i2f(qi.w), m_i, VS[i], V_a, n, vb, ab, I);
-        csum_add(s[0], e[0], -f.x);
-        csum_add(s[1], e[1], -f.y);
-        if (D == 3) csum_add(s[2], e[2], -f.z);
-      }
-    }
+    for (int c = 0; c < 3; ++c) s[c] = e[c] = 0.f;
+    for_near_chunks<D, FluidRec>(qa, (n_near + 31) / 32, fbox, I.R2,
+        [&](int64_t c) {
+          const int64_t k = c * 32 + lane;
+          const int i = near[min(k, (int64_t)n_near - 1)];
+          return FluidRec{PH[i], VS[i], mass ? mass[i] : I.mass, k < n_near};
+        },
+        [&](const FluidRec& r) {
+          const FsiPair P = fsi_geometry<D>(r.q, qa, I);
+          if (!P.in || !r.in) return;
+          const float3 f = fsi_force(P, i2f(r.q.w), r.m, r.v, V_a, n, vb, ab, I);
+          csum_add(s[0], e[0], -f.x);
+          csum_add(s[1], e[1], -f.y);
+          if (D == 3) csum_add(s[2], e[2], -f.z);
+        });
     const float fx = csum_warp(s[0], e[0]), fy = csum_warp(s[1], e[1]), fz = D == 3 ? csum_warp(s[2], e[2]) : 0.f;
     if (lane == 0) force[a] = make_float4(fx, fy, fz, 0.f);
   }
@@ -439,26 +468,20 @@ k_fsi_fluid_continuity(const Inst I, const int* __restrict__ n_near_p, const int
     const float rho_i = I.rho0 + dev_h;
     const float p_i = I.c0sq * dev_h;
     float s = 0.f, e = 0.f;
-    for (int64_t c0 = 0; c0 < nch; c0 += 32) {
-      const int64_t c = c0 + lane;
-      unsigned hits = __ballot_sync(0xffffffffu, c < nch && box_within<D>(qi, sbox[2 * c], sbox[2 * c + 1], I.R2));
-      while (hits) {
-        const int64_t a = (c0 + __ffs(hits) - 1) * 32 + lane;
-        hits &= hits - 1;
-        if (a >= ns) continue;
-        const int4 qa = X[a];
-        const FsiPair P = fsi_geometry<D>(qi, qa, I);
-        if (!P.in) continue;
-        const float4 n = N[a], vb = vbar[a];
-        const float UL = -(n.x * vi.x + n.y * vi.y + n.z * vi.z);
-        const float uw = -(n.x * vb.x + n.y * vb.y + n.z * vb.z);
-        const float UR = -UL + 2.0f * uw;
-        const float PR = imaginary_pressure(p_i, rho_i, P, n, abar[a], I);
-        const float rhoR = I.rho0 + PR * I.inv_c0sq;
-        const float Us = 0.5f * (UL + UR) + (p_i - PR) / ((rho_i + rhoR) * I.c0);   // (P_L - P_R)/(2 rho_bar c0)
-        csum_add(s, e, 2.0f * rho_i * i2f(qa.w) * (Us - UL) * P.dW);
-      }
-    }
+    for_near_chunks<D, SolidRec>(qi, nch, sbox, I.R2,
+        [&](int64_t c) { return solid_rec(c, ns, X, N, vbar, abar); },
+        [&](const SolidRec& r) {
+          const FsiPair P = fsi_geometry<D>(qi, r.q, I);
+          if (!P.in || !r.in) return;
+          const float4 n = r.n, vb = r.vbar;
+          const float UL = -(n.x * vi.x + n.y * vi.y + n.z * vi.z);
+          const float uw = -(n.x * vb.x + n.y * vb.y + n.z * vb.z);
+          const float UR = -UL + 2.0f * uw;
+          const float PR = imaginary_pressure(p_i, rho_i, P, n, r.abar, I);
+          const float rhoR = I.rho0 + PR * I.inv_c0sq;
+          const float Us = 0.5f * (UL + UR) + (p_i - PR) / ((rho_i + rhoR) * I.c0);   // (P_L - P_R)/(2 rho_bar c0)
+          csum_add(s, e, 2.0f * rho_i * i2f(r.q.w) * (Us - UL) * P.dW);
+        });
     const float drho = csum_warp(s, e);
     if (lane == 0) {
       const float hdt = 0.5f * (float)dtd;
@@ -975,6 +998,243 @@ k_solid_steps(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict__ ct
 }
 
 // The solid's state in the caller's order (perm: internal index -> caller's), FP64.
+// The same steps for a 2D solid of which every thread group holds one particle (four lanes a
+// particle, at most kRegRow reference neighbours and kRegThreads / 4 particles a block): a
+// step is then a chain of dependent accesses, two gathers from the neighbours' shared memory
+// (about 210 cycles each) and two cluster barriers (about 600), so everything that does not
+// change over the steps (the neighbours' shared-memory addresses, V_b grad0 W, B0, c_a, the
+// fluid force) and the particle's own state stay in registers, all of a lane's neighbours are
+// fetched at once, every lane of a group carries the particle's update (no broadcasts), and
+// the sums of v and dv/dt and the position are brought up to date between a barrier's arrival
+// and its wait. A launch of about 40 steps on the 1,536-particle plate takes SOLID_FIGURES.
+constexpr int kRegRow = 24, kRegLanes = 4, kRegThreads = 512;
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+// shared-memory address of p in block `rank` of the cluster
+__device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(a), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float4 remote_f4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 remote_f2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
+  return v;
+}
+
+__global__ void __launch_bounds__(kRegThreads, 1)
+k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict__ ctrl) {
+  cg::cluster_group cl = cg::this_cluster();
+  const double dtF = ctrl[0].dt;           // the same in every block
+  if (dtF == 0.0) return;
+  constexpr int L = kRegLanes, NB = kRegRow / kRegLanes;
+  if (S.lanes != L || S.row > kRegRow || S.per_block * L > (int)blockDim.x || S.per_block * L > kRegThreads ||
+      (int64_t)S.per_block * cl.num_blocks() < S.ns) {   // the host sizes these
+    if (gt_is_first() && S.g) atomicOr(&S.g->err, ERR_BOUNDS);
+    return;
+  }
+  __shared__ float4 sPB[kRegThreads / kRegLanes];   // published: P B0
+  __shared__ float2 sV[kRegThreads / kRegLanes];    // published: velocity
+  __shared__ float red[2][kSolidThreads / 32];
+  __shared__ float blk[2];
+  __shared__ int s_kappa;
+  const int P = S.per_block;
+  const unsigned rank = cl.block_rank();
+  const int64_t first = (int64_t)rank * P;
+  const int own = (int)max((int64_t)0, min((int64_t)P, S.ns - first));
+  const int l = (int)threadIdx.x / L, lane = (int)threadIdx.x & (L - 1);
+  const bool live = l < own;
+  const int64_t a = live ? first + l : 0;
+
+  // the particle: its state and constants
+  float2 v = make_float2(0.f, 0.f), acc = v, vsum = v, asum = v, cv = v, fm = v;
+  int4 q = make_int4(0, 0, 0, 0);
+  float F[4] = {}, dF[4] = {}, B[4] = {};
+  bool moves = false;
+  uint32_t addr[NB], addr_v[NB];
+  float2 gv[NB];
+#pragma unroll
+  for (int k = 0; k < NB; ++k) {
+    addr[k] = remote_addr(&sPB[min(l, P - 1)], rank);
+    addr_v[k] = remote_addr(&sV[min(l, P - 1)], rank);
+    gv[k] = make_float2(0.f, 0.f);         // no neighbour: the particle itself with weight 0
+  }
+  float vm = 0.f, am = 0.f;
+  const float inv_rho0 = 1.0f / M.rho0;
+  if (live) {
+    const float4 v4 = S.V[a], ac = S.acc[a], c4 = S.cA[a], f = S.force[a];
+    v = make_float2(v4.x, v4.y);
+    acc = make_float2(ac.x, ac.y);
+    cv = make_float2(c4.x, c4.y);
+    q = S.X[a];
+    const float inv_m = inv_rho0 / S.vol[a];
+    fm = make_float2(f.x * inv_m, f.y * inv_m);
+    moves = S.fixed[a] == 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      F[k] = S.F[(int64_t)k * S.ns + a];
+      dF[k] = S.dFdt[(int64_t)k * S.ns + a];
+      B[k] = S.B0[(int64_t)k * S.ns + a];
+    }
+    const int nc = min(S.cnt[a], kRegRow);
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const int t = lane + L * k;
+      if (t < nc) {
+        const int pk = S.nb[(int64_t)t * S.ns + a];
+        const float4 g = S.gV[(int64_t)t * S.ns + a];
+        addr[k] = remote_addr(&sPB[pk & 0xffff], (uint32_t)pk >> 16);
+        addr_v[k] = remote_addr(&sV[pk & 0xffff], (uint32_t)pk >> 16);
+        gv[k] = make_float2(g.x, g.y);
+      }
+    }
+    vm = v4.x * v4.x + v4.y * v4.y + v4.z * v4.z;
+    am = ac.x * ac.x + ac.y * ac.y + ac.z * ac.z;
+  }
+  cluster_vmax(cl, vm, am, red, blk);
+  if (threadIdx.x == 0) {
+    const double dts = solid_dt(M, vm, am);
+    const double r = dtF / dts;
+    int kappa = 0;
+    if (dts > 0.0 && r < (double)kMaxSolidSteps) kappa = (int)floor(r) + 1;
+    else if (rank == 0 && S.g) atomicOr(&S.g->err, ERR_DT);
+    s_kappa = kappa;
+    if (rank == 0) {
+      *S.kappa_last = kappa;
+      *S.steps += kappa;
+    }
+  }
+  __syncthreads();
+  const int kappa = s_kappa;
+  if (kappa == 0) return;                  // the same decision in every block; nothing written
+  const double hd = dtF / kappa;
+  const float h = (float)hd, hh = 0.5f * h;
+  float PB[4];
+  auto move = [&] {                        // half a step of the position
+    if (moves) {
+      q.x += __float2int_rn(hh * v.x * I.inv_dq);
+      q.y += __float2int_rn(hh * v.y * I.inv_dq);
+    }
+  };
+  // the first half of a step: F += dt/2 dF/dt and P B0, published; the caller moves r
+  auto first_half = [&] {
+    float Pk[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) F[k] += hh * dF[k];
+    first_piola<2>(M, F, Pk);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) s += Pk[i * 2 + k] * B[k * 2 + j];
+        PB[i * 2 + j] = s;
+      }
+    if (live && lane == 0) sPB[l] = make_float4(PB[0], PB[1], PB[2], PB[3]);
+  };
+  first_half();
+  cluster_arrive();
+  move();
+  cluster_wait();
+  for (int step = 0; step < kappa; ++step) {
+    // A: dv/dt, v (the stress divergence as in k_solid_steps)
+    float4 pb[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) pb[k] = remote_f4(addr[k]);
+    float sx = 0.f, sy = 0.f;
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      sx = fmaf(pb[k].y, gv[k].y, fmaf(pb[k].x, gv[k].x, sx));
+      sy = fmaf(pb[k].w, gv[k].y, fmaf(pb[k].z, gv[k].x, sy));
+    }
+#pragma unroll
+    for (int o = L >> 1; o > 0; o >>= 1) {
+      sx += __shfl_xor_sync(0xffffffffu, sx, o);
+      sy += __shfl_xor_sync(0xffffffffu, sy, o);
+    }
+    acc = make_float2(0.f, 0.f);
+    if (moves) {
+      acc.x = (sx + fmaf(PB[1], cv.y, PB[0] * cv.x)) * inv_rho0 + M.g[0] + fm.x;
+      acc.y = (sy + fmaf(PB[3], cv.y, PB[2] * cv.x)) * inv_rho0 + M.g[1] + fm.y;
+      v.x += h * acc.x;
+      v.y += h * acc.y;
+    }
+    if (live && lane == 0) sV[l] = v;
+    cluster_arrive();                      // v published; every read of P B0 done
+    move();
+    vsum.x += v.x;
+    vsum.y += v.y;
+    asum.x += acc.x;
+    asum.y += acc.y;
+    cluster_wait();
+    // B: dF/dt from the new velocities, F the second half, then the next step's first half
+    float2 vb[NB];
+#pragma unroll
+    for (int k = 0; k < NB; ++k) vb[k] = remote_f2(addr_v[k]);
+    float G[4] = {};
+#pragma unroll
+    for (int k = 0; k < NB; ++k) {
+      const float dx = vb[k].x - v.x, dy = vb[k].y - v.y;
+      G[0] = fmaf(dx, gv[k].x, G[0]);
+      G[1] = fmaf(dx, gv[k].y, G[1]);
+      G[2] = fmaf(dy, gv[k].x, G[2]);
+      G[3] = fmaf(dy, gv[k].y, G[3]);
+    }
+#pragma unroll
+    for (int o = L >> 1; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) G[k] += __shfl_xor_sync(0xffffffffu, G[k], o);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        float s = 0.f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) s += G[i * 2 + k] * B[k * 2 + j];
+        dF[i * 2 + j] = s;
+      }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) F[k] = F[k] + hh * dF[k];
+    const bool more = step + 1 < kappa;
+    if (more) first_half();
+    cluster_arrive();                      // P B0 published; every read of v done
+    if (more) move();
+    cluster_wait();
+  }
+  // the particle back to global memory, with the step averages v~ and a~, and (single time
+  // stepping) the next fluid step's cap
+  const float inv = 1.0f / (float)kappa;
+  vm = 0.f;
+  am = 0.f;
+  if (live && lane == 0) {
+    S.V[a] = make_float4(v.x, v.y, 0.f, 0.f);
+    S.X[a] = q;
+    S.acc[a] = make_float4(acc.x, acc.y, 0.f, 0.f);
+    S.vbar[a] = make_float4(vsum.x * inv, vsum.y * inv, 0.f, 0.f);
+    S.abar[a] = make_float4(asum.x * inv, asum.y * inv, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      S.F[(int64_t)k * S.ns + a] = F[k];
+      S.dFdt[(int64_t)k * S.ns + a] = dF[k];
+    }
+    vm = v.x * v.x + v.y * v.y;
+    am = acc.x * acc.x + acc.y * acc.y;
+  }
+  if (M.single_step && S.dt_cap) {
+    // as in k_solid_steps
+    cluster_vmax(cl, vm, am, red, blk);
+    if (threadIdx.x == 0 && rank == 0) S.dt_cap[0] = solid_dt(M, vm, am) * (1.0 - 1e-9);
+  }
+}
+
 __global__ void k_solid_export(int64_t ns, int d, const int* __restrict__ perm, const int4* __restrict__ X,
                                const float4* __restrict__ V, const float4* __restrict__ force,
                                const float* __restrict__ F, double lo0, double lo1, double lo2, double dq,
@@ -1007,6 +1267,7 @@ struct sph_solid {
   int dim = 2, cap = 0;
   int cluster = 1, threads = 32, lanes = 1, per_block = 1, tile_bytes = 0, row = 1;   // shape of the solid-step launch
   bool staged = false;          // constant rows staged in shared memory
+  bool reg = false;             // a particle a thread group, state in registers (k_solid_steps_reg)
   sph::SolidMat mat{};
   std::vector<void*> allocs;
   int4* X = nullptr;
@@ -1020,6 +1281,7 @@ struct sph_solid {
   long long* steps = nullptr;
   int* perm = nullptr;          // internal index -> the caller's (device)
   int4 *sbox = nullptr, *fbox = nullptr;   // chunk boxes: solid, near fluid list
+  double* stage = nullptr;      // export staging, allocated by the first sph_solid_get_state
   std::vector<int> perm_host;
   uint32_t *flag = nullptr, *off = nullptr, *scan_tmp = nullptr;
 };
@@ -1143,11 +1405,36 @@ bool choose_cluster(sph_solid* s, int max_row) {
   return false;
 }
 
+// Whether the chosen launch shape lets a 2D solid's steps run in registers.
+bool reg_steps_fit(const sph_solid* s) {
+  if (s->dim != 2 || s->lanes != sph::kRegLanes || s->row > sph::kRegRow || s->threads < s->per_block * s->lanes ||
+      s->per_block * s->lanes > sph::kRegThreads || s->threads > sph::kRegThreads)
+    return false;
+  const void* kern = (const void*)sph::k_solid_steps_reg;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  cfg.gridDim = dim3((unsigned)s->cluster);
+  cfg.blockDim = dim3((unsigned)s->threads);
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)s->cluster;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int active = 0;
+  if (cudaOccupancyMaxActiveClusters(&active, kern, &cfg) != cudaSuccess) cudaGetLastError();
+  return active > 0;
+}
+
 void cluster_config(const sph_solid* s, cudaStream_t st, cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at) {
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3((unsigned)s->cluster);
   cfg->blockDim = dim3((unsigned)s->threads);
-  cfg->dynamicSmemBytes = (size_t)s->tile_bytes;
+  cfg->dynamicSmemBytes = s->reg ? 0 : (size_t)s->tile_bytes;
   cfg->stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)s->cluster;
@@ -1188,20 +1475,18 @@ void sph_fsi_after_pressure(sph_handle* h, cudaStream_t st, int64_t* launches) {
   if (!s || s->ns == 0 || h->b.n == 0) return;
   sph::Buffers& b = h->b;
   // chunk boxes of the solid's positions and of the near fluid list's mid-point positions;
-  // then a warp per near fluid particle (the list's length is on the device), a warp per
-  // solid particle
-  sph::k_chunk_boxes<<<sph::wgrid((s->ns + 31) / 32), sph::kFBlock, 0, st>>>(s->ns, nullptr, nullptr, s->X, s->sbox);
-  sph::k_chunk_boxes<<<sph::wgrid((b.n + 31) / 32), sph::kFBlock, 0, st>>>(0, s->n_near, s->near, b.PH, s->fbox);
-  auto fp = b.dim == 2 ? sph::k_fsi_fluid_pressure<2> : sph::k_fsi_fluid_pressure<3>;
-  fp<<<sph::wgrid(b.n), sph::kFBlock, 0, st>>>(b.inst0, s->n_near, s->near, b.PH, b.VH, b.VS, b.mass, b.ctrl, s->ns,
-                                               s->X, s->N, s->vbar, s->abar, s->sbox, b.acc_keep);
-  auto sf = b.dim == 2 ? sph::k_fsi_solid_force<2> : sph::k_fsi_solid_force<3>;
-  sf<<<sph::wgrid(s->ns), sph::kFBlock, 0, st>>>(b.inst0, s->n_near, s->near, b.PH, b.VS, b.mass, b.ctrl, s->ns, s->X,
-                                                 s->N, s->vbar, s->abar, s->fbox, s->force);
-  sph::Buffers vb = b;                     // |v|max over the corrected new velocities
+  // then a warp per near fluid particle (the list's length is on the device) and a warp per
+  // solid particle; then |v|max over the corrected new velocities
+  sph::k_fsi_boxes<<<sph::wgrid((s->ns + 31) / 32 + (b.n + 31) / 32), sph::kFBlock, 0, st>>>(
+      s->ns, s->X, s->sbox, s->n_near, s->near, b.PH, s->fbox, b.ctrl);
+  const unsigned gf = sph::wgrid(b.n), gs = sph::wgrid(s->ns);
+  auto ff = b.dim == 2 ? sph::k_fsi_force<2> : sph::k_fsi_force<3>;
+  ff<<<gf + gs, sph::kFBlock, 0, st>>>(b.inst0, s->n_near, s->near, b.PH, b.VH, b.VS, b.mass, b.ctrl, s->ns, s->X, s->N,
+                                       s->vbar, s->abar, s->sbox, s->fbox, b.acc_keep, s->force, (int)gf);
+  sph::Buffers vb = b;
   vb.VS = b.VH;
-  sph::launch_vmax(vb, st, launches);
-  *launches += 4;
+  sph::launch_vmax(vb, st, launches, false);
+  *launches += 2;
 }
 
 void sph_fsi_after_density(sph_handle* h, cudaStream_t st, int64_t* launches) {
@@ -1217,7 +1502,8 @@ void sph_fsi_after_density(sph_handle* h, cudaStream_t st, int64_t* launches) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at[1];
   cluster_config(s, st, &cfg, at);
-  auto ks = b.dim == 2 ? (s->staged ? sph::k_solid_steps<2, true> : sph::k_solid_steps<2, false>)
+  auto ks = s->reg ? sph::k_solid_steps_reg
+          : b.dim == 2 ? (s->staged ? sph::k_solid_steps<2, true> : sph::k_solid_steps<2, false>)
                        : (s->staged ? sph::k_solid_steps<3, true> : sph::k_solid_steps<3, false>);
   cudaLaunchKernelEx(&cfg, ks, b.inst0, s->mat, ptrs(s), (const sph::Ctrl*)b.ctrl);
   *launches += 1;
@@ -1376,6 +1662,7 @@ int sph_solid_create(sph_handle* h, const sph_solid_params* p, int64_t n, const 
   }
   if (!choose_cluster(s, *std::max_element(hcnt.begin(), hcnt.end())))
     return sfail(s, SPH_E_CAPACITY, "the solid does not fit the shared memory of one thread-block cluster");
+  s->reg = reg_steps_fit(s);
   sph::k_solid_pack_rows<<<sph::fgrid(n), sph::kFBlock>>>(n, s->cap, s->cnt, s->per_block, s->nb);
   if (cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
@@ -1418,11 +1705,8 @@ int sph_solid_get_state(sph_handle* h, sph_solid* s, double* pos, double* vel, d
   const size_t n = (size_t)s->ns;
   double* dst[4] = {pos, vel, force, F};
   const size_t sz[4] = {n * d, n * d, n * d, n * d * d};
-  double* tmp = nullptr;
-  if (cudaMalloc(&tmp, sizeof(double) * (3 * n * d + n * d * d)) != cudaSuccess) {
-    cudaGetLastError();
-    return sfail(s, SPH_E_OOM, "staging allocation failed");
-  }
+  if (!s->stage && !salloc(s, &s->stage, 3 * n * d + n * d * d)) return sfail(s, SPH_E_OOM, "staging allocation failed");
+  double* tmp = s->stage;                  // kept: an allocation and its release cost more than the copy
   double* t[4] = {tmp, tmp + n * d, tmp + 2 * n * d, tmp + 3 * n * d};
   const sph::Inst& I = h->b.inst0;
   sph::k_solid_export<<<sph::fgrid(s->ns), sph::kFBlock, 0, st>>>(s->ns, d, s->perm, s->X, s->V, s->force, s->F, I.lo[0],
@@ -1434,7 +1718,6 @@ int sph_solid_get_state(sph_handle* h, sph_solid* s, double* pos, double* vel, d
   long long steps = 0;
   if (cudaMemcpyAsync(&steps, s->steps, sizeof(long long), cudaMemcpyDeviceToHost, st) != cudaSuccess) rc = SPH_E_CUDA;
   if (cudaStreamSynchronize(st) != cudaSuccess) rc = SPH_E_CUDA;
-  cudaFree(tmp);
   if (rc != SPH_OK) {
     cudaGetLastError();
     return sfail(s, rc, "copy of the solid's state failed");

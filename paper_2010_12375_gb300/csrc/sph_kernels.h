@@ -125,7 +125,7 @@ void launch_export_neighbours(const Buffers& b, int32_t* fc, int32_t* wc, int32_
 
 // physics
 void launch_pair_count(const Buffers& b, unsigned long long* out2, cudaStream_t s);
-void launch_vmax(const Buffers& b, cudaStream_t s, int64_t* launches);
+void launch_vmax(const Buffers& b, cudaStream_t s, int64_t* launches, bool reset = true);   // reset: |v|max to 0 first
 void launch_dt_advection(const Buffers& b, cudaStream_t s, int64_t* launches);
 void launch_density(const Buffers& b, cudaStream_t s, int64_t* launches);
 void launch_viscous(const Buffers& b, cudaStream_t s, int64_t* launches);

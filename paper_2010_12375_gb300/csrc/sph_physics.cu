@@ -318,9 +318,11 @@ void launch_pair_count(const Buffers& b, unsigned long long* out2, cudaStream_t 
   k_pair_count<<<grid_for(b.n), kBlock, 0, s>>>(b.n, b.nbc, out2);
 }
 
-void launch_vmax(const Buffers& b, cudaStream_t s, int64_t* launches) {
-  k_reset_vmax<<<1, 256, 0, s>>>(b.n_inst, b.ctrl);
-  ++*launches;
+void launch_vmax(const Buffers& b, cudaStream_t s, int64_t* launches, bool reset) {
+  if (reset) {
+    k_reset_vmax<<<1, 256, 0, s>>>(b.n_inst, b.ctrl);
+    ++*launches;
+  }
   if (b.n == 0) return;
   SPH_DIM_LAUNCH(b, k_vmax, grid_for(b.n), kBlock, s, b.n, b.VS, b.inst_of, b.ctrl);
   ++*launches;
