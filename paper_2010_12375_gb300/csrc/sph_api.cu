@@ -214,43 +214,36 @@ Inst make_inst(const sph_params& p) {
   I.cfl_ac = p.cfl_ac;
   I.dt_min = 1e-12 * p.h / p.c0;
   I.dq_d = dq;
+  I.inv_dq_d = 1.0 / dq;
   I.rho0_d = p.rho0;
   return I;
 }
 
-// Memory the current device addresses directly: its own device memory or managed memory.
-bool is_device_ptr(const void* p) {
-  if (!p) return false;
+// Where a caller array lives: host memory (or none), memory the current device addresses
+// directly (its own or managed), or device memory of another GPU, which the entry points
+// refuse: the kernels run on the current device. One query a pointer: they are host time in
+// every transfer of a small state.
+enum class Mem { host, device, foreign };
+
+Mem memory_of(const void* p) {
+  if (!p) return Mem::host;
   cudaPointerAttributes at;
   if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return Mem::host;
   }
-  if (at.type == cudaMemoryTypeManaged) return true;
+  if (at.type == cudaMemoryTypeManaged) return Mem::device;
+  if (at.type != cudaMemoryTypeDevice) return Mem::host;
   int cur = -1;
-  if (at.type != cudaMemoryTypeDevice || cudaGetDevice(&cur) != cudaSuccess) {
+  if (cudaGetDevice(&cur) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return Mem::host;
   }
-  return at.device == cur;
+  return at.device == cur ? Mem::device : Mem::foreign;
 }
 
-// Device memory of a GPU other than the current one. The kernels run on the current
-// device, so the entry points reject such arrays instead of dereferencing them.
-bool foreign_device_ptr(const void* p) {
-  if (!p) return false;
-  cudaPointerAttributes at;
-  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  int cur = -1;
-  if (at.type != cudaMemoryTypeDevice || cudaGetDevice(&cur) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return at.device != cur;
-}
+bool is_device_ptr(const void* p) { return memory_of(p) == Mem::device; }
+bool foreign_device_ptr(const void* p) { return memory_of(p) == Mem::foreign; }
 
 bool any_foreign(std::initializer_list<const void*> ptrs) {
   for (const void* p : ptrs)
@@ -724,6 +717,7 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
   }
   CK(h, cudaMemcpy(b.inst, h->hinst.data(), sizeof(Inst) * n_instances, cudaMemcpyHostToDevice));
   b.inst0 = h->hinst[0];
+  h->sigma0 = lattice_sum(params[0].dp, params[0].h, dim);
   std::vector<Ctrl> hc(n_instances);
   std::memset(hc.data(), 0, sizeof(Ctrl) * n_instances);
   CK(h, cudaMemcpy(b.ctrl, hc.data(), sizeof(Ctrl) * n_instances, cudaMemcpyHostToDevice));
@@ -767,7 +761,7 @@ int sph_get_info(const sph_handle* h, sph_info* out) {
   out->n_cells = h->b.n_cells;
   out->cell = I.dq_d * (double)(1u << I.bits);
   out->dq = I.dq_d;
-  out->sigma0 = lattice_sum(h->params[0].dp, h->params[0].h, h->b.dim);
+  out->sigma0 = h->sigma0;
   out->R2 = I.R2;
   out->device_bytes = h->device_bytes;
   return SPH_OK;
@@ -778,11 +772,18 @@ int sph_set_state(sph_handle* h, const double* pos, const double* vel, const dou
   if (!h) return SPH_E_INVALID;
   Buffers& b = h->b;
   if (b.n > 0 && (!pos || !vel || !rho)) return fail(h, SPH_E_INVALID, "pos, vel and rho are required");
-  if (any_foreign({pos, vel, rho, drho_dt})) return fail(h, SPH_E_INVALID, "an array lives on another device");
+  const double* src[4] = {pos, vel, rho, drho_dt};
+  Mem mem[4];
+  for (int k = 0; k < 4; ++k) {
+    mem[k] = memory_of(src[k]);
+    if (mem[k] == Mem::foreign) return fail(h, SPH_E_INVALID, "an array lives on another device");
+  }
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)b.n, d = (size_t)b.dim;
-  const bool host_all = b.n >= kUploadChunkMin && !is_device_ptr(pos) && !is_device_ptr(vel) &&
-                        !is_device_ptr(rho) && (!drho_dt || !is_device_ptr(drho_dt));
+  const bool host_all = b.n >= kUploadChunkMin && mem[0] == Mem::host && mem[1] == Mem::host &&
+                        mem[2] == Mem::host && mem[3] == Mem::host;
+  sph::launch_import_begin(b, t, s);
+  ++h->launches;
   if (host_all) {
     // host arrays: kUploadChunks row chunks, each imported while the next one is copied
     if (!h->up_stream) {
@@ -809,22 +810,14 @@ int sph_set_state(sph_handle* h, const double* pos, const double* vel, const dou
       ++h->launches;
     }
   } else if (b.n > 0) {
-    cudaError_t e[4];
-    const double* p = device_view(h, pos, n * d, 0, s, &e[0]);
-    const double* v = device_view(h, vel, n * d, n * d, s, &e[1]);
-    const double* r = device_view(h, rho, n, 2 * n * d, s, &e[2]);
-    const double* dr = device_view(h, drho_dt, n, 2 * n * d + n, s, &e[3]);
-    for (auto ee : e)
-      if (ee != cudaSuccess) return cuda_fail(h, ee, "copy state");
-    sph::launch_import(b, p, v, r, dr, s);
+    const size_t len[4] = {n * d, n * d, n, n}, off[4] = {0, n * d, 2 * n * d, 2 * n * d + n};
+    for (int k = 0; k < 4; ++k) {            // host arrays through the staging buffer
+      if (!src[k] || mem[k] == Mem::device) continue;
+      CK(h, cudaMemcpyAsync(h->stage + off[k], src[k], sizeof(double) * len[k], cudaMemcpyHostToDevice, s));
+      src[k] = h->stage + off[k];
+    }
+    sph::launch_import(b, src[0], src[1], src[2], src[3], s);
     ++h->launches;
-  }
-  // slot k holds caller row k until the next cell build
-  sph::launch_iota(b.id, b.n, s);
-  if (b.n) ++h->launches;
-  sph::launch_vmax(b, s, &h->launches);
-  if (t >= 0.0) {
-    CK(h, cudaMemcpyAsync(&b.ctrl[0].t, &t, sizeof(double), cudaMemcpyHostToDevice, s));
   }
   CK(h, cudaStreamSynchronize(s));          // the caller's arrays may be reused on return
   h->cells_valid = false;
@@ -993,15 +986,19 @@ int sph_get_state(sph_handle* h, double* pos, double* vel, double* rho, double* 
   Buffers& b = h->b;
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)b.n, d = (size_t)b.dim;
-  if (any_foreign({pos, vel, rho, drho_dt})) return fail(h, SPH_E_INVALID, "an array lives on another device");
-  if (n == 0) return SPH_OK;
   double* dst[4] = {pos, vel, rho, drho_dt};
+  Mem mem[4];
+  for (int k = 0; k < 4; ++k) {
+    mem[k] = memory_of(dst[k]);
+    if (mem[k] == Mem::foreign) return fail(h, SPH_E_INVALID, "an array lives on another device");
+  }
+  if (n == 0) return SPH_OK;
   size_t sz[4] = {n * d, n * d, n, n};
   size_t off[4] = {0, n * d, 2 * n * d, 2 * n * d + n};
   double* tgt[4];
   bool dev[4];
   for (int k = 0; k < 4; ++k) {
-    dev[k] = dst[k] && is_device_ptr(dst[k]);
+    dev[k] = mem[k] == Mem::device;
     tgt[k] = dst[k] ? (dev[k] ? dst[k] : h->stage + off[k]) : nullptr;
   }
   sph::launch_export(b, tgt[0], tgt[1], tgt[2], tgt[3], s);

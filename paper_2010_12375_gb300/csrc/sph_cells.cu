@@ -452,10 +452,6 @@ void launch_check_table(const Buffers& b, cudaStream_t s, int64_t* launches) {
   ++*launches;
 }
 
-void launch_iota(int* a, int64_t n, cudaStream_t s) {
-  if (n > 0) k_iota<<<grid_for(n), kBlock, 0, s>>>(n, a);
-}
-
 // b.wnear from the sorted walls; tmp holds n_cells bytes of scratch.
 void flag_near_wall_cells(const Buffers& b, uint8_t* tmp, cudaStream_t s) {
   if (b.n_cells == 0) return;

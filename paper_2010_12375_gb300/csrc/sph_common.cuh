@@ -56,7 +56,7 @@ struct Inst {
   double h_d, c0_d, u_ref, nu, cfl_ad, cfl_ac;
   double dt_min;                 // 1e-12 h / c0: a smaller acoustic step is an error
   double lo[3];                  // cell-grid origin
-  double dq_d;                   // position quantum in double precision
+  double dq_d, inv_dq_d;         // position quantum in double precision, and its reciprocal
   double rho0_d;
 };
 

@@ -10,6 +10,7 @@ struct sph_handle {
   sph::Buffers b;
   std::vector<sph_params> params;
   std::vector<sph::Inst> hinst;
+  double sigma0 = 0.0;             // lattice sum of tank 0 (sph_get_info)
   uint32_t flags = 0;
   std::string err;
   std::vector<void*> allocs;

@@ -109,10 +109,11 @@ void launch_row_tasks(const Buffers& b, cudaStream_t s, int64_t* launches);
 inline bool row_form(int block) { return block == kRowBlock; }
 void sort_walls(Buffers& b, int4* WP_tmp, float4* WN_tmp, int* wid_tmp, cudaStream_t s);
 void flag_near_wall_cells(const Buffers& b, uint8_t* tmp, cudaStream_t s);
-void launch_iota(int* a, int64_t n, cudaStream_t s);     // a[i] = i
 
 // import / export
-// rows [i0, i1) of the caller's arrays (i1 < 0: to the end)
+// the start of a state import: |v|max cleared, and tank 0's clock (t < 0: kept)
+void launch_import_begin(const Buffers& b, double t, cudaStream_t s);
+// rows [i0, i1) of the caller's arrays (i1 < 0: to the end): records, ids (slot = row) and |v|max
 void launch_import(const Buffers& b, const double* pos, const double* vel, const double* rho,
                    const double* drho, cudaStream_t s, int64_t i0 = 0, int64_t i1 = -1);
 void launch_import_walls(const Buffers& b, const double* pos, const double* nrm, const double* vol,
