@@ -637,7 +637,7 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
   DALLOC(h, b.ctrl, n_instances);
   DALLOC(h, b.glob, 1);
   DALLOC(h, b.pbar, 1);
-  DALLOC(h, b.PS, n_fluid);
+  DALLOC(h, b.PS, n_fluid + 1);               // the neighbour search reads one record past an odd run
   DALLOC(h, b.VS, n_fluid);
   DALLOC(h, b.PH, nmax);
   DALLOC(h, b.VH, nmax);
@@ -669,7 +669,7 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
     CK(h, cudaGetDevice(&dev));
     CK(h, cudaDeviceGetAttribute(&b.n_sm, cudaDevAttrMultiProcessorCount, dev));
   }
-  DALLOC(h, b.WP, n_wall);
+  DALLOC(h, b.WP, n_wall + 1);                // as PS
   DALLOC(h, b.WN, n_wall);
   DALLOC(h, b.wid, n_wall);
   DALLOC(h, b.nbr, (size_t)n_fluid * b.cap);

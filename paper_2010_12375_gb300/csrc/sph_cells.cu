@@ -194,44 +194,54 @@ __global__ void k_copy_back(int64_t n, const int4* __restrict__ Pin, const float
 }
 
 // ---------------------------------------------------------------- neighbours ---------
+// All neighbours of particle i among the records R of one cell-linked list (`self`: R holds
+// the particle itself) into its row from slot0 on; returns their number. The candidates of a
+// run are tested first, their hits kept as bits, and written then: the stores of 32 lanes
+// diverge, and inside the test loop every test paid for them. With it, the sign bits of the
+// keys as hits, the tank's constants in the argument (48 registers in 3D, five blocks an SM for
+// four) and 32-bit chords, the search of 1.02M particles of the 3D dam break takes 442 us (580).
 template <int D, bool PER>
+__device__ __forceinline__ int list_neighbours(const Inst& I, int64_t n, int64_t i, const int4& pi, const int4* R,
+                                               const uint32_t* start, bool self, int slot0, int cap, int* nbr,
+                                               bool& overflow) {
+  const float R2f = (float)I.R2, band = R2f * 1.9073486328125e-06f;
+  RowWriter w(nbr, n, i, slot0, cap);
+  for_neighbour_runs<D, PER>(I, pi, start, [&](uint32_t b, uint32_t e) {
+    for (; b < e; b += 32) {
+      const uint32_t m = min(e - b, 32u);
+      const int4* r = R + b;
+      unsigned bits = 0;                             // candidate k at bit m' - 1 - k, m' = m made even
+      for (uint32_t k = 0; k < m; k += 2, r += 2) {   // one past an odd run: masked out (the arrays are padded)
+        const float2 key = candidate_keys<D, PER>(pi, r[0], r[1], I, R2f, band);
+        bits = push_sign(push_sign(bits, key.x), key.y);
+      }
+      bits = __brev(bits) >> ((32u - m) & ~1u);       // candidate k at bit k
+      if (m < 32u) bits &= (1u << m) - 1u;
+      if (self && (uint32_t)i - b < 32u) bits &= ~(1u << ((uint32_t)i - b));
+      for (; bits; bits &= bits - 1) w.push((int)(b + __ffs((int)bits) - 1), overflow);
+    }
+  });
+  return w.count;
+}
+
+// UNI: a single tank, its constants in the kernel argument.
+template <int D, bool PER, bool UNI>
 __global__ void __launch_bounds__(kBlock)
-k_neighbours(int64_t n, const int4* __restrict__ P, const int* __restrict__ inst_of,
+k_neighbours(const Inst Ip, int64_t n, const int4* __restrict__ P, const int* __restrict__ inst_of,
              const Inst* __restrict__ inst, const uint32_t* __restrict__ fstart,
              const int4* __restrict__ WP, const uint32_t* __restrict__ wstart,
              const uint8_t* __restrict__ wnear, int cap, int* __restrict__ nbr,
              uint32_t* __restrict__ nbc, Global* g) {
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
-  const Inst& I = inst[inst_of ? inst_of[i] : 0];
-  const float R2f = (float)I.R2;
-  const float lo = R2f * (1.0f - 9.5367431640625e-07f), hi = R2f * (1.0f + 9.5367431640625e-07f);
+  const Inst& I = UNI ? Ip : inst[inst_of ? inst_of[i] : 0];
   const int4 pi = P[i];
   bool overflow = false;
-  RowWriter fw(nbr, n, i, 0, cap);
-  for_neighbour_runs<D, PER>(I, pi, fstart, [&](uint32_t b, uint32_t e) {
-    for (uint32_t j = b; j < e; j += 2) {
-      const uint32_t j2 = j + 1 < e ? j + 1 : j;     // odd tail: test j twice, keep once
-      bool in_a, in_b;
-      within_fast2<D, PER>(pi, P[j], P[j2], I, lo, hi, in_a, in_b);
-      if (in_a && (int64_t)j != i) fw.push((int)j, overflow);
-      if (in_b && j2 != j && (int64_t)j2 != i) fw.push((int)j2, overflow);
-    }
-  });
-  const int nf = min(fw.count, cap);
+  const int nf = min(list_neighbours<D, PER>(I, n, i, pi, P, fstart, true, 0, cap, nbr, overflow), cap);
   int nw = 0;
   if (WP && wnear[search_cell<D>(I, pi)]) {           // no wall within reach: skip the pass
-    RowWriter ww(nbr, n, i, wall_slot0(nf), cap);
-    for_neighbour_runs<D, PER>(I, pi, wstart, [&](uint32_t b, uint32_t e) {
-      for (uint32_t j = b; j < e; j += 2) {
-        const uint32_t j2 = j + 1 < e ? j + 1 : j;
-        bool in_a, in_b;
-        within_fast2<D, PER>(pi, WP[j], WP[j2], I, lo, hi, in_a, in_b);
-        if (in_a) ww.push((int)j, overflow);
-        if (in_b && j2 != j) ww.push((int)j2, overflow);
-      }
-    });
-    nw = min(ww.count, max(cap - wall_slot0(nf), 0));
+    const int w0 = wall_slot0(nf);
+    nw = min(list_neighbours<D, PER>(I, n, i, pi, WP, wstart, false, w0, cap, nbr, overflow), max(cap - w0, 0));
   }
   if (overflow) raise_error(g, ERR_CAPACITY, i);
   nbc[i] = (uint32_t)nf | ((uint32_t)nw << 16);
@@ -397,9 +407,12 @@ void launch_sort_fluid(const Buffers& b, cudaStream_t s, int64_t* launches) {
 void launch_neighbours(const Buffers& b, cudaStream_t s, int64_t* launches) {
   if (b.n == 0) return;
   const int4* wp = b.nw ? b.WP : nullptr;
-  auto kern = b.dim == 2 ? (b.any_periodic ? k_neighbours<2, true> : k_neighbours<2, false>)
-                         : (b.any_periodic ? k_neighbours<3, true> : k_neighbours<3, false>);
-  kern<<<grid_for(b.n), kBlock, 0, s>>>(b.n, b.PS, b.inst_of, b.inst, b.fstart, wp, b.wstart, b.wnear,
+  auto kern = b.n_inst == 1
+      ? (b.dim == 2 ? (b.any_periodic ? k_neighbours<2, true, true> : k_neighbours<2, false, true>)
+                    : (b.any_periodic ? k_neighbours<3, true, true> : k_neighbours<3, false, true>))
+      : (b.dim == 2 ? (b.any_periodic ? k_neighbours<2, true, false> : k_neighbours<2, false, false>)
+                    : (b.any_periodic ? k_neighbours<3, true, false> : k_neighbours<3, false, false>));
+  kern<<<grid_for(b.n), kBlock, 0, s>>>(b.inst0, b.n, b.PS, b.inst_of, b.inst, b.fstart, wp, b.wstart, b.wnear,
                                         b.cap, b.nbr, b.nbc, b.glob);
   ++*launches;
 }

@@ -54,9 +54,10 @@ template <bool PER, typename F>
 __device__ __forceinline__ void chord_runs(const Inst& I, int x, float rem, long long row, const uint32_t* start,
                                            F&& visit) {
   const int nx = I.scell[0];
-  // |dx| of a neighbour is below sqrt(rem); rsqrt-based root within 2 quanta
-  const long long xr = (long long)(rem * rsqrtf(rem)) + 2;
-  int xa = (int)(((long long)x - xr) >> I.sbits), xb = (int)(((long long)x + xr) >> I.sbits);
+  // |dx| of a neighbour is below sqrt(rem); rsqrt-based root within 2 quanta. A coordinate in
+  // the grid lies in [0, 2^31) and the root below 2^23, so the upper end fits 32 unsigned bits.
+  const int xr = (int)(rem * rsqrtf(rem)) + 2;
+  int xa = (x - xr) >> I.sbits, xb = (int)(((unsigned)x + (unsigned)xr) >> I.sbits);
   if (PER && I.period[0]) {
     if (xa < 0) {
       visit(start[row + xa + nx], start[row + nx]);
@@ -142,15 +143,15 @@ struct RowWriter {
   }
 };
 
-// Candidate test: the squared distance in FP32 from exactly converted integer
-// differences (error < 3 ulp); only inside a +-2^-20 band around the threshold is
-// the exact integer test needed, so the decision is always the integer one.
-// Two candidates at once in the lanes of packed FP32 instructions. The exact test sits
-// behind a warp vote: a warp takes it only when one of its candidates falls in the band
-// (measured 0.1 ms faster per build at 8M than selecting between the two tests).
+// Candidate test: the squared distance in FP32 from exactly converted integer differences
+// (error < 3 ulp) less R2; only within 2^-19 R2 of the threshold is the exact integer test
+// needed, so the decision is always the integer one. Two candidates at once in the lanes of
+// packed FP32 instructions; a candidate is a neighbour when its key is negative (callers take
+// the sign bit as it is). The exact test sits behind a warp vote: a warp takes it only when
+// one of its candidates falls in the band.
 template <int D, bool PER>
-__device__ __forceinline__ void within_fast2(const int4& p, const int4& a, const int4& b, const Inst& I,
-                                             float lo, float hi, bool& in_a, bool& in_b) {
+__device__ __forceinline__ float2 candidate_keys(const int4& p, const int4& a, const int4& b, const Inst& I, float R2f,
+                                                 float band) {
   const float2 M = f2(-kMagic);
   const float2 dx = add2(make_float2(biased_diff<PER>(p.x, a.x, I.period[0]), biased_diff<PER>(p.x, b.x, I.period[0])), M);
   const float2 dy = add2(make_float2(biased_diff<PER>(p.y, a.y, I.period[1]), biased_diff<PER>(p.y, b.y, I.period[1])), M);
@@ -159,13 +160,16 @@ __device__ __forceinline__ void within_fast2(const int4& p, const int4& a, const
     const float2 dz = add2(make_float2(biased_diff<PER>(p.z, a.z, I.period[2]), biased_diff<PER>(p.z, b.z, I.period[2])), M);
     d2 = fma2(dz, dz, d2);
   }
-  in_a = d2.x < lo;
-  in_b = d2.y < lo;
-  const bool ea = !in_a && d2.x < hi, eb = !in_b && d2.y < hi;
-  if (__any_sync(__activemask(), ea || eb)) {
-    if (ea) in_a = within<D>(p, a, I);
-    if (eb) in_b = within<D>(p, b, I);
+  float2 key = add2(d2, f2(-R2f));
+  if (__any_sync(__activemask(), fminf(fabsf(key.x), fabsf(key.y)) < band)) {
+    if (fabsf(key.x) < band) key.x = within<D>(p, a, I) ? -1.0f : 1.0f;
+    if (fabsf(key.y) < band) key.y = within<D>(p, b, I) ? -1.0f : 1.0f;
   }
+  return key;
+}
+// bits shifted up by one, with the sign bit of key below
+__device__ __forceinline__ unsigned push_sign(unsigned bits, float key) {
+  return __funnelshift_l(__float_as_uint(key), bits, 1);
 }
 
 // Row r of for_neighbour_runs on a grid without periodic axes, (dz, dy) = (r / 5 - 2,
@@ -188,8 +192,8 @@ __device__ __forceinline__ void row_cells(const Inst& I, const int4& p, int r, F
   if (D == 3 && gz2 >= R2m) return;
   const float rem = R2m - gz2 - gy * gy;
   if (rem <= 0.0f) return;
-  const long long xr = (long long)(rem * rsqrtf(rem)) + 2;
-  const int xa = max((int)(((long long)p.x - xr) >> sb), 0), xb = min((int)(((long long)p.x + xr) >> sb), nx - 1);
+  const int xr = (int)(rem * rsqrtf(rem)) + 2;                // as in chord_runs
+  const int xa = max((p.x - xr) >> sb, 0), xb = min((int)(((unsigned)p.x + (unsigned)xr) >> sb), nx - 1);
   if (xa > xb) return;
   const long long row = I.cell_base + ((long long)z * ny + y) * nx;
   visit(row + xa, row + xb + 1);

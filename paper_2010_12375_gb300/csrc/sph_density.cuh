@@ -90,7 +90,7 @@ __device__ __forceinline__ float density_dev(const Inst& I, int64_t i, int sub, 
 // Eq. eqviscous over the fluid pairs: (2 eta / rho_i) sum_j V_j (dW/dr)/r (v_i - v_j), pairs
 // past 2h or at zero distance adding nothing. The four records of a quad are gathered
 // together. terms (LPP > 1): this warp's [1 + D][32] float4; the result is valid on lane 0.
-template <int D, int LPP, typename PP, typename PV, typename PM, typename PN>
+template <int D, bool PER, int LPP, typename PP, typename PV, typename PM, typename PN>
 __device__ __forceinline__ float4 viscous_acc(const Inst& I, int64_t i, int sub, int nf, int64_t n, PP P, PV V, PM mass,
                                               PN nb4, float4* terms) {
   if (!(I.eta > 0.0f)) nf = 0;
@@ -119,11 +119,11 @@ __device__ __forceinline__ float4 viscous_acc(const Inst& I, int64_t i, int sub,
       float f[4], ux[4], uy[4], uz[4];
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
-        const float dx = (float)wrap_diff(pi.x - pj[k].x, I.period[0]) * I.dq;
-        const float dy = (float)wrap_diff(pi.y - pj[k].y, I.period[1]) * I.dq;
+        const float dx = (float)wrap_diff(pi.x - pj[k].x, PER ? I.period[0] : 0) * I.dq;
+        const float dy = (float)wrap_diff(pi.y - pj[k].y, PER ? I.period[1] : 0) * I.dq;
         float r2 = dx * dx + dy * dy;
         if (D == 3) {
-          const float dz = (float)wrap_diff(pi.z - pj[k].z, I.period[2]) * I.dq;
+          const float dz = (float)wrap_diff(pi.z - pj[k].z, PER ? I.period[2] : 0) * I.dq;
           r2 += dz * dz;
         }
         const float fw = kernel_dW_over_r(sqrtf(r2), I);            // (dW/dr)/r

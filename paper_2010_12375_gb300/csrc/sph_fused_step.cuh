@@ -118,8 +118,7 @@ __device__ __forceinline__ uint32_t search_group(const Buffers& b, const Inst& I
                                                  const int4* P) {
   constexpr int kRows = D == 3 ? 25 : 5;
   static_assert(LS >= kRows, "a lane per search row");
-  const float R2f = (float)I.R2;
-  const float lo = R2f * (1.0f - 9.5367431640625e-07f), hi = R2f * (1.0f + 9.5367431640625e-07f);
+  const float R2f = (float)I.R2, band = R2f * 1.9073486328125e-06f;
   const uint32_t me = (uint32_t)i;
   uint32_t s[2] = {0u, 0u}, e[2] = {0u, 0u};      // the row's run of fluid and of wall records
   if (r < kRows)
@@ -137,12 +136,12 @@ __device__ __forceinline__ uint32_t search_group(const Buffers& b, const Inst& I
     for (uint32_t k = 0; k < 4; ++k) p[k] = R[min(j + k, end - 1)];
   };
   auto test = [&](const int4 (&p)[4], uint32_t j, uint32_t end, uint32_t skip) {
-    bool in[4];
-    within_fast2<D, false>(pi, p[0], p[1], I, lo, hi, in[0], in[1]);
-    within_fast2<D, false>(pi, p[2], p[3], I, lo, hi, in[2], in[3]);
+    const float2 k01 = candidate_keys<D, false>(pi, p[0], p[1], I, R2f, band);
+    const float2 k23 = candidate_keys<D, false>(pi, p[2], p[3], I, R2f, band);
+    const float key[4] = {k01.x, k01.y, k23.x, k23.y};
     unsigned h = 0;
 #pragma unroll
-    for (uint32_t k = 0; k < 4; ++k) h |= (unsigned)(in[k] && j + k < end && j + k != skip) << k;
+    for (uint32_t k = 0; k < 4; ++k) h |= (unsigned)(key[k] < 0.0f && j + k < end && j + k != skip) << k;
     return h;
   };
   int4 pf[4], pw[4];
@@ -192,8 +191,7 @@ __device__ __forceinline__ uint32_t search_group_periodic(const Buffers& b, cons
                                                  const int4* P) {
   constexpr int kRows = D == 3 ? 25 : 5;
   static_assert(LS >= kRows, "a lane per search row");
-  const float R2f = (float)I.R2;
-  const float lo = R2f * (1.0f - 9.5367431640625e-07f), hi = R2f * (1.0f + 9.5367431640625e-07f);
+  const float R2f = (float)I.R2, band = R2f * 1.9073486328125e-06f;
   const unsigned gm = search_mask<LS>();
   bool overflow = false;
   // all hits of one cell-linked list into the row from slot0 on; returns their number
@@ -206,9 +204,9 @@ __device__ __forceinline__ uint32_t search_group_periodic(const Buffers& b, cons
       for (uint32_t j = s; j < e; j += 4) {
         const uint32_t j1 = min(j + 1, e - 1), j2 = min(j + 2, e - 1), j3 = min(j + 3, e - 1);
         const int4 p0 = R[j], p1 = R[j1], p2 = R[j2], p3 = R[j3];
-        bool in0, in1, in2, in3;
-        within_fast2<D, PER>(pi, p0, p1, I, lo, hi, in0, in1);
-        within_fast2<D, PER>(pi, p2, p3, I, lo, hi, in2, in3);
+        const float2 k01 = candidate_keys<D, PER>(pi, p0, p1, I, R2f, band);
+        const float2 k23 = candidate_keys<D, PER>(pi, p2, p3, I, R2f, band);
+        const bool in0 = k01.x < 0.0f, in1 = k01.y < 0.0f, in2 = k23.x < 0.0f, in3 = k23.y < 0.0f;
         take(j, (unsigned)(in0 && j != me) | (unsigned)(in1 && j + 1 < e && j1 != me) << 1 |
                     (unsigned)(in2 && j + 2 < e && j2 != me) << 2 | (unsigned)(in3 && j + 3 < e && j3 != me) << 3);
       }
@@ -380,7 +378,7 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
     if (!grid_barrier(&c->count, target, g)) return;
     if (b.acc_prior) {   // read back by the lane that wrote it: no barrier
       for (int64_t i = first; i < n; i += step) {
-        const float4 a = viscous_acc<D, LPP>(I, i, sub, (int)(b.nbc[i] & 0xffffu), n, (const int4*)b.PS,
+        const float4 a = viscous_acc<D, PER, LPP>(I, i, sub, (int)(b.nbc[i] & 0xffffu), n, (const int4*)b.PS,
                                              (const float4*)b.VS, (const float*)b.mass, nb4, terms);
         if (sub == 0) b.acc_prior[i] = a;
       }

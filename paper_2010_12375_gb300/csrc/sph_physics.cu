@@ -283,7 +283,7 @@ k_density(int64_t n, int4* P, const int* __restrict__ inst_of, const Inst* __res
   reinterpret_cast<int*>(P + i)[3] = f2i(dev);        // only .w changes; others read .xyz
 }
 
-template <int D>
+template <int D, bool PER>
 __global__ void __launch_bounds__(kBlock)
 k_viscous(int64_t n, const int4* __restrict__ P, const float4* __restrict__ V,
           const float* __restrict__ mass, const int* __restrict__ inst_of,
@@ -292,7 +292,7 @@ k_viscous(int64_t n, const int4* __restrict__ P, const float4* __restrict__ V,
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const Inst& I = inst[inst_index(inst_of, i)];
-  acc_prior[i] = viscous_acc<D, 1>(I, i, 0, (int)(nbc[i] & 0xffffu), n, P, V, mass,
+  acc_prior[i] = viscous_acc<D, PER, 1>(I, i, 0, (int)(nbc[i] & 0xffffu), n, P, V, mass,
                                    reinterpret_cast<const int4*>(nbr), nullptr);
 }
 
@@ -374,8 +374,9 @@ void launch_density(const Buffers& b, cudaStream_t s, int64_t* launches) {
 
 void launch_viscous(const Buffers& b, cudaStream_t s, int64_t* launches) {
   if (b.n == 0 || !b.acc_prior) return;
-  SPH_DIM_LAUNCH(b, k_viscous, grid_for(b.n), kBlock, s, b.n, b.PS, b.VS, b.mass, b.inst_of, b.inst,
-                 b.nbr, b.nbc, b.acc_prior);
+  auto kern = b.dim == 2 ? (b.any_periodic ? k_viscous<2, true> : k_viscous<2, false>)
+                         : (b.any_periodic ? k_viscous<3, true> : k_viscous<3, false>);
+  kern<<<grid_for(b.n), kBlock, 0, s>>>(b.n, b.PS, b.VS, b.mass, b.inst_of, b.inst, b.nbr, b.nbc, b.acc_prior);
   ++*launches;
 }
 
