@@ -521,6 +521,20 @@ std::string format_cfg(const sph::LaunchCfg& c) {
   return o.str();
 }
 
+// Launch configuration of a handle that no autotuned entry covers (every configuration gives
+// the same bits). One thread per particle: in 2D in blocks of 128 (pressure / density
+// relaxation 70 / 60 us at 980,000 particles, 77 / 62 in blocks of 256, 68 / 66 as row tasks);
+// in 3D in blocks of 256 below 300,000 particles, where blocks of 128 leave a fuller last wave
+// (62 / 59 against 69 / 61 us at 208,000), of 128 above (117 / 106 against 119 / 110 us at
+// 432,000), and as row tasks from 900,000 on (218 / 208 against 234 / 217 us at 1.02M, 796 /
+// 769 against 826 / 780 us at 4.0M; even at 2.0M, and 169 / 166 against 169 / 154 us at 686,000).
+sph::LaunchCfg default_launch(int dim, int64_t n, bool single) {
+  sph::LaunchCfg c;
+  c.pr_block = c.dr_block = dim == 2 || n >= 300000 ? 128 : 256;
+  if (dim == 3 && single && n >= 900000) c.pr_block = c.dr_block = sph::kRowBlock;
+  return c;
+}
+
 void drop_graph(sph_handle* h) {
   if (h->gexec) cudaGraphExecDestroy(h->gexec);
   if (h->graph) cudaGraphDestroy(h->graph);
@@ -738,6 +752,7 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
   }
   sph::sort_walls(b, b.PH, b.VH, b.wid, s);
   sph::flag_near_wall_cells(b, reinterpret_cast<uint8_t*>(b.count), s);   // count: scratch here
+  b.cfg = default_launch(b.dim, b.n, n_instances == 1);
   {
     const auto cache = read_autotune_cache();
     const auto it = cache.find(autotune_key(h));
