@@ -475,299 +475,417 @@ __global__ void k_segsum(int64_t n, const uint32_t* __restrict__ off, const floa
   XN[i * 144 + F + f] = __float2bfloat16_rn(s * inv_nbar);
 }
 
-// Edge network of one round, fused for inference. Each warp takes a run of kFuseNodes
-// nodes and walks their edges in 16-row tiles. The next tile's h_j rows and static edge
-// features are loaded (whole rows, 16-byte pieces) while the current tile is multiplied,
-// and the neighbour indices one tile ahead of that. A tile's A fragments are read from a
-// per-warp staging copy of those rows, column by column as k_edge_rows lays a round input
-// row out (static features, bf16(h_j) or zero for a wall, the bias 1, zero padding). Both
+// Edge network of one round, fused for inference. Each warp takes a run of nodes and walks
+// their edges in 32-row tiles. A tile's rows are assembled as k_edge_rows lays a round input
+// row out (static features, bf16(h_j) or zero for a wall, the bias 1, zero padding) in one
+// of the warp's two buffers: 16-byte pieces of the neighbours' row templates (see
+// k_node_templates) by cp.async, and the one piece that holds static features and node state
+// merged in registers, all one tile ahead of the products, the neighbour indices two. Both
 // edge layers run on the tensor cores (mma.sync m16n8k16, k-steps in k_dense's order; the
 // first layer's accumulators become the second layer's A fragments after k_dense's ReLU
 // and bfloat16 rounding), and the messages are added per node in edge order as k_segsum
 // does. After its edges, the run's node rows go through the node network (both node
-// layers, the update added to h) into the other node-state buffer. XN and the new node
-// states are therefore bit-identical to the unfused path's, and no per-edge row,
-// activation or message goes to memory.
-constexpr int kFuseWarps = 8;
-constexpr int kFuseNodes = 8;
-constexpr int kFuseLd = 88;                   // padded weight row of 80 bf16
-constexpr int kStageLd = 68;                  // staged h row: 64 floats + pad (16-byte rows)
-constexpr int kStageWords = 16 * kStageLd + 16 * 8;   // h rows, then the static features (bf16 pairs)
-constexpr int kMsgLd = 72;                    // message row stride: conflict-free float2 stores
+// layers, the update added to h) into the other node-state buffer and, as the next round's
+// templates (after the last round the decoder's input rows), into Tout. The new node states
+// are therefore bit-identical to the unfused path's, and no per-edge row, activation or
+// message goes to memory.
+// What bounds it: the shared-memory pipe. A warp reads 20 KB of weight fragments per tile,
+// so a tile has 32 rows, whose two m16 halves share them, and the operands are read by
+// ldmatrix from bf16 rows; with 16-row tiles of FP32 node states, converted element by
+// element, the pipe moved about twice the bytes for a row and took 263 us a round
+// at 100,128 particles (2.7 M edges) against 154 us now, at 68 % of the pipe and 49 % of the
+// mma.sync rate; 12 warps with 168 registers 170 us, 14 that spill 181 us.
+constexpr int kFuseWarps = 16;                // one block an SM, 128 registers a thread
+constexpr int kFuseRun = 64;                  // nodes in a run, at most (their edge offsets stay in two registers)
+constexpr int kFuseRunMin = 4;
+constexpr int kFuseBuf = 32 * 80;             // bf16 elements of one tile buffer
+constexpr int kMsgLd = 40;                    // message row stride: 32 columns + pad, conflict-free float2 stores
 
-static_assert(16 * kMsgLd <= kStageWords, "messages must fit the staging area");
-
-constexpr int kNodeLd = 152;                  // padded weight row of 144 bf16 (node layer 1)
+static_assert(32 * kMsgLd * sizeof(float) <= kFuseBuf * sizeof(bf16), "32 columns of messages must fit a tile buffer");
 
 inline size_t fused_smem() {
-  return (size_t)(3 * 64 * kFuseLd + 64 * kNodeLd) * sizeof(bf16) + (size_t)kFuseWarps * kStageWords * sizeof(float);
+  return (size_t)(3 * 64 * 80 + 64 * 144 + kFuseWarps * 2 * kFuseBuf) * sizeof(bf16);
 }
 
-// column of slot q (0..19) of a lane with quad index t: k-step q / 4, position q % 4 in
-// {0, 1, 8, 9}
-__device__ __forceinline__ int fuse_col(int q, int t) { return (q >> 2) * 16 + 2 * t + (q & 1) + ((q >> 1) & 1) * 8; }
+// Column c of row r in a row-major operand of 80 or 144 columns: pieces of 8 columns trade
+// places in pairs in every second group of four rows, so that the eight rows of an ldmatrix
+// (10 or 18 pieces apart) lie in different banks without padding.
+__device__ __forceinline__ int fuse_at(int ld, int r, int c) { return r * ld + (c ^ ((r & 4) << 1)); }
 
-// B fragments of two n-tiles (nt, nt + 1) at k-step k0 from a row-major [n][kFuseLd] weight
-// copy: lane i addresses row i % 8 of 8x8 matrix i / 8 (matrices: (nt, k0), (nt, k0 + 8),
-// (nt + 1, k0), (nt + 1, k0 + 8)), and receives row lane / 4, columns 2 (lane % 4), +1 of
-// each, which is the m16n8k16 B fragment.
-template <int LD = kFuseLd>
-__device__ __forceinline__ void ldsm_b4(const bf16* W, int nt, int k0, int lane, uint32_t& b0, uint32_t& b1,
-                                        uint32_t& c0, uint32_t& c1) {
-  const int m = lane >> 3;
-  const bf16* p = W + ((nt + (m >> 1)) * 8 + (lane & 7)) * LD + k0 + (m & 1) * 8;
-  const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+__device__ __forceinline__ void ldsm_x4(uint32_t a, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(b0), "=r"(b1), "=r"(c0), "=r"(c1)
-               : "r"(a));
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(a)
+               : "memory");
 }
 
-// bf16 of column c of a staged row: static feature, h value, bias or zero padding
-template <int FE>
-__device__ __forceinline__ bf16 fuse_elem(const float* __restrict__ hrow, const bf16* __restrict__ xrow, int c,
-                                          bool valid) {
-  if (c < FE) return xrow[c];
-  if (c < FE + F) return __float2bfloat16_rn(hrow[c - FE]);
-  return __float2bfloat16_rn(valid && c == FE + F ? 1.0f : 0.f);
+// This lane's ldmatrix address in an [n][ld] weight copy, and the B fragments of two n-tiles
+// (nt, nt + 1) at k-step k0 read with it: lane i addresses row i % 8 of 8x8 matrix i / 8
+// (matrices: (nt, k0), (nt, k0 + 8), (nt + 1, k0), (nt + 1, k0 + 8)), and receives row
+// lane / 4, columns 2 (lane % 4), +1 of each, which is the m16n8k16 B fragment.
+__device__ __forceinline__ uint32_t b_lane(const bf16* W, int ld, int lane) {
+  return tc::smem_u32(W + fuse_at(ld, (lane >> 4) * 8 + (lane & 7), ((lane >> 3) & 1) * 8));
+}
+template <int LD = 80>
+__device__ __forceinline__ void ldsm_b4(uint32_t base, int nt, int k0, uint32_t& b0, uint32_t& b1, uint32_t& c0,
+                                        uint32_t& c1) {
+  ldsm_x4(base + (nt * 8 * LD + k0) * 2, b0, b1, c0, c1);
 }
 
+// The same for the A fragments of rows r0 .. r0 + 15 of an [.][80] tile: matrices (rows 0..7,
+// k0), (rows 8..15, k0), (rows 0..7, k0 + 8), (rows 8..15, k0 + 8)
+__device__ __forceinline__ uint32_t a_lane(const bf16* X, int lane) {
+  return tc::smem_u32(X + fuse_at(80, lane & 15, (lane >> 4) * 8));
+}
+__device__ __forceinline__ void ldsm_a4(uint32_t base, int r0, int k0, uint32_t* r) {
+  ldsm_x4(base + (r0 * 80 + k0) * 2, r[0], r[1], r[2], r[3]);
+}
+
+// bf16(relu(lo)), bf16(relu(hi)): rounded by one packed conversion, then clamped (rounding
+// keeps the sign; a NaN becomes 0 as under fmaxf)
+__device__ __forceinline__ uint32_t relu2(float lo, float hi) {
+  const __nv_bfloat162 v = __hmax2(__floats2bfloat162_rn(lo, hi), __floats2bfloat162_rn(0.f, 0.f));
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+
+// A fragments of the layer after a 64-wide one, from its accumulators: [bf16(relu(z)), 1, 0...]
+__device__ __forceinline__ void relu_frags(const float (*acc)[4], uint32_t (*A)[4]) {
+#pragma unroll
+  for (int kk = 0; kk < 4; ++kk) {
+    const float* lo = acc[2 * kk];
+    const float* hi = acc[2 * kk + 1];
+    A[kk][0] = relu2(lo[0], lo[1]);
+    A[kk][1] = relu2(lo[2], lo[3]);
+    A[kk][2] = relu2(hi[0], hi[1]);
+    A[kk][3] = relu2(hi[2], hi[3]);
+  }
+}
+
+// read-only loads that stay where they are written: issued a tile before their use, and not
+// moved down to it
+__device__ __forceinline__ uint4 ld_early(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_early(const uint16_t* p) {
+  uint32_t v;
+  asm volatile("ld.global.nc.u16 %0, [%1];\n" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int ld_early(const int* p) {
+  int v;
+  asm volatile("ld.global.nc.s32 %0, [%1];\n" : "=r"(v) : "l"(p));
+  return v;
+}
+
+// Templates T: row 0 serves wall neighbours, row j + 1 fluid node j. Tout: row i at
+// 80 i, its 64 node-state columns at ocol (then the bias 1, zeros elsewhere); with ocol > 0
+// it is the next round's templates, whose row 0 (at -80) is written too.
 template <int FE>
-__global__ void __launch_bounds__(kFuseWarps * 32, 2)
-k_edge_round_fused(int64_t n, const uint32_t* __restrict__ off, const bf16* __restrict__ XS,
-                   const int* __restrict__ enbr, const float* __restrict__ H, const bf16* __restrict__ W1,
-                   const bf16* __restrict__ W2, const bf16* __restrict__ Wn1, const bf16* __restrict__ Wn2,
-                   float inv_nbar, bf16* __restrict__ XN, float* __restrict__ Hout) {
+__global__ void __launch_bounds__(kFuseWarps * 32, 1)
+k_edge_round_fused(int64_t n, int run, const uint32_t* __restrict__ off, const bf16* __restrict__ XS,
+                   const int* __restrict__ enbr, const float* __restrict__ H, const bf16* __restrict__ T,
+                   const bf16* __restrict__ W1, const bf16* __restrict__ W2, const bf16* __restrict__ Wn1,
+                   const bf16* __restrict__ Wn2, float inv_nbar, bf16* __restrict__ XN, float* __restrict__ Hout,
+                   bf16* __restrict__ Tout, int ocol) {
+  constexpr int MP = FE / 8;                  // the piece of static features and node state
+  static_assert((FE == 7 || FE == 9) && FE + F + 1 <= 8 * (MP + 9), "pieces MP + 1 .. MP + 8 hold the rest of a row");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
   bf16* sW1 = reinterpret_cast<bf16*>(smem_raw);
-  bf16* sW2 = sW1 + 64 * kFuseLd;
-  bf16* sN2 = sW2 + 64 * kFuseLd;             // node layer 2, rows of kFuseLd
-  bf16* sN1 = sN2 + 64 * kFuseLd;             // node layer 1, rows of kNodeLd
-  float* stage = reinterpret_cast<float*>(sN1 + 64 * kNodeLd) + warp * kStageWords;   // h rows
-  bf16* xstage = reinterpret_cast<bf16*>(stage + 16 * kStageLd);                       // [16][16]
-  float* sM = stage;                          // the messages reuse the staging rows (16 x kMsgLd)
+  bf16* sW2 = sW1 + 64 * 80;
+  bf16* sN2 = sW2 + 64 * 80;                  // node layer 2
+  bf16* sN1 = sN2 + 64 * 80;                  // node layer 1, 144 columns
+  bf16* buf = sN1 + 64 * 144 + warp * 2 * kFuseBuf;
   for (int idx = threadIdx.x; idx < 64 * 10; idx += blockDim.x) {
-    const int r = idx / 10, c = (idx % 10) * 8;
-    *reinterpret_cast<uint4*>(&sW1[r * kFuseLd + c]) = *reinterpret_cast<const uint4*>(&W1[r * 80 + c]);
-    *reinterpret_cast<uint4*>(&sW2[r * kFuseLd + c]) = *reinterpret_cast<const uint4*>(&W2[r * 80 + c]);
-    *reinterpret_cast<uint4*>(&sN2[r * kFuseLd + c]) = *reinterpret_cast<const uint4*>(&Wn2[r * 80 + c]);
+    const int r = idx / 10, c = (idx % 10) * 8, o = fuse_at(80, r, c);
+    *reinterpret_cast<uint4*>(&sW1[o]) = *reinterpret_cast<const uint4*>(&W1[r * 80 + c]);
+    *reinterpret_cast<uint4*>(&sW2[o]) = *reinterpret_cast<const uint4*>(&W2[r * 80 + c]);
+    *reinterpret_cast<uint4*>(&sN2[o]) = *reinterpret_cast<const uint4*>(&Wn2[r * 80 + c]);
   }
   for (int idx = threadIdx.x; idx < 64 * 18; idx += blockDim.x) {
     const int r = idx / 18, c = (idx % 18) * 8;
-    *reinterpret_cast<uint4*>(&sN1[r * kNodeLd + c]) = *reinterpret_cast<const uint4*>(&Wn1[r * 144 + c]);
+    *reinterpret_cast<uint4*>(&sN1[fuse_at(144, r, c)]) = *reinterpret_cast<const uint4*>(&Wn1[r * 144 + c]);
   }
   __syncthreads();
-  const int64_t chunks = (n + kFuseNodes - 1) / kFuseNodes;
-  for (int64_t ch = (int64_t)blockIdx.x * kFuseWarps + warp; ch < chunks; ch += (int64_t)gridDim.x * kFuseWarps) {
-    const int64_t i0 = ch * kFuseNodes, i1 = min(i0 + (int64_t)kFuseNodes, n);
+  if (ocol > 0 && blockIdx.x == 0 && threadIdx.x < 80)   // the wall template of the next round
+    Tout[(int)threadIdx.x - 80] = __float2bfloat16_rn((int)threadIdx.x == ocol + F ? 1.0f : 0.f);
+  const uint32_t w1_base = b_lane(sW1, 80, lane), n1_base = b_lane(sN1, 144, lane), a_base = a_lane(buf, lane);
+  const uint32_t bias = t == 0 ? pack2(__float2bfloat16_rn(1.0f), __float2bfloat16_rn(0.f)) : 0u;
+  const int64_t runs = (n + run - 1) / run;
+  // few runs: over the blocks first, then over a block's warps
+  for (int64_t rr = (int64_t)warp * gridDim.x + blockIdx.x; rr < runs; rr += (int64_t)gridDim.x * kFuseWarps) {
+    const int64_t i0 = rr * run, i1 = min(i0 + (int64_t)run, n);
+    const int nodes = (int)(i1 - i0);
     const uint32_t e_begin = off[i0], e_end = off[i1];
-    int64_t cur = i0;                         // node whose sum is open
-    uint32_t cur_end = off[cur + 1];
-    float s0 = 0.f, s1 = 0.f;                 // this lane's columns 2 lane, 2 lane + 1
-    // close every node whose edges end at or before edge e (edgeless nodes included)
-    auto close_until = [&](uint32_t e) {
-      while (cur < i1 && cur_end <= e) {
-        const int f = 2 * lane;
-        const float2 hv = *reinterpret_cast<const float2*>(&H[cur * F + f]);
-        *reinterpret_cast<uint32_t*>(&XN[cur * 144 + f]) = pack2(__float2bfloat16_rn(hv.x), __float2bfloat16_rn(hv.y));
-        *reinterpret_cast<uint32_t*>(&XN[cur * 144 + F + f]) =
-            pack2(__float2bfloat16_rn(s0 * inv_nbar), __float2bfloat16_rn(s1 * inv_nbar));
-        s0 = s1 = 0.f;
+    // ends of the run's nodes: node k in lane k % 32 of register k / 32
+    const uint32_t endA = off[min(i0 + lane + 1, i1)], endB = off[min(i0 + lane + 33, i1)];
+    auto end_of = [&](int k) {
+      const uint32_t a = __shfl_sync(0xffffffffu, endA, k & 31), b = __shfl_sync(0xffffffffu, endB, k & 31);
+      return k < 32 ? a : b;
+    };
+    // The open node and, per half of the 64 columns, its sum in column 32 half + lane. Nodes
+    // that end at or before edge e are closed (edgeless ones included); both halves pass the
+    // same nodes, so the second returns to where the first began.
+    int cur = 0;
+    uint32_t cur_end = end_of(0);
+    float sum[2] = {0.f, 0.f};
+    auto close_until = [&](uint32_t e, int half) {
+      while (cur < nodes && cur_end <= e) {
+        XN[(i0 + cur) * 144 + F + 32 * half + lane] = __float2bfloat16_rn(sum[half] * inv_nbar);
+        sum[half] = 0.f;
         ++cur;
-        if (cur < i1) cur_end = off[cur + 1];
+        cur_end = end_of(cur & 63);           // past the run's last node: not used
       }
     };
-    close_until(e_begin);
-    // neighbour index of row `lane` (lanes 0..15) of the tile at t0, -1 past the end
-    auto idx_of = [&](uint32_t t0) { return lane < 16 && t0 + lane < e_end ? __ldg(&enbr[t0 + lane]) : -1; };
-    // the tile's rows: piece p of lane l is row 2p + l / 16, floats 4 (l % 16) .. + 3
-    float4 hq[8];
-    uint4 xq;
-    auto load_tile = [&](uint32_t t0, int jrow) {
+    // neighbour of edge t0 + lane (not worked on until its use, a tile later); rows past the
+    // end repeat the last edge
+    auto idx_of = [&](uint32_t t0) { return ld_early(&enbr[min(t0 + lane, e_end - 1)]); };
+    // this lane's row: piece MP and the one element of it that comes from the other source
+    // (7 static features: XS and element 7 of T; 9: T and element 0 of XS)
+    uint4 mq;
+    uint32_t me;
+    auto load_tile = [&](uint32_t t0, int nb, bf16* dst) {
+      const int jrow = max(nb, -1) + 1;       // template row
 #pragma unroll
       for (int p = 0; p < 8; ++p) {
-        const int row = 2 * p + (lane >> 4);
+        const int row = 4 * p + (lane >> 3), c = (MP + 1 + (lane & 7)) * 8;
         const int j = __shfl_sync(0xffffffffu, jrow, row);
-        hq[p] = (t0 + row < e_end && j >= 0) ? __ldg(reinterpret_cast<const float4*>(&H[(int64_t)j * F]) + (lane & 15))
-                                             : make_float4(0.f, 0.f, 0.f, 0.f);
+        cp_async16(dst + fuse_at(80, row, c), T + (int64_t)j * 80 + c, true);
       }
-      const int xrow = lane >> 1;
-      xq = t0 + xrow < e_end ? __ldg(reinterpret_cast<const uint4*>(&XS[((int64_t)t0 + xrow) * 16]) + (lane & 1))
-                             : make_uint4(0u, 0u, 0u, 0u);
+      const bf16* x = XS + (int64_t)min(t0 + lane, e_end - 1) * 16;
+      if (MP) cp_async16(dst + fuse_at(80, lane, 0), x, true);
+      cp_async_commit();
+      const bf16* tj = T + (int64_t)jrow * 80 + MP * 8;
+      mq = ld_early(reinterpret_cast<const uint4*>(MP ? tj : x));
+      me = ld_early(reinterpret_cast<const uint16_t*>(MP ? x + 8 : tj + 7));
     };
-    load_tile(e_begin, idx_of(e_begin));
-    int jn = idx_of(e_begin + 16);
-    for (uint32_t t0 = e_begin; t0 < e_end; t0 += 16) {
-      // stage the current tile's rows and read this lane's A fragments of the first layer
-#pragma unroll
-      for (int p = 0; p < 8; ++p)
-        *reinterpret_cast<float4*>(&stage[(2 * p + (lane >> 4)) * kStageLd + 4 * (lane & 15)]) = hq[p];
-      *reinterpret_cast<uint4*>(&xstage[(lane >> 1) * 16 + 8 * (lane & 1)]) = xq;
+    int jn = 0;
+    if (e_begin < e_end) {
+      load_tile(e_begin, idx_of(e_begin), buf);
+      jn = idx_of(e_begin + 32);
+    }
+    int par = 0;
+    for (uint32_t t0 = e_begin; t0 < e_end; t0 += 32, par ^= 1) {
+      bf16* tile = buf + par * kFuseBuf;
+      if (MP) mq.x = (mq.x & 0xffff0000u) | me;
+      else mq.w = (mq.w & 0x0000ffffu) | (me << 16);
+      *reinterpret_cast<uint4*>(&tile[fuse_at(80, lane, MP * 8)]) = mq;
+      if (MP == 0) *reinterpret_cast<uint4*>(&tile[fuse_at(80, lane, 72)]) = make_uint4(0u, 0u, 0u, 0u);
+      cp_async_wait_all();
       __syncwarp();
-      const bool va = t0 + g < e_end, vb = t0 + g + 8 < e_end;
-      const float* ha = stage + g * kStageLd;
-      const float* hb = ha + 8 * kStageLd;
-      const bf16* xa = xstage + g * 16;
-      const bf16* xb = xa + 8 * 16;
-      uint32_t A[5][4];
+      // next tile's rows in flight during this tile's products
+      if (t0 + 32 < e_end) {
+        load_tile(t0 + 32, jn, buf + (par ^ 1) * kFuseBuf);
+        jn = idx_of(t0 + 64);
+      }
+      const uint32_t at = a_base + par * kFuseBuf * 2;
+      float acc[2][8][4];
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) acc[q][nt][0] = acc[q][nt][1] = acc[q][nt][2] = acc[q][nt][3] = 0.f;
 #pragma unroll
       for (int kk = 0; kk < 5; ++kk) {
+        uint32_t A0[4], A1[4];
+        ldsm_a4(at, 0, kk * 16, A0);
+        ldsm_a4(at, 16, kk * 16, A1);
+#pragma unroll
+        for (int nt = 0; nt < 8; nt += 2) {
+          uint32_t b0, b1, c0, c1;
+          ldsm_b4(w1_base, nt, kk * 16, b0, b1, c0, c1);
+          mma16816(acc[0][nt], A0[0], A0[1], A0[2], A0[3], b0, b1);
+          mma16816(acc[0][nt + 1], A0[0], A0[1], A0[2], A0[3], c0, c1);
+          mma16816(acc[1][nt], A1[0], A1[1], A1[2], A1[3], b0, b1);
+          mma16816(acc[1][nt + 1], A1[0], A1[1], A1[2], A1[3], c0, c1);
+        }
+      }
+      uint32_t Z[2][4][4];
+      relu_frags(acc[0], Z[0]);
+      relu_frags(acc[1], Z[1]);
+      // second layer and the messages, 32 columns at a time, through the tile's buffer
+      float* sM = reinterpret_cast<float*>(tile);
+      const int cur0 = cur;
+      const uint32_t cur_end0 = cur_end;
+#pragma unroll
+      for (int half = 0; half < 2; ++half) {
+        float out[2][4][4];
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) out[q][nt][0] = out[q][nt][1] = out[q][nt][2] = out[q][nt][3] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < 5; ++kk)
+#pragma unroll
+          for (int nt = 0; nt < 4; nt += 2) {
+            uint32_t b0, b1, c0, c1;
+            ldsm_b4(w1_base + 64 * 80 * 2, 4 * half + nt, kk * 16, b0, b1, c0, c1);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const uint32_t a0 = kk < 4 ? Z[q][kk & 3][0] : bias, a1 = kk < 4 ? Z[q][kk & 3][1] : bias;
+              const uint32_t a2 = kk < 4 ? Z[q][kk & 3][2] : 0u, a3 = kk < 4 ? Z[q][kk & 3][3] : 0u;
+              mma16816(out[q][nt], a0, a1, a2, a3, b0, b1);
+              mma16816(out[q][nt + 1], a0, a1, a2, a3, c0, c1);
+            }
+          }
+        __syncwarp();                         // layer 1's rows, or the first half's messages, read
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+#pragma unroll
+          for (int nt = 0; nt < 4; ++nt) {
+            float* m = &sM[(16 * q + g) * kMsgLd + nt * 8 + 2 * t];
+            *reinterpret_cast<float2*>(m) = make_float2(out[q][nt][0], out[q][nt][1]);
+            *reinterpret_cast<float2*>(m + 8 * kMsgLd) = make_float2(out[q][nt][2], out[q][nt][3]);
+          }
+        __syncwarp();
+        cur = cur0;
+        cur_end = cur_end0;
+        const int rows = (int)min(32u, e_end - t0);
+        for (int r = 0; r < rows;) {
+          close_until(t0 + (uint32_t)r, half);
+          // rows r .. r1 - 1 belong to the open node
+          const int r1 = (int)min((uint32_t)rows, cur_end - t0);
+          for (; r + 8 <= r1; r += 8) {
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = sM[(r + k) * kMsgLd + lane];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sum[half] += v[k];
+          }
+          if (r < r1) {                       // +0 leaves a sum that started at +0 unchanged, bit for bit
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = sM[min(r + k, 31) * kMsgLd + lane];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) sum[half] += r + k < r1 ? v[k] : 0.f;
+            r = r1;
+          }
+        }
+      }
+      __syncwarp();                           // the buffer is free for the tile after the next
+    }
+    {
+      const int cur0 = cur;
+      const uint32_t cur_end0 = cur_end;
+      close_until(e_end, 0);
+      cur = cur0;
+      cur_end = cur_end0;
+      close_until(e_end, 1);
+    }
+    __syncwarp();                             // the run's sums in XN, written above, visible
+    // node network of the run, 16 nodes at a time, as the unfused node layers compute it:
+    // z = relu(W_n1 [h, a, 1]), h_out = h + W_n2 [z, 1]
+    for (int m0 = 0; m0 < nodes; m0 += 16) {
+      const int64_t ib = i0 + m0;
+      const int left = nodes - m0;
+      const bool vg = g < left, vh = g + 8 < left;
+      const float* hg = H + (ib + (vg ? g : 0)) * F;
+      const float* hh = H + (ib + (vh ? g + 8 : 0)) * F;
+      const bf16* xg = XN + (ib + (vg ? g : 0)) * 144;
+      const bf16* xh = XN + (ib + (vh ? g + 8 : 0)) * 144;
+      auto state = [&](const float* p) {
+        const float2 v = *reinterpret_cast<const float2*>(p);
+        return pack2(__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y));
+      };
+      uint32_t A[9][4];
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
         const int c = kk * 16 + 2 * t;
-        A[kk][0] = pack2(fuse_elem<FE>(ha, xa, c, va), fuse_elem<FE>(ha, xa, c + 1, va));
-        A[kk][1] = pack2(fuse_elem<FE>(hb, xb, c, vb), fuse_elem<FE>(hb, xb, c + 1, vb));
-        A[kk][2] = pack2(fuse_elem<FE>(ha, xa, c + 8, va), fuse_elem<FE>(ha, xa, c + 9, va));
-        A[kk][3] = pack2(fuse_elem<FE>(hb, xb, c + 8, vb), fuse_elem<FE>(hb, xb, c + 9, vb));
+        A[kk][0] = state(hg + c);
+        A[kk][1] = state(hh + c);
+        A[kk][2] = state(hg + c + 8);
+        A[kk][3] = state(hh + c + 8);
+        A[kk + 4][0] = ld_u32(xg + F + c);
+        A[kk + 4][1] = ld_u32(xh + F + c);
+        A[kk + 4][2] = ld_u32(xg + F + c + 8);
+        A[kk + 4][3] = ld_u32(xh + F + c + 8);
       }
-      __syncwarp();                           // staging read: free for the messages
-      // next tile's rows in flight during this tile's products
-      const uint32_t t1 = t0 + 16;
-      if (t1 < e_end) {
-        load_tile(t1, jn);
-        jn = idx_of(t1 + 16);
-      }
+      A[8][0] = A[8][1] = bias;
+      A[8][2] = A[8][3] = 0u;
       float acc[8][4];
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
 #pragma unroll
-      for (int kk = 0; kk < 5; ++kk)
+      for (int kk = 0; kk < 9; ++kk)
 #pragma unroll
         for (int nt = 0; nt < 8; nt += 2) {
           uint32_t b0, b1, c0, c1;
-          ldsm_b4(sW1, nt, kk * 16, lane, b0, b1, c0, c1);
+          ldsm_b4<144>(n1_base, nt, kk * 16, b0, b1, c0, c1);
           mma16816(acc[nt], A[kk][0], A[kk][1], A[kk][2], A[kk][3], b0, b1);
           mma16816(acc[nt + 1], A[kk][0], A[kk][1], A[kk][2], A[kk][3], c0, c1);
         }
-      // second layer: A = [bf16(relu(z)) | 1 | 0...], z's fragments reused in place
-      float acc2[8][4];
+      uint32_t Z[4][4];
+      relu_frags(acc, Z);
+      float out[8][4];
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt) acc2[nt][0] = acc2[nt][1] = acc2[nt][2] = acc2[nt][3] = 0.f;
+      for (int nt = 0; nt < 8; ++nt) out[nt][0] = out[nt][1] = out[nt][2] = out[nt][3] = 0.f;
 #pragma unroll
       for (int kk = 0; kk < 5; ++kk) {
-        uint32_t a0, a1, a2, a3;
-        if (kk < 4) {
-          const float* lo = acc[2 * kk];
-          const float* hi = acc[2 * kk + 1];
-          a0 = pack2(__float2bfloat16_rn(fmaxf(lo[0], 0.f)), __float2bfloat16_rn(fmaxf(lo[1], 0.f)));
-          a1 = pack2(__float2bfloat16_rn(fmaxf(lo[2], 0.f)), __float2bfloat16_rn(fmaxf(lo[3], 0.f)));
-          a2 = pack2(__float2bfloat16_rn(fmaxf(hi[0], 0.f)), __float2bfloat16_rn(fmaxf(hi[1], 0.f)));
-          a3 = pack2(__float2bfloat16_rn(fmaxf(hi[2], 0.f)), __float2bfloat16_rn(fmaxf(hi[3], 0.f)));
-        } else {                              // columns 64..79: the bias column, then zeros
-          a0 = a1 = t == 0 ? pack2(__float2bfloat16_rn(1.0f), __float2bfloat16_rn(0.f)) : 0u;
-          a2 = a3 = 0u;
-        }
+        const uint32_t a0 = kk < 4 ? Z[kk & 3][0] : bias, a1 = kk < 4 ? Z[kk & 3][1] : bias;
+        const uint32_t a2 = kk < 4 ? Z[kk & 3][2] : 0u, a3 = kk < 4 ? Z[kk & 3][3] : 0u;
 #pragma unroll
         for (int nt = 0; nt < 8; nt += 2) {
           uint32_t b0, b1, c0, c1;
-          ldsm_b4(sW2, nt, kk * 16, lane, b0, b1, c0, c1);
-          mma16816(acc2[nt], a0, a1, a2, a3, b0, b1);
-          mma16816(acc2[nt + 1], a0, a1, a2, a3, c0, c1);
+          ldsm_b4(w1_base + 2 * 64 * 80 * 2, nt, kk * 16, b0, b1, c0, c1);
+          mma16816(out[nt], a0, a1, a2, a3, b0, b1);
+          mma16816(out[nt + 1], a0, a1, a2, a3, c0, c1);
         }
       }
+      // new states out; their rows of Tout through the buffer
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
         const int c = nt * 8 + 2 * t;
-        *reinterpret_cast<float2*>(&sM[g * kMsgLd + c]) = make_float2(acc2[nt][0], acc2[nt][1]);
-        *reinterpret_cast<float2*>(&sM[(g + 8) * kMsgLd + c]) = make_float2(acc2[nt][2], acc2[nt][3]);
+        const float2 ha = *reinterpret_cast<const float2*>(hg + c), hb = *reinterpret_cast<const float2*>(hh + c);
+        const float2 na = make_float2(ha.x + out[nt][0], ha.y + out[nt][1]);
+        const float2 nb = make_float2(hb.x + out[nt][2], hb.y + out[nt][3]);
+        if (vg) *reinterpret_cast<float2*>(&Hout[(ib + g) * F + c]) = na;
+        if (vh) *reinterpret_cast<float2*>(&Hout[(ib + g + 8) * F + c]) = nb;
+        buf[fuse_at(80, g, ocol + c)] = __float2bfloat16_rn(na.x);
+        buf[fuse_at(80, g, ocol + c + 1)] = __float2bfloat16_rn(na.y);
+        buf[fuse_at(80, g + 8, ocol + c)] = __float2bfloat16_rn(nb.x);
+        buf[fuse_at(80, g + 8, ocol + c + 1)] = __float2bfloat16_rn(nb.y);
+      }
+      // the 16 other columns: static features (zero), bias, padding
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int r = 2 * k + (lane >> 4), q = lane & 15, c = q < ocol ? q : F + q;
+        buf[fuse_at(80, r, c)] = __float2bfloat16_rn(c == ocol + F ? 1.0f : 0.f);
       }
       __syncwarp();
-      const int rows = (int)min(16u, e_end - t0);
-      for (int r = 0; r < rows; ++r) {
-        close_until(t0 + (uint32_t)r);
-        const float2 m = *reinterpret_cast<const float2*>(&sM[r * kMsgLd + 2 * lane]);
-        s0 += m.x;
-        s1 += m.y;
+      for (int idx = lane; idx < min(left, 16) * 10; idx += 32) {
+        const int r = idx / 10, c = (idx - r * 10) * 8;
+        *reinterpret_cast<uint4*>(&Tout[(ib + r) * 80 + c]) = *reinterpret_cast<const uint4*>(&buf[fuse_at(80, r, c)]);
       }
-      __syncwarp();                           // sM free for the next tile's staging
+      __syncwarp();
     }
-    close_until(e_end);
-    // node network of the run's nodes (the rows of one MMA tile), as the unfused node layers
-    // compute it: z = relu(W_n1 XN), h_out = h + W_n2 [z, 1]
-    __syncwarp();                             // the run's XN rows, written above, visible
-    const int nrows = (int)(i1 - i0);
-    const bool vg = g < nrows, vh = g + 8 < nrows;
-    const bf16* xn = XN + (i0 + g) * 144;
-    const bf16* xh = xn + 8 * 144;
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 9; ++kk) {
-      const uint32_t a0 = vg ? ld_u32(xn + kk * 16 + 2 * t) : 0u;
-      const uint32_t a1 = vh ? ld_u32(xh + kk * 16 + 2 * t) : 0u;
-      const uint32_t a2 = vg ? ld_u32(xn + kk * 16 + 2 * t + 8) : 0u;
-      const uint32_t a3 = vh ? ld_u32(xh + kk * 16 + 2 * t + 8) : 0u;
-#pragma unroll
-      for (int nt = 0; nt < 8; nt += 2) {
-        uint32_t b0, b1, c0, c1;
-        ldsm_b4<kNodeLd>(sN1, nt, kk * 16, lane, b0, b1, c0, c1);
-        mma16816(acc[nt], a0, a1, a2, a3, b0, b1);
-        mma16816(acc[nt + 1], a0, a1, a2, a3, c0, c1);
-      }
-    }
-    float acc2[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) acc2[nt][0] = acc2[nt][1] = acc2[nt][2] = acc2[nt][3] = 0.f;
-#pragma unroll
-    for (int kk = 0; kk < 5; ++kk) {
-      uint32_t a0, a1, a2, a3;
-      if (kk < 4) {
-        const float* lo = acc[2 * kk];
-        const float* hi = acc[2 * kk + 1];
-        a0 = pack2(__float2bfloat16_rn(fmaxf(lo[0], 0.f)), __float2bfloat16_rn(fmaxf(lo[1], 0.f)));
-        a1 = pack2(__float2bfloat16_rn(fmaxf(lo[2], 0.f)), __float2bfloat16_rn(fmaxf(lo[3], 0.f)));
-        a2 = pack2(__float2bfloat16_rn(fmaxf(hi[0], 0.f)), __float2bfloat16_rn(fmaxf(hi[1], 0.f)));
-        a3 = pack2(__float2bfloat16_rn(fmaxf(hi[2], 0.f)), __float2bfloat16_rn(fmaxf(hi[3], 0.f)));
-      } else {
-        a0 = a1 = t == 0 ? pack2(__float2bfloat16_rn(1.0f), __float2bfloat16_rn(0.f)) : 0u;
-        a2 = a3 = 0u;
-      }
-#pragma unroll
-      for (int nt = 0; nt < 8; nt += 2) {
-        uint32_t b0, b1, c0, c1;
-        ldsm_b4(sN2, nt, kk * 16, lane, b0, b1, c0, c1);
-        mma16816(acc2[nt], a0, a1, a2, a3, b0, b1);
-        mma16816(acc2[nt + 1], a0, a1, a2, a3, c0, c1);
-      }
-    }
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const int64_t o = (i0 + g) * F + nt * 8 + 2 * t;
-      if (vg) {
-        const float2 h = *reinterpret_cast<const float2*>(&H[o]);
-        *reinterpret_cast<float2*>(&Hout[o]) = make_float2(h.x + acc2[nt][0], h.y + acc2[nt][1]);
-      }
-      if (vh) {
-        const float2 h = *reinterpret_cast<const float2*>(&H[o + 8 * F]);
-        *reinterpret_cast<float2*>(&Hout[o + 8 * F]) = make_float2(h.x + acc2[nt][2], h.y + acc2[nt][3]);
-      }
-    }
-    __syncwarp();
   }
 }
 
 // ------------------------------------------------------------------ fused edge round, pipelined (tcgen05)
-// Round input row templates: T[j] is edge row [XS | bf16(h_j) | 1 | 0...] of any edge whose
-// neighbour is fluid node j, with zeros where the static features go; T[n] serves wall
-// neighbours (h = 0). An edge row is its neighbour's template with the static features
-// merged into the first one or two 16-byte pieces. The same launch writes the h part of
-// the round's node rows, XN[i][0, 64) = bf16(h_i). One thread per 16-byte piece.
+// Round input row templates: row j + 1 is edge row [XS | bf16(h_j) | 1 | 0...] of any edge
+// whose neighbour is fluid node j, with zeros where the static features go; row 0 serves
+// wall neighbours (h = 0). An edge row is its neighbour's template with the static features
+// merged into the first one or two 16-byte pieces. Threads past the templates (the pipelined
+// form launches them) write the h part of the round's node rows, XN[i][0, 64) = bf16(h_i).
+// One thread per 16-byte piece.
 template <int FE>
 __global__ void k_node_templates(int64_t n, const float* __restrict__ H, bf16* __restrict__ T,
                                  bf16* __restrict__ XN) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   __align__(16) bf16 v[8];
   if (idx < (n + 1) * 10) {
-    const int64_t j = idx / 10;
-    const int c0 = (int)(idx - j * 10) * 8;
+    const int64_t row = idx / 10, j = row - 1;
+    const int c0 = (int)(idx - row * 10) * 8;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int c = c0 + k;
       float x = 0.f;
-      if (c >= FE && c < FE + F) x = j < n ? H[j * F + (c - FE)] : 0.f;
+      if (c >= FE && c < FE + F) x = j >= 0 ? H[j * F + (c - FE)] : 0.f;
       else if (c == FE + F) x = 1.0f;
       v[k] = __float2bfloat16_rn(x);
     }
-    *reinterpret_cast<uint4*>(T + j * 80 + c0) = *reinterpret_cast<const uint4*>(v);
+    *reinterpret_cast<uint4*>(T + row * 80 + c0) = *reinterpret_cast<const uint4*>(v);
   } else if (idx < (n + 1) * 10 + n * 8) {
     const int64_t q = idx - (n + 1) * 10, i = q / 8;
     const int c0 = (int)(q - i * 8) * 8;
@@ -947,7 +1065,7 @@ k_edge_round_ws(int64_t n, int run, const uint32_t* __restrict__ off, const bf16
           const uint32_t e = e0 + (uint32_t)(lane + 32 * k);
           vr[k] = e < te;
           const int j = vr[k] ? __ldg(&enbr[e]) : 0;
-          jr[k] = j < 0 ? (int)n : j;                 // walls: the zero template
+          jr[k] = max(j, -1) + 1;                     // row 0: the walls' template
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
@@ -1380,6 +1498,7 @@ struct sph_learned {
   bf16* U = nullptr;
   bf16* XS = nullptr;                        // [E][16] static edge features
   bf16* T = nullptr;                         // [n + 1][80] round input row templates
+  bf16* T2 = nullptr;                        // ... of every second fused round
   int* erev = nullptr;                       // [E] reverse of each fluid edge, -1 for walls
   bf16* XE[ROUNDS] = {nullptr};
   bf16* A1[ROUNDS] = {nullptr};
@@ -1448,7 +1567,7 @@ int ensure_workspace(sph_learned* L, int64_t n, int64_t E) {
             nalloc(L, &L->Y, n * 16) && nalloc(L, &L->dH, n * F) && nalloc(L, &L->dXN, n * 144) &&
             nalloc(L, &L->dYb, n * 16) && nalloc(L, &L->dZn, n * F) && nalloc(L, &L->dM, E * F) &&
             nalloc(L, &L->dZe, std::max(E, n) * F) && nalloc(L, &L->dXE, E * 80) && nalloc(L, &L->loss, 1) &&
-            nalloc(L, &L->saveP, n) && nalloc(L, &L->saveV, n) && nalloc(L, &L->T, (n + 1) * 80);
+            nalloc(L, &L->saveP, n) && nalloc(L, &L->saveV, n) && nalloc(L, &L->T, (n + 1) * 80) && nalloc(L, &L->T2, (n + 1) * 80);
   for (int r = 0; r < ROUNDS && ok; ++r)
     ok = nalloc(L, &L->XE[r], E * 80) && nalloc(L, &L->A1[r], E * 80) && nalloc(L, &L->XN[r], n * 144) &&
          nalloc(L, &L->A2[r], n * 80);
@@ -1563,20 +1682,31 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
   if (train) cudaMemcpyAsync(L->H0, L->H, sizeof(float) * n * F, cudaMemcpyDeviceToDevice, s);
   for (int r = 0; r < ROUNDS; ++r) {
     if (fused) {
-      const int64_t chunks = (n + kFuseNodes - 1) / kFuseNodes;
-      int per_sm = 1, sms = 1, dev = 0;
+      if (n == 0) continue;
+      int sms = 1, dev = 0;
       cudaGetDevice(&dev);
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      auto kern = d == 2 ? k_edge_round_fused<7> : k_edge_round_fused<9>;
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kFuseWarps * 32, fused_smem());
-      const unsigned grid = (unsigned)std::min<int64_t>((chunks + kFuseWarps - 1) / kFuseWarps,
-                                                        (int64_t)std::max(per_sm, 1) * sms);
-      // node states ping-pong between H and H0 (H0 is only kept for training's backward)
-      float* hin = (r & 1) ? L->H0 : L->H;
+      // runs of equal node counts, a whole number of them per warp where possible; short runs
+      // where the warps would outnumber them, down to a half tile of edges
+      const int64_t slots = (int64_t)sms * kFuseWarps;
+      const int64_t per = (n + slots * kFuseRun - 1) / (slots * kFuseRun);
+      const int run = (int)std::max<int64_t>(kFuseRunMin, (n + slots * per - 1) / (slots * per));
+      const unsigned grid = (unsigned)std::min<int64_t>((n + run - 1) / run, sms);
+      // node states ping-pong between H and H0 (H0 is only kept for training's backward), the
+      // templates between T and T2; the last round leaves the decoder's input rows instead
+      const float* hin = (r & 1) ? L->H0 : L->H;
       float* hout = (r & 1) ? L->H : L->H0;
-      if (n > 0)
-        kern<<<grid, kFuseWarps * 32, fused_smem(), s>>>(n, L->off, L->XS, L->enbr, hin, Wl(L, L_E1), Wl(L, L_E2),
-                                                         Wl(L, L_N1), Wl(L, L_N2), inv_nbar, L->XN[r], hout);
+      const bf16* tin = (r & 1) ? L->T2 : L->T;
+      const bool last = r == ROUNDS - 1;
+      bf16* tout = last ? L->XD : ((r & 1) ? L->T : L->T2) + 80;
+      if (r == 0) {
+        auto tmpl = d == 2 ? k_node_templates<7> : k_node_templates<9>;
+        tmpl<<<blocks_for((n + 1) * 10), 256, 0, s>>>(n, hin, L->T, L->XN[r]);
+      }
+      auto kern = d == 2 ? k_edge_round_fused<7> : k_edge_round_fused<9>;
+      kern<<<grid, kFuseWarps * 32, fused_smem(), s>>>(n, run, L->off, L->XS, L->enbr, hin, tin, Wl(L, L_E1),
+                                                       Wl(L, L_E2), Wl(L, L_N1), Wl(L, L_N2), inv_nbar, L->XN[r], hout,
+                                                       tout, last ? 0 : fe);
     } else if (piped) {
       auto tmpl = d == 2 ? k_node_templates<7> : k_node_templates<9>;
       tmpl<<<blocks_for((n + 1) * 10 + n * 8), 256, 0, s>>>(n, L->H, L->T, L->XN[r]);
@@ -1605,9 +1735,8 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
       dense<64>(n, 80, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
     }
   }
-  // the fused rounds leave the final node states in H0 after an odd number of rounds
-  const float* hfin = (fused && (ROUNDS & 1)) ? L->H0 : L->H;
-  k_rows_bf16<<<blocks_for(n * F), 256, 0, s>>>(n, F, hfin, F, L->XD, 80);
+  // the fused rounds leave the decoder's input rows
+  if (!fused) k_rows_bf16<<<blocks_for(n * F), 256, 0, s>>>(n, F, L->H, F, L->XD, 80);
   dense<64>(n, 80, L->XD, 80, Wl(L, L_D1), nullptr, 0, 0, 0, L->A3, 80, 0, F, 1, nullptr, 0, L->tc_err, s);
   dense<16>(n, 80, L->A3, 80, Wl(L, L_D2), L->Y, 16, 16, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
 }

@@ -189,3 +189,24 @@ def test_one_launch_diffusion_equals_the_stage_launches(sph, case):
     assert not np.array_equal(out[0], C0.astype(np.float32))
     sph.sph_species_destroy(sp)
     sim.close()
+
+
+@pytest.mark.parametrize("nx, ny", [(3, 1), (4, 33), (130, 75), (131, 75), (220, 190), (480, 330)])
+def test_fused_edge_rounds_at_run_boundaries(sph, nx, ny):
+    # node runs of the shortest length (and one node past it), of a whole tile of nodes and
+    # two more, and several runs a warp; tiles of edges with every remainder: the same bits as
+    # the layers one by one
+    prob = _block(nx, ny)
+    sim = sph.Simulation(prob)
+    sim.build_cells()
+    sim.advection_step()
+    W = mpnn.init_weights(2, seed=6)
+    net = sph.sph_learned_create(2, np.concatenate([W[k].ravel() for k in ("enc", "e1", "e2", "n1", "n2", "d1", "d2")]))
+    y = []
+    for form in (1, 0):
+        sph.sph_learned_set_fused(net, form)
+        y.append(sph.sph_learned_predict(sim.handle, net, prob.n_fluid, 2))
+    assert np.all(np.isfinite(y[0])) and np.abs(y[0]).max() > 0
+    np.testing.assert_array_equal(y[0], y[1])
+    sph.sph_learned_destroy(net)
+    sim.close()
