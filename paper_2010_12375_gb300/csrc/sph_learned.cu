@@ -80,24 +80,29 @@ __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uin
 // warpgroup of 128 threads) keeps W [NO x K] in shared memory in the core-matrix layout and
 // walks 128-row tiles (grid-stride): the tile's rows are copied into the A operand, one
 // thread issues the K/16 MMAs into TMEM, and each warp then reads its 32 rows' accumulators
-// (TMEM lane = row) 16 columns at a time for the epilogue. Epilogue per element
-// (m, n < NO): y = acc; y = 0 where mask[m, n] <= 0 (ReLU backward) if mask;
-// y = max(y, 0) if relu; out_f32[m, n] = y (or += y with accum) for n < nf_store;
-// out_b[m, col0 + n] = bf16(y) for n < nb_store. Copies are shaped for the memory system:
-// a quarter-warp moves one core matrix (8 rows x 16 bytes: one 128-byte shared-memory
-// wavefront, two full global sectors per row pair of pieces), and each warp stages its
-// 32 x 16 block of results in shared memory (in the tile the tensor core has just read, so
-// the staging costs no shared memory of its own) to store them as 64-byte row segments.
-// K is a multiple of 16, ldx, ldo, col0 and nb_store multiples of 8, ldf and nf_store of 4,
-// ldm of 2 (checked by the host wrapper). A wait for the tensor core that runs out sets
+// (TMEM lane = row) 32 columns at a time for the epilogue. Epilogue per element
+// (m, n < NO): y = acc, y = max(y, 0) if relu; out_f32[m, n] = y (or += y with accum)
+// for n < nf_store; out_b[m, col0 + n] = bf16(y) for n < nb_store <= 64, 0 where
+// mask[m, n] <= 0 with MASK (ReLU backward; read ahead of the results). Copies are shaped
+// for the memory system: a quarter-warp moves one core matrix (8 rows x 16 bytes: one
+// 128-byte shared-memory wavefront, two full global sectors per row pair of pieces), and each
+// warp stages 128 bytes of its 32 rows in shared memory (in the tile the tensor core has just
+// read, so the staging costs no shared memory of its own) to store them as whole lines.
+// A CTA mostly has one tile, so the chain of latencies counts: W comes with the first tile,
+// the mask is read in whole lines during the MMAs, and the epilogue has one staging round per
+// 128 bytes of a row. With W loaded first, 16 columns a round in 4-byte shared accesses and the
+// mask read row by row, the 28 layers of a training step of 3,200 particles (86,000 edges) took
+// 380 us and take 290. One tile buffer and more CTAs an SM instead of two buffers was no faster.
+// K is a multiple of 16, ldx, ldo, col0, nb_store and ldm multiples of 8, ldf and nf_store of 4
+// (checked by the host wrapper). A wait for the tensor core that runs out sets
 // ERR_TIMEOUT in *err and the CTA stops.
-constexpr int kDenseStageLd = 17;           // staged row stride (floats): conflict-free columns
+constexpr int kDenseStageLd = 144;          // staged row stride (bytes): 128 and a piece of padding
 
 // shared memory of k_dense: W, then two row tiles of 128 x K, each large enough to serve as
 // the four warps' staging blocks once the tensor core has read it
 __host__ __device__ constexpr int dense_w_bytes(int NO, int K) { return (NO * K * 2 + 127) / 128 * 128; }
 __host__ __device__ constexpr int dense_tile_bytes(int K) {
-  return ((128 * K * 2 > 4 * 32 * kDenseStageLd * 4 ? 128 * K * 2 : 4 * 32 * kDenseStageLd * 4) + 127) / 128 * 128;
+  return ((128 * K * 2 > 128 * kDenseStageLd ? 128 * K * 2 : 128 * kDenseStageLd) + 127) / 128 * 128;
 }
 
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, bool valid) {
@@ -133,9 +138,14 @@ __device__ __forceinline__ void load_operand(unsigned char* dst, int R, int K, c
   }
 }
 
-template <int NO>
+// all ones in the halves of a pair of bf16 that are > 0
+__device__ __forceinline__ uint32_t positive2(uint32_t m) {
+  return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&m), __floats2bfloat162_rn(0.f, 0.f));
+}
+
+template <int NO, int K, bool MASK>
 __global__ void __launch_bounds__(128)
-k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __restrict__ W,
+k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__ W,
         float* __restrict__ out_f32, int ldf, int nf_store, int accum, bf16* __restrict__ out_b, int ldo,
         int col0, int nb_store, int relu, const bf16* __restrict__ mask, int ldm, int* __restrict__ err) {
   constexpr int COLS = tc::tmem_cols(NO);
@@ -143,10 +153,15 @@ k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __res
   __shared__ __align__(8) uint64_t bar;
   __shared__ uint32_t tmem_slot;
   unsigned char* sB = tc_smem;                        // NO x K
-  const int tile_bytes = dense_tile_bytes(K);
+  constexpr int tile_bytes = dense_tile_bytes(K);
   unsigned char* sA0 = tc_smem + dense_w_bytes(NO, K);   // two 128 x K row tiles
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  load_operand<false>(sB, NO, K, W, K, NO);
+  if ((int64_t)blockIdx.x * 128 < M) {                // the first tile and W stream in
+    const int64_t m0 = (int64_t)blockIdx.x * 128;
+    load_operand<true>(sA0, 128, K, X + m0 * ldx, ldx, M - m0);
+    load_operand<true>(sB, NO, K, W, K, NO);
+  }
+  cp_async_commit();
   if (threadIdx.x == 0) tc::mbar_init(&bar);
   if (warp == 0) tc::tmem_alloc(&tmem_slot, COLS);
   tc::fence_before_sync();
@@ -156,13 +171,7 @@ k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __res
   const uint32_t b_addr = tc::smem_u32(sB);
   const int64_t tiles = (M + 127) / 128;
   uint32_t phase = 0;
-  if (blockIdx.x < tiles) {                           // the first tile streams in
-    const int64_t m0 = (int64_t)blockIdx.x * 128;
-    load_operand<true>(sA0, 128, K, X + m0 * ldx, ldx, M - m0);
-  }
-  cp_async_commit();
   int buf = 0;
-  float* st = nullptr;                                // this warp's staging block, in the tile just multiplied
   for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x, buf ^= 1) {
     const int64_t m0 = tile * 128;
     unsigned char* sA = sA0 + buf * tile_bytes;
@@ -177,6 +186,16 @@ k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __res
       tc::fence_after_sync();
       tc::mma_tile<NO>(tmem, tc::smem_u32(sA), b_addr, K, false, &bar);
     }
+    const int64_t mw = m0 + warp * 32;                // this warp's first row
+    // the mask of this lane's bf16 pieces (below), in flight during the MMAs
+    uint4 mk[MASK ? 8 : 1];
+    if (MASK)
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int64_t m = mw + 4 * q + (lane >> 3);
+        mk[q] = make_uint4(0u, 0u, 0u, 0u);
+        if (m < M && (lane & 7) * 8 < nb_store) mk[q] = *reinterpret_cast<const uint4*>(&mask[m * ldm + (lane & 7) * 8]);
+      }
     const bool done = tc::mbar_wait(&bar, phase);
     phase ^= 1u;
     if (!__syncthreads_and(done)) {                   // the same decision in every thread
@@ -184,32 +203,35 @@ k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __res
       break;
     }
     tc::fence_after_sync();
-    st = reinterpret_cast<float*>(sA) + warp * 32 * kDenseStageLd;   // the tensor core is done with the tile
-    const int64_t mw = m0 + warp * 32;                // this warp's first row
-    const int64_t my = mw + lane;                     // the row whose accumulators this lane reads
-#pragma unroll 1
-    for (int c0 = 0; c0 < NO; c0 += 16) {
-      float y[16];
-      tc::tmem_ld16(tc::tmem_addr(tmem, warp, c0), y);
-      if (mask && my < M) {
+    // this warp's staging block, in the tile the tensor core is done with: 32 rows of 128
+    // bytes, padded so that rows of 16-byte pieces go in and lines come out without conflicts
+    unsigned char* st = sA + warp * 32 * kDenseStageLd;
+    unsigned char* mine = st + lane * kDenseStageLd;  // the row whose accumulators this lane reads
+    if (out_f32) {
 #pragma unroll
-        for (int q = 0; q < 16; q += 2) {
-          const uint32_t mk = ld_u32(&mask[my * ldm + c0 + q]);
-          if (!(__bfloat162float(__ushort_as_bfloat16((unsigned short)(mk & 0xffffu))) > 0.f)) y[q] = 0.f;
-          if (!(__bfloat162float(__ushort_as_bfloat16((unsigned short)(mk >> 16))) > 0.f)) y[q + 1] = 0.f;
+      for (int c0 = 0; c0 < NO; c0 += 32) {           // 32 (or the last 16) columns at a time
+        constexpr int kW = NO % 32;
+        const int w = NO - c0 < 32 ? kW : 32;
+        if (c0 >= nf_store) break;
+        float y[32];
+        tc::tmem_ld16_async(tc::tmem_addr(tmem, warp, c0), y);
+        if (w == 32) tc::tmem_ld16_async(tc::tmem_addr(tmem, warp, c0 + 16), y + 16);
+        tc::tmem_wait(y);
+        if (w == 32) tc::tmem_wait(y + 16);
+#pragma unroll
+        for (int q = 0; q < w; q += 4) {
+          float4 v = make_float4(y[q], y[q + 1], y[q + 2], y[q + 3]);
+          if (relu) v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+          *reinterpret_cast<float4*>(mine + q * 4) = v;
         }
-      }
+        __syncwarp();
+        const int pieces = w / 4;                     // 16-byte pieces of a row
 #pragma unroll
-      for (int q = 0; q < 16; ++q) st[lane * kDenseStageLd + q] = relu ? fmaxf(y[q], 0.f) : y[q];
-      __syncwarp();
-      if (out_f32 && c0 < nf_store) {                 // 8 rows x 4 float4 pieces per pass
-#pragma unroll
-        for (int pass = 0; pass < 4; ++pass) {
-          const int r = pass * 8 + (lane >> 2), c = (lane & 3) * 4;
+        for (int q = 0; q < pieces; ++q) {
+          const int r = (q * 32 + lane) / pieces, c = (q * 32 + lane) % pieces * 4;
           const int64_t m = mw + r;
           if (m < M && c0 + c < nf_store) {
-            const float* v = st + r * kDenseStageLd + c;
-            float4 o = make_float4(v[0], v[1], v[2], v[3]);
+            float4 o = *reinterpret_cast<const float4*>(st + r * kDenseStageLd + c * 4);
             float4* dst = reinterpret_cast<float4*>(&out_f32[m * ldf + c0 + c]);
             if (accum) {
               const float4 p = *dst;
@@ -218,24 +240,46 @@ k_dense(int64_t M, int K, const bf16* __restrict__ X, int ldx, const bf16* __res
             *dst = o;
           }
         }
+        __syncwarp();                                 // the staging block is reused next
       }
-      if (out_b && c0 < nb_store) {                   // 16 rows x 2 pieces of 8 bf16 per pass
+    }
+    if (out_b) {                                      // at most 64 columns
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-          const int r = pass * 16 + (lane >> 1), c = (lane & 1) * 8;
-          const int64_t m = mw + r;
-          if (m < M && c0 + c < nb_store) {
-            const float* v = st + r * kDenseStageLd + c;
-            uint4 o;
-            o.x = pack2(__float2bfloat16_rn(v[0]), __float2bfloat16_rn(v[1]));
-            o.y = pack2(__float2bfloat16_rn(v[2]), __float2bfloat16_rn(v[3]));
-            o.z = pack2(__float2bfloat16_rn(v[4]), __float2bfloat16_rn(v[5]));
-            o.w = pack2(__float2bfloat16_rn(v[6]), __float2bfloat16_rn(v[7]));
-            *reinterpret_cast<uint4*>(&out_b[m * ldo + col0 + c0 + c]) = o;
+      for (int c0 = 0; c0 < (NO < 64 ? NO : 64); c0 += 32) {
+        const int w = NO - c0 < 32 ? NO % 32 : 32;
+        float y[32];
+        tc::tmem_ld16_async(tc::tmem_addr(tmem, warp, c0), y);
+        if (w == 32) tc::tmem_ld16_async(tc::tmem_addr(tmem, warp, c0 + 16), y + 16);
+        tc::tmem_wait(y);
+        if (w == 32) tc::tmem_wait(y + 16);
+#pragma unroll
+        for (int q = 0; q < w; q += 8) {
+          uint4 o;
+          uint32_t* u = reinterpret_cast<uint32_t*>(&o);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const float lo = y[q + 2 * k], hi = y[q + 2 * k + 1];
+            const __nv_bfloat162 v = relu ? __floats2bfloat162_rn(fmaxf(lo, 0.f), fmaxf(hi, 0.f)) : __floats2bfloat162_rn(lo, hi);
+            u[k] = *reinterpret_cast<const uint32_t*>(&v);
           }
+          *reinterpret_cast<uint4*>(mine + (c0 + q) * 2) = o;
         }
       }
-      __syncwarp();                                   // the staging block is reused next
+      __syncwarp();
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int r = 4 * q + (lane >> 3), c = (lane & 7) * 8;
+        const int64_t m = mw + r;
+        if (m < M && c < nb_store) {
+          uint4 o = *reinterpret_cast<const uint4*>(st + r * kDenseStageLd + c * 2);
+          if (MASK) {
+            const uint4 k = mk[MASK ? q : 0];
+            o = make_uint4(o.x & positive2(k.x), o.y & positive2(k.y), o.z & positive2(k.z), o.w & positive2(k.w));
+          }
+          *reinterpret_cast<uint4*>(&out_b[m * ldo + col0 + c]) = o;
+        }
+      }
+      __syncwarp();
     }
     tc::fence_before_sync();
     __syncthreads();                                  // TMEM read and the A tile free before the next
@@ -338,22 +382,37 @@ k_dense_dw(int64_t M, int64_t rows, const bf16* __restrict__ dY, int ldy, const 
   }
 }
 
-// grad[o] += sum over blocks of partial[block][o], in a fixed order: eight warps take every
-// eighth block of 32 consecutive outputs, then their sums are added in warp order. count is a
-// multiple of 32.
+// grad[dst + o] += sum over blocks of partial[src + block count + o] for the weight gradients
+// of several layers in one launch, each in a fixed order: eight warps take every eighth block
+// of 32 consecutive outputs, then their sums are added in warp order. Counts are multiples of 32.
+// A launch of its own for each layer left most of the chip idle (160 blocks) fifteen times a
+// training step; the layers of a round share one.
+struct DwSum {
+  int blocks, count, dst;
+  size_t src;
+};
+constexpr int kDwSums = 6;                // layers in one launch, at most
+struct DwSums {
+  DwSum job[kDwSums];
+};
 __global__ void __launch_bounds__(256)
-k_reduce_partials(int blocks, int count, const float* __restrict__ partial, float* __restrict__ grad) {
+k_reduce_partials(DwSums S, int jobs, const float* __restrict__ partial, float* __restrict__ grad) {
   __shared__ float red[8][32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, o = blockIdx.x * 32 + lane;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int at = blockIdx.x * 32, q = 0;
+  while (q + 1 < jobs && at >= S.job[q].count) at -= S.job[q++].count;
+  const DwSum j = S.job[q];
+  const int o = at + lane;
+  const float* p = partial + j.src;
   float s = 0.f;
-#pragma unroll 4
-  for (int b = warp; b < blocks; b += 8) s += partial[(size_t)b * count + o];
+#pragma unroll 8
+  for (int b = warp; b < j.blocks; b += 8) s += p[(size_t)b * j.count + o];
   red[warp][lane] = s;
   __syncthreads();
   if (warp == 0) {
 #pragma unroll
     for (int w = 1; w < 8; ++w) s += red[w][lane];
-    grad[o] += s;
+    grad[j.dst + o] += s;
   }
 }
 
@@ -365,13 +424,11 @@ __global__ void k_edge_count(int64_t n, const uint32_t* __restrict__ nbc, uint32
   if (i < n) cnt[i] = (nbc[i] & 0xffffu) + (nbc[i] >> 16);
 }
 
-// Node features (one 32-byte row per particle) and the edge list of the frozen table.
+// Node features (one 32-byte row per particle).
 template <int D>
 __global__ void k_node_features(int64_t n, const int4* __restrict__ P, const float4* __restrict__ V,
                                 const int* __restrict__ inst_of, const Inst* __restrict__ inst,
-                                const Ctrl* __restrict__ ctrl, const int* __restrict__ nbr,
-                                const uint32_t* __restrict__ nbc, const uint32_t* __restrict__ off,
-                                int* __restrict__ esrc, int* __restrict__ enbr, bf16* __restrict__ U) {
+                                const Ctrl* __restrict__ ctrl, bf16* __restrict__ U) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int k = inst_of ? inst_of[i] : 0;
@@ -389,54 +446,65 @@ __global__ void k_node_features(int64_t n, const int4* __restrict__ P, const flo
   uint4* dst = reinterpret_cast<uint4*>(U + i * 16);
   dst[0] = reinterpret_cast<const uint4*>(u)[0];
   dst[1] = reinterpret_cast<const uint4*>(u)[1];
-  const uint32_t cnt = nbc[i];
-  const int nf = (int)(cnt & 0xffffu), nw = (int)(cnt >> 16);
-  uint32_t e = off[i];
-  for (int s = 0; s < nf + nw; ++s, ++e) {
+}
+
+// The edge list of the frozen table and each edge's static features, 16 bf16 per edge:
+// [r_ij/h, (v_i - v_j)/c0, 100 dev_i, 100 dev_j, is_wall, 0...]; the rounds' input rows are
+// assembled from them by k_edge_rows. A warp takes kEdgeNodes consecutive nodes, whose edges
+// are consecutive, and its lanes take 32 of them at a time: the lists and rows are written
+// in whole lines (a thread per node that walked its edges, and a second pass over the edges
+// for the features, took 25 + 20 us for 2.7 M edges where this takes 27 us).
+constexpr int kEdgeNodes = 4;
+template <int D>
+__global__ void k_edge_features(int64_t n, const int4* __restrict__ P, const float4* __restrict__ V,
+                                const int* __restrict__ inst_of, const Inst* __restrict__ inst,
+                                const int* __restrict__ nbr, const uint32_t* __restrict__ nbc,
+                                const uint32_t* __restrict__ off, const int4* __restrict__ WP, int* __restrict__ esrc,
+                                int* __restrict__ enbr, bf16* __restrict__ XS) {
+  const int64_t i0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kEdgeNodes;
+  if (i0 >= n) return;
+  uint32_t o[kEdgeNodes + 1];
+#pragma unroll
+  for (int k = 0; k <= kEdgeNodes; ++k) o[k] = off[min(i0 + k, n)];
+  for (uint32_t e = o[0] + (threadIdx.x & 31); e < o[kEdgeNodes]; e += 32) {
+    int k = 0;                                          // the last node whose edges begin at or before e
+#pragma unroll
+    for (int q = 1; q < kEdgeNodes; ++q) k += o[q] <= e;
+    uint32_t first = o[0];
+#pragma unroll
+    for (int q = 1; q < kEdgeNodes; ++q) first = k == q ? o[q] : first;
+    const int64_t i = i0 + k;
+    const int s = (int)(e - first), nf = (int)(nbc[i] & 0xffffu);
     const bool wall = s >= nf;
     const int j = nbr[slot_index(n, i, wall ? wall_slot0(nf) + (s - nf) : s)];
     esrc[e] = (int)i;
     enbr[e] = wall ? -1 - j : j;
+    const Inst& I = inst[inst_of ? inst_of[i] : 0];
+    const int4 pi = P[i];
+    const float4 vi = V[i];
+    const int4 pj = wall ? WP[j] : P[j];
+    float4 vj = make_float4(0.f, 0.f, 0.f, 0.f);
+    float dev_j = 0.f;
+    if (!wall) {
+      vj = V[j];
+      dev_j = i2f(pj.w) / I.rho0;
+    }
+    const float inv_c0 = 1.0f / I.c0;
+    const int qi[3] = {pi.x, pi.y, pi.z}, qj[3] = {pj.x, pj.y, pj.z};
+    const float ui[3] = {vi.x, vi.y, vi.z}, uj[3] = {vj.x, vj.y, vj.z};
+    __align__(16) bf16 row[16];
+    for (int c = 0; c < 16; ++c) row[c] = __float2bfloat16_rn(0.f);
+    for (int a = 0; a < D; ++a) {
+      row[a] = __float2bfloat16_rn((float)wrap_diff(qi[a] - qj[a], I.period[a]) * I.dq * I.inv_h);
+      row[D + a] = __float2bfloat16_rn((ui[a] - uj[a]) * inv_c0);
+    }
+    row[2 * D] = __float2bfloat16_rn(S_RHO * (i2f(pi.w) / I.rho0));
+    row[2 * D + 1] = __float2bfloat16_rn(S_RHO * dev_j);
+    row[2 * D + 2] = __float2bfloat16_rn(wall ? 1.0f : 0.0f);
+    uint4* dst = reinterpret_cast<uint4*>(XS + e * 16);
+    dst[0] = reinterpret_cast<const uint4*>(row)[0];
+    dst[1] = reinterpret_cast<const uint4*>(row)[1];
   }
-}
-
-// Static features of edge e, 16 bf16 per edge: [r_ij/h, (v_i - v_j)/c0, 100 dev_i,
-// 100 dev_j, is_wall, 0...]; the rounds' input rows are assembled from them by k_edge_rows.
-template <int D>
-__global__ void k_edge_features(int64_t E, const int4* __restrict__ P, const float4* __restrict__ V,
-                                const int* __restrict__ inst_of, const Inst* __restrict__ inst,
-                                const int* __restrict__ esrc, const int* __restrict__ enbr,
-                                const int4* __restrict__ WP, bf16* __restrict__ XS) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= E) return;
-  const int i = esrc[e], jj = enbr[e];
-  const bool wall = jj < 0;
-  const int j = wall ? -1 - jj : jj;
-  const Inst& I = inst[inst_of ? inst_of[i] : 0];
-  const int4 pi = P[i];
-  const float4 vi = V[i];
-  const int4 pj = wall ? WP[j] : P[j];
-  float4 vj = make_float4(0.f, 0.f, 0.f, 0.f);
-  float dev_j = 0.f;
-  if (!wall) {
-    vj = V[j];
-    dev_j = i2f(pj.w) / I.rho0;
-  }
-  const float inv_c0 = 1.0f / I.c0;
-  const int qi[3] = {pi.x, pi.y, pi.z}, qj[3] = {pj.x, pj.y, pj.z};
-  const float ui[3] = {vi.x, vi.y, vi.z}, uj[3] = {vj.x, vj.y, vj.z};
-  __align__(16) bf16 row[16];
-  for (int c = 0; c < 16; ++c) row[c] = __float2bfloat16_rn(0.f);
-  for (int a = 0; a < D; ++a) {
-    row[a] = __float2bfloat16_rn((float)wrap_diff(qi[a] - qj[a], I.period[a]) * I.dq * I.inv_h);
-    row[D + a] = __float2bfloat16_rn((ui[a] - uj[a]) * inv_c0);
-  }
-  row[2 * D] = __float2bfloat16_rn(S_RHO * (i2f(pi.w) / I.rho0));
-  row[2 * D + 1] = __float2bfloat16_rn(S_RHO * dev_j);
-  row[2 * D + 2] = __float2bfloat16_rn(wall ? 1.0f : 0.0f);
-  uint4* dst = reinterpret_cast<uint4*>(XS + e * 16);
-  dst[0] = reinterpret_cast<const uint4*>(row)[0];
-  dst[1] = reinterpret_cast<const uint4*>(row)[1];
 }
 
 // Round input row of edge e: XE[e] = [static features (fe) | bf16(h_j) (64, zero for a
@@ -470,7 +538,14 @@ __global__ void k_segsum(int64_t n, const uint32_t* __restrict__ off, const floa
   const int64_t i = idx / F;
   const int f = (int)(idx % F);
   float s = 0.f;
-  for (uint32_t e = off[i]; e < off[i + 1]; ++e) s += Mm[(int64_t)e * F + f];
+  const uint32_t end = off[i + 1];
+  for (uint32_t e = off[i]; e < end; e += 8) {        // eight rows in flight; +0 changes no sum
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = e + k < end ? Mm[(int64_t)(e + k) * F + f] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s += v[k];
+  }
   XN[i * 144 + f] = __float2bfloat16_rn(H[i * F + f]);
   XN[i * 144 + F + f] = __float2bfloat16_rn(s * inv_nbar);
 }
@@ -1325,22 +1400,21 @@ __global__ void k_loss(int64_t n, int dout, const float* __restrict__ Y, const d
   if ((threadIdx.x & 31) == 0) atomicAdd(loss, l / ((double)n * dout));
 }
 
-// dh += dXN[:, :F]; dM[e] = bf16(dXN[src(e), F + f] / nbar)
-__global__ void k_node_back(int64_t n, const float* __restrict__ dXN, float* __restrict__ dH) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * F) return;
-  const int64_t i = idx / F;
-  const int f = (int)(idx % F);
-  dH[i * F + f] += dXN[i * 144 + f];
-}
-
+// dM[e] = bf16(dXN[src(e), F + f] / nbar), 8 columns a thread
 __global__ void k_edge_back(int64_t E, const int* __restrict__ esrc, const float* __restrict__ dXN, float inv_nbar,
                             bf16* __restrict__ dM) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= E * F) return;
-  const int64_t e = idx / F;
-  const int f = (int)(idx % F);
-  dM[e * F + f] = __float2bfloat16_rn(dXN[(int64_t)esrc[e] * 144 + F + f] * inv_nbar);
+  if (idx >= E * (F / 8)) return;
+  const int64_t e = idx / (F / 8);
+  const int f = (int)(idx % (F / 8)) * 8;
+  const float4* x = reinterpret_cast<const float4*>(&dXN[(int64_t)esrc[e] * 144 + F + f]);
+  const float4 a = x[0], b = x[1];
+  uint4 o;
+  o.x = pack2(__float2bfloat16_rn(a.x * inv_nbar), __float2bfloat16_rn(a.y * inv_nbar));
+  o.y = pack2(__float2bfloat16_rn(a.z * inv_nbar), __float2bfloat16_rn(a.w * inv_nbar));
+  o.z = pack2(__float2bfloat16_rn(b.x * inv_nbar), __float2bfloat16_rn(b.y * inv_nbar));
+  o.w = pack2(__float2bfloat16_rn(b.z * inv_nbar), __float2bfloat16_rn(b.w * inv_nbar));
+  *reinterpret_cast<uint4*>(&dM[e * F + f]) = o;
 }
 
 // Reverse of each fluid edge: erev[e] for e = (i -> j) is the edge (j -> i) (the frozen
@@ -1360,28 +1434,50 @@ __global__ void k_reverse_edges(int64_t E, const int* __restrict__ esrc, const i
   erev[e] = r;
 }
 
-// Transpose of the gather h_j -> x_ij: dh[j] += sum over edges (i -> j) of dXE[e, fe + f],
-// taken over j's own fluid edges (j -> i) through their reverses, in edge order.
+// Node-state gradient of a round: dh[j] = (dh[j] + dXN[j, :F]) + sum over edges (i -> j) of
+// dXE[e, fe + f], the transpose of the gather h_j -> x_ij, taken over j's own fluid edges
+// (j -> i) through their reverses, in edge order. dZ = bf16(dh), the next round's operand, or
+// with H0 (the encoder's ReLU) bf16(dh) where h0 > 0 and 0 elsewhere. A warp per node: the
+// reverses of 32 edges come in one load, and eight edges' rows are in flight at a time (a
+// thread per element that followed enbr, erev and the row edge by edge took twice the time).
 __global__ void k_gather_dh(int64_t n, int fe, const uint32_t* __restrict__ off, const int* __restrict__ enbr,
-                            const int* __restrict__ erev, const float* __restrict__ dXE, float* __restrict__ dH) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * F) return;
-  const int64_t j = idx / F;
-  const int f = (int)(idx % F);
-  float acc = 0.f;
-  for (uint32_t e2 = off[j]; e2 < off[j + 1] && enbr[e2] >= 0; ++e2) {
-    const int r = erev[e2];
-    if (r >= 0) acc += dXE[(int64_t)r * 80 + fe + f];
-  }
-  dH[j * F + f] += acc;
-}
-
-// dZ0 = bf16(dh * (h0 > 0))
-__global__ void k_relu_back(int64_t n, const float* __restrict__ dH, const float* __restrict__ H0,
+                            const int* __restrict__ erev, const float* __restrict__ dXE,
+                            const float* __restrict__ dXN, const float* __restrict__ H0, float* __restrict__ dH,
                             bf16* __restrict__ dZ) {
-  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n * F) return;
-  dZ[idx] = __float2bfloat16_rn(H0[idx] > 0.f ? dH[idx] : 0.f);
+  const int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int lane = threadIdx.x & 31;
+  if (j >= n) return;
+  const uint32_t end = off[j + 1];
+  float a0 = 0.f, a1 = 0.f;
+  for (uint32_t e0 = off[j]; e0 < end; e0 += 32) {
+    const uint32_t e = e0 + lane;
+    const bool fluid = e < end && enbr[e] >= 0;       // fluid edges come first
+    const int rev = fluid ? erev[e] : -1;
+    const int cnt = __popc(__ballot_sync(0xffffffffu, fluid));
+    for (int k0 = 0; k0 < cnt; k0 += 8) {
+      float v0[8], v1[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int r = __shfl_sync(0xffffffffu, rev, (k0 + k) & 31);
+        const bool use = k0 + k < cnt && r >= 0;
+        const float* x = dXE + (int64_t)(use ? r : 0) * 80 + fe + lane;
+        v0[k] = use ? x[0] : 0.f;
+        v1[k] = use ? x[32] : 0.f;
+      }
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {                   // +0 leaves a sum that started at +0 unchanged
+        a0 += v0[k];
+        a1 += v1[k];
+      }
+    }
+  }
+#pragma unroll
+  for (int half = 0; half < 2; ++half) {
+    const int64_t o = j * F + 32 * half + lane;
+    const float h = dH[o] + dXN[j * 144 + 32 * half + lane] + (half ? a1 : a0);
+    dH[o] = h;
+    dZ[o] = __float2bfloat16_rn(!H0 || H0[o] > 0.f ? h : 0.f);
+  }
 }
 
 // Adam (beta1 0.9, beta2 0.999, eps 1e-8); b1pow = beta1^t, b2pow = beta2^t
@@ -1461,10 +1557,9 @@ size_t dense_smem(int K) {
 template <int NO, int K>
 constexpr int dw_smem() { return 2 * kTile * ((NO + 8) + (K + 8)) * (int)sizeof(bf16); }
 
-template <int NO>
+template <int NO, int K, bool MASK = false>
 void set_smem_attrs() {
-  cudaFuncSetAttribute(k_dense<NO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)std::max(dense_smem<NO>(144), dense_smem<NO>(16)));
+  cudaFuncSetAttribute(k_dense<NO, K, MASK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense_smem<NO>(K));
 }
 
 template <int NO, int K>
@@ -1571,7 +1666,8 @@ int ensure_workspace(sph_learned* L, int64_t n, int64_t E) {
   for (int r = 0; r < ROUNDS && ok; ++r)
     ok = nalloc(L, &L->XE[r], E * 80) && nalloc(L, &L->A1[r], E * 80) && nalloc(L, &L->XN[r], n * 144) &&
          nalloc(L, &L->A2[r], n * 80);
-  L->partial_elems = (size_t)kDwBlocks * 64 * 144;
+  // one round's layers and the decoder's or the encoder's
+  L->partial_elems = (size_t)kDwBlocks * (64 * 144 + 4 * 64 * 80 + 16 * 80);
   ok = ok && nalloc(L, &L->partial, L->partial_elems);
   if (!ok) {
     L->err = "device allocation of the network workspace failed";
@@ -1598,33 +1694,46 @@ int ensure_workspace(sph_learned* L, int64_t n, int64_t E) {
   return SPH_OK;
 }
 
-template <int NO>
-void dense(int64_t M, int K, const bf16* X, int ldx, const bf16* W, float* of, int ldf, int nf, int accum,
+template <int NO, int K, bool MASK = false>
+void dense(int64_t M, const bf16* X, int ldx, const bf16* W, float* of, int ldf, int nf, int accum,
            bf16* ob, int ldo, int col0, int nb, int relu, const bf16* mask, int ldm, int* err, cudaStream_t s) {
+  static_assert(K % 16 == 0, "K in MMA steps of 16");
   if (M == 0) return;
-  // K in MMA steps of 16; rows move as 16-byte pieces, results as 16-byte pieces: strides
-  // and column ranges must allow it
-  if (K % 16 || K > 144 || ldx % 8 || (of && (ldf % 4 || nf % 4)) || (ob && (ldo % 8 || col0 % 8 || nb % 8)) ||
-      (mask && ldm % 2)) {
+  // rows move as 16-byte pieces, results as 16-byte pieces: strides and column ranges must
+  // allow it; a mask applies to the bfloat16 results
+  if (ldx % 8 || (of && (ldf % 4 || nf % 4)) || (ob && (ldo % 8 || col0 % 8 || nb % 8 || nb > 64)) ||
+      (mask != nullptr) != MASK || (MASK && (ldm % 8 || of || !ob))) {
     std::fprintf(stderr, "sph_learned: dense layer with unaligned shape\n");
     return;
   }
   const int64_t tiles = (M + 127) / 128;
   const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
-  k_dense<NO><<<grid, 128, dense_smem<NO>(K), s>>>(M, K, X, ldx, W, of, ldf, nf, accum, ob, ldo, col0, nb, relu,
-                                                   mask, ldm, err);
+  k_dense<NO, K, MASK><<<grid, 128, dense_smem<NO>(K), s>>>(M, X, ldx, W, of, ldf, nf, accum, ob, ldo, col0, nb, relu,
+                                                            mask, ldm, err);
 }
 
-// grad[layer] += dY^T X over M rows
+// The weight gradients pending for one launch of k_reduce_partials
+struct DwPending {
+  DwSums S;
+  int jobs = 0, outputs = 0;
+  size_t used = 0;
+};
+
+// grad[layer] += dY^T X over M rows, complete after flush_dw
 template <int NO, int K>
-void dense_dw(sph_learned* L, int layer, int64_t M, const bf16* dY, int ldy, const bf16* X, int ldx,
+void dense_dw(sph_learned* L, DwPending& p, int layer, int64_t M, const bf16* dY, int ldy, const bf16* X, int ldx,
               cudaStream_t s) {
   if (M == 0) return;
   const int64_t rows = dw_rows(M);
   const int blocks = (int)((M + rows - 1) / rows);
-  k_dense_dw<NO, K><<<blocks, 256, dw_smem<NO, K>(), s>>>(M, rows, dY, ldy, X, ldx, L->partial);
-  const int count = NO * K;
-  k_reduce_partials<<<count / 32, 256, 0, s>>>(blocks, count, L->partial, L->grad + w_offset(layer));
+  k_dense_dw<NO, K><<<blocks, 256, dw_smem<NO, K>(), s>>>(M, rows, dY, ldy, X, ldx, L->partial + p.used);
+  p.S.job[p.jobs++] = {blocks, NO * K, w_offset(layer), p.used};
+  p.used += (size_t)blocks * NO * K;
+  p.outputs += NO * K;
+}
+void flush_dw(sph_learned* L, DwPending& p, cudaStream_t s) {
+  if (p.jobs) k_reduce_partials<<<p.outputs / 32, 256, 0, s>>>(p.S, p.jobs, L->partial, L->grad);
+  p = DwPending();
 }
 
 const bf16* Wl(const sph_learned* L, int l) { return L->wb + w_offset(l); }
@@ -1652,19 +1761,11 @@ int build_inputs(sph_handle* h, sph_learned* L, cudaStream_t s) {
     sph::scan_exclusive(L->cnt, L->off, n, L->scan_tmp, s, &dummy);
   }
   L->E = E;
-  if (b.dim == 2) {
-    k_node_features<2><<<blocks_for(n), 256, 0, s>>>(n, b.PS, b.VS, b.inst_of, b.inst, b.ctrl, b.nbr, b.nbc, L->off,
-                                                     L->esrc, L->enbr, L->U);
-    if (E > 0)
-      k_edge_features<2><<<blocks_for(E), 256, 0, s>>>(E, b.PS, b.VS, b.inst_of, b.inst, L->esrc, L->enbr, b.WP,
-                                                     L->XS);
-  } else {
-    k_node_features<3><<<blocks_for(n), 256, 0, s>>>(n, b.PS, b.VS, b.inst_of, b.inst, b.ctrl, b.nbr, b.nbc, L->off,
-                                                     L->esrc, L->enbr, L->U);
-    if (E > 0)
-      k_edge_features<3><<<blocks_for(E), 256, 0, s>>>(E, b.PS, b.VS, b.inst_of, b.inst, L->esrc, L->enbr, b.WP,
-                                                     L->XS);
-  }
+  auto nodes = b.dim == 2 ? k_node_features<2> : k_node_features<3>;
+  nodes<<<blocks_for(n), 256, 0, s>>>(n, b.PS, b.VS, b.inst_of, b.inst, b.ctrl, L->U);
+  auto edges = b.dim == 2 ? k_edge_features<2> : k_edge_features<3>;
+  edges<<<blocks_for((n + kEdgeNodes - 1) / kEdgeNodes * 32), 256, 0, s>>>(
+      n, b.PS, b.VS, b.inst_of, b.inst, b.nbr, b.nbc, L->off, b.WP, L->esrc, L->enbr, L->XS);
   return cudaGetLastError() == cudaSuccess ? SPH_OK : SPH_E_CUDA;
 }
 
@@ -1678,7 +1779,7 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
   const bool fused = L->fused == 1 && !train;
   const bool piped = L->fused == 2 && !train;
   // encoder: H = relu(U W_enc^T); H0 keeps h0 for the encoder's backward
-  dense<64>(n, 16, L->U, 16, Wl(L, L_ENC), L->H, F, F, 0, nullptr, 0, 0, 0, 1, nullptr, 0, L->tc_err, s);
+  dense<64, 16>(n, L->U, 16, Wl(L, L_ENC), L->H, F, F, 0, nullptr, 0, 0, 0, 1, nullptr, 0, L->tc_err, s);
   if (train) cudaMemcpyAsync(L->H0, L->H, sizeof(float) * n * F, cudaMemcpyDeviceToDevice, s);
   for (int r = 0; r < ROUNDS; ++r) {
     if (fused) {
@@ -1724,21 +1825,21 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
         kern<<<grid, kWsThreads, ws_smem(), s>>>(n, run, L->off, L->XS, L->enbr, L->T, Wl(L, L_E1), Wl(L, L_E2),
                                                  inv_nbar, L->XN[r], L->tc_err);
       }
-      dense<64>(n, 144, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64>(n, 80, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
+      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
     } else {
       if (E > 0) k_edge_rows<<<blocks_for(E * 10), 256, 0, s>>>(E, fe, L->XS, L->enbr, L->H, L->XE[r]);
-      dense<64>(E, 80, L->XE[r], 80, Wl(L, L_E1), nullptr, 0, 0, 0, L->A1[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64>(E, 80, L->A1[r], 80, Wl(L, L_E2), L->Mbuf, F, F, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 80>(E, L->XE[r], 80, Wl(L, L_E1), nullptr, 0, 0, 0, L->A1[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
+      dense<64, 80>(E, L->A1[r], 80, Wl(L, L_E2), L->Mbuf, F, F, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
       k_segsum<<<blocks_for(n * F), 256, 0, s>>>(n, L->off, L->Mbuf, L->H, inv_nbar, L->XN[r]);
-      dense<64>(n, 144, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64>(n, 80, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
+      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
     }
   }
   // the fused rounds leave the decoder's input rows
   if (!fused) k_rows_bf16<<<blocks_for(n * F), 256, 0, s>>>(n, F, L->H, F, L->XD, 80);
-  dense<64>(n, 80, L->XD, 80, Wl(L, L_D1), nullptr, 0, 0, 0, L->A3, 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-  dense<16>(n, 80, L->A3, 80, Wl(L, L_D2), L->Y, 16, 16, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+  dense<64, 80>(n, L->XD, 80, Wl(L, L_D1), nullptr, 0, 0, 0, L->A3, 80, 0, F, 1, nullptr, 0, L->tc_err, s);
+  dense<16, 80>(n, L->A3, 80, Wl(L, L_D2), L->Y, 16, 16, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
 }
 
 void backward(sph_handle* h, sph_learned* L, cudaStream_t s) {
@@ -1748,29 +1849,30 @@ void backward(sph_handle* h, sph_learned* L, cudaStream_t s) {
   const float inv_nbar = 1.0f / nbar(d);
   cudaMemsetAsync(L->grad, 0, sizeof(float) * kWeights, s);
   if (E > 0) k_reverse_edges<<<blocks_for(E), 256, 0, s>>>(E, L->esrc, L->enbr, L->off, L->erev);
-  // decoder
-  dense_dw<16, 80>(L, L_D2, n, L->dYb, 16, L->A3, 80, s);
-  dense<80>(n, 16, L->dYb, 16, WTl(L, L_D2), nullptr, 0, 0, 0, L->dZn, F, 0, F, 0, L->A3, 80, L->tc_err, s);
-  dense_dw<64, 80>(L, L_D1, n, L->dZn, F, L->XD, 80, s);
-  dense<80>(n, 64, L->dZn, F, WTl(L, L_D1), L->dH, F, F, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+  DwPending p;
+  // decoder; dZe is the edge buffer (at least n rows)
+  dense_dw<16, 80>(L, p, L_D2, n, L->dYb, 16, L->A3, 80, s);
+  dense<80, 16, true>(n, L->dYb, 16, WTl(L, L_D2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A3, 80, L->tc_err, s);
+  dense_dw<64, 80>(L, p, L_D1, n, L->dZe, F, L->XD, 80, s);
+  dense<80, 64>(n, L->dZe, F, WTl(L, L_D1), L->dH, F, F, 0, L->dZn, F, 0, F, 0, nullptr, 0, L->tc_err, s);
   for (int r = ROUNDS - 1; r >= 0; --r) {
-    // h_new = h + W_n2 [relu(W_n1 XN), 1]
-    k_rows_bf16<<<blocks_for(n * F), 256, 0, s>>>(n, F, L->dH, F, L->dZn, F);
-    dense_dw<64, 80>(L, L_N2, n, L->dZn, F, L->A2[r], 80, s);
-    bf16* dZ2 = L->dZe;   // reuse the edge buffer (E >= n)
-    dense<80>(n, 64, L->dZn, F, WTl(L, L_N2), nullptr, 0, 0, 0, dZ2, F, 0, F, 0, L->A2[r], 80, L->tc_err, s);
-    dense_dw<64, 144>(L, L_N1, n, dZ2, F, L->XN[r], 144, s);
-    dense<144>(n, 64, dZ2, F, WTl(L, L_N1), L->dXN, 144, 144, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
-    k_node_back<<<blocks_for(n * F), 256, 0, s>>>(n, L->dXN, L->dH);
-    if (E > 0) k_edge_back<<<blocks_for(E * F), 256, 0, s>>>(E, L->esrc, L->dXN, inv_nbar, L->dM);
-    dense_dw<64, 80>(L, L_E2, E, L->dM, F, L->A1[r], 80, s);
-    dense<80>(E, 64, L->dM, F, WTl(L, L_E2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A1[r], 80, L->tc_err, s);
-    dense_dw<64, 80>(L, L_E1, E, L->dZe, F, L->XE[r], 80, s);
-    dense<80>(E, 64, L->dZe, F, WTl(L, L_E1), L->dXE, 80, 80, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
-    if (E > 0) k_gather_dh<<<blocks_for(n * F), 256, 0, s>>>(n, fe, L->off, L->enbr, L->erev, L->dXE, L->dH);
+    // h_new = h + W_n2 [relu(W_n1 XN), 1]; dZn = bf16(dh)
+    dense_dw<64, 80>(L, p, L_N2, n, L->dZn, F, L->A2[r], 80, s);
+    bf16* dZ2 = L->dZe;
+    dense<80, 64, true>(n, L->dZn, F, WTl(L, L_N2), nullptr, 0, 0, 0, dZ2, F, 0, F, 0, L->A2[r], 80, L->tc_err, s);
+    dense_dw<64, 144>(L, p, L_N1, n, dZ2, F, L->XN[r], 144, s);
+    dense<144, 64>(n, dZ2, F, WTl(L, L_N1), L->dXN, 144, 144, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+    if (E > 0) k_edge_back<<<blocks_for(E * (F / 8)), 256, 0, s>>>(E, L->esrc, L->dXN, inv_nbar, L->dM);
+    dense_dw<64, 80>(L, p, L_E2, E, L->dM, F, L->A1[r], 80, s);
+    dense<80, 64, true>(E, L->dM, F, WTl(L, L_E2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A1[r], 80, L->tc_err, s);
+    dense_dw<64, 80>(L, p, L_E1, E, L->dZe, F, L->XE[r], 80, s);
+    dense<80, 64>(E, L->dZe, F, WTl(L, L_E1), L->dXE, 80, 80, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+    k_gather_dh<<<blocks_for(n * 32), 256, 0, s>>>(n, fe, L->off, L->enbr, L->erev, L->dXE, L->dXN,
+                                                   r == 0 ? L->H0 : nullptr, L->dH, L->dZn);
+    if (r > 0) flush_dw(L, p, s);
   }
-  k_relu_back<<<blocks_for(n * F), 256, 0, s>>>(n, L->dH, L->H0, L->dZn);
-  dense_dw<64, 16>(L, L_ENC, n, L->dZn, F, L->U, 16, s);
+  dense_dw<64, 16>(L, p, L_ENC, n, L->dZn, F, L->U, 16, s);
+  flush_dw(L, p, s);
 }
 
 }  // namespace
@@ -1867,10 +1969,14 @@ int sph_learned_create(int32_t dim, const float* weights, sph_learned** out) {
   cudaFuncSetAttribute(k_edge_round_fused<9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem());
   cudaFuncSetAttribute(k_edge_round_ws<7>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws_smem());
   cudaFuncSetAttribute(k_edge_round_ws<9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ws_smem());
-  set_smem_attrs<16>();
-  set_smem_attrs<64>();
-  set_smem_attrs<80>();
-  set_smem_attrs<144>();
+  set_smem_attrs<64, 16>();
+  set_smem_attrs<64, 80>();
+  set_smem_attrs<64, 144>();
+  set_smem_attrs<16, 80>();
+  set_smem_attrs<80, 16, true>();
+  set_smem_attrs<80, 64>();
+  set_smem_attrs<80, 64, true>();
+  set_smem_attrs<144, 64>();
   set_dw_attrs<16, 80>();
   set_dw_attrs<64, 16>();
   set_dw_attrs<64, 80>();
