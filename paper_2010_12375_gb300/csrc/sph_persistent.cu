@@ -70,7 +70,7 @@ k_substeps_persistent(const Inst Ip, int64_t n, int n_inst, const Inst* __restri
       if (dtd == 0.0) valid = false;
       const Inst& I = UNI ? Ip : inst[k];
       bool writer;
-      const float v2 = pr_particle<D, PER, false, TV, const int4*, const float4*>(
+      const float v2 = pr_particle<D, PER, false, TV, false, const int4*, const float4*>(
           I, i, valid, dtd, nullptr, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
       warp_vmax(v2, writer, k, ctrl);
     }

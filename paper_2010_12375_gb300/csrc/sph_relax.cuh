@@ -494,7 +494,15 @@ __device__ __forceinline__ float pr_group(const Inst& I, int64_t i, int sub, boo
 // Returns |v^{n+1}|^2 when the particle was written (*writer), else 0. The array pointers
 // carry the caller's aliasing qualifiers: the per-launch kernels pass __restrict__ ones, the
 // persistent loop plain ones (its phases read what other blocks wrote in the previous phase).
-template <int D, bool PER, bool FG, bool TV, typename PI, typename PF>
+//
+// EARLY: the particle's state, counts and first quad are read (i in [0, n) also where !valid)
+// without waiting for the tank's step and constants or for the counts, which put three more
+// memory latencies before a row's first gather. It pays in the per-launch 2D kernel, whose
+// rows have seven quads (19.1 -> 17.7 us at 180,000 particles, 35.5 -> 33.5 us at 500,000,
+// 94.2 -> 90.8 us for 64 tanks of 1.07M); in 3D, twenty quads, it takes registers from the
+// gathers (one 8.04M step 3 % slower as row tasks), and it gains nothing in the persistent
+// loop and in the density relaxation.
+template <int D, bool PER, bool FG, bool TV, bool EARLY, typename PI, typename PF>
 __device__ __forceinline__ float pr_particle(const Inst& I, int64_t i, bool valid, double dtd,
                                              const float4* __restrict__ geo, int64_t n, PI PS, PF VS,
                                              int4* PH, float4* VH, const float* __restrict__ mass,
@@ -508,24 +516,33 @@ __device__ __forceinline__ float pr_particle(const Inst& I, int64_t i, bool vali
   C.sx = C.sy = C.sz = C.nx = C.ny = C.nz = f2(0.f);
   C.bx = C.by = C.bz = f2(0.f);
   const float dt = (float)dtd;
-  int4 pi = make_int4(0, 0, 0, 0);
+  const int4* __restrict__ nb4 = reinterpret_cast<const int4*>(nbr);
+  int4 pi = make_int4(0, 0, 0, 0), cur = pi;
   float4 vi = make_float4(0.f, 0.f, 0.f, 0.f);
+  uint32_t cnt = 0;
+  if (EARLY) {
+    pi = PS[i];
+    cnt = nbc[i];
+    cur = nb4[i];                                     // not looked at without neighbours
+    vi = VS[i];
+  }
   if (valid) {
     C.hdt = 0.5f * dt;
     C.px = PER ? I.period[0] : 0;
     C.py = PER ? I.period[1] : 0;
     C.pz = PER ? I.period[2] : 0;
-    pi = PS[i];
-    vi = VS[i];
+    if (!EARLY) {
+      pi = PS[i];
+      vi = VS[i];
+      cnt = nbc[i];
+    }
     C.dev_i = i2f(pi.w) + C.hdt * vi.w;               // Eq. verlet-first-half (density)
     C.rho_i = I.rho0 + C.dev_i;
     C.pr_i = I.c0sq * C.dev_i;                        // Eq. eqeos
     const float2 DQ = f2(I.dq);
-    const uint32_t cnt = nbc[i];
     const int nf = (int)(cnt & 0xffffu), nw = (int)(cnt >> 16);
-    const int4* __restrict__ nb4 = reinterpret_cast<const int4*>(nbr);
     const int nq = (nf + 3) >> 2;
-    int4 cur = nq > 0 ? nb4[i] : make_int4(0, 0, 0, 0);
+    if (!EARLY && nq > 0) cur = nb4[i];
     for (int q = 0; q < nq; ++q) {
       int4 nxt = cur;
       if (q + 1 < nq) nxt = nb4[(int64_t)(q + 1) * n + i];  // next quad in flight
@@ -616,8 +633,8 @@ k_pressure_relaxation(const Inst Ip, const float4* __restrict__ geo, int64_t n, 
   bool writer;
   float v2;
   if (TPP == 1) {
-    v2 = pr_particle<D, PER, FG, TV, const int4* __restrict__, const float4* __restrict__>(
-        I, i, valid, dtd, geo, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
+    v2 = pr_particle<D, PER, FG, TV, D == 2, const int4* __restrict__, const float4* __restrict__>(
+        I, min(i, n - 1), valid, dtd, geo, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
   } else {
     __shared__ float4 terms[TPP > 1 ? BLK / 32 : 1][(1 + D) * 32];
     RowHead head;
@@ -998,7 +1015,7 @@ k_pressure_relaxation_rows(const Inst I, int64_t n, const int4* __restrict__ PS,
       const int2 piece = row_task[t];
       const bool valid = lane < piece.y;
       bool writer;
-      const float v2 = pr_particle<D, PER, false, TV, const int4* __restrict__, const float4* __restrict__>(
+      const float v2 = pr_particle<D, PER, false, TV, false, const int4* __restrict__, const float4* __restrict__>(
           I, valid ? (int64_t)piece.x + lane : 0, valid, dtd, nullptr, n, PS, VS, PH, VH, mass, nbr, nbc,
           WP, WN, acc_prior, acc_keep, g, &writer);
       if (writer) m = fmaxf(m, v2);
