@@ -522,7 +522,11 @@ std::string format_cfg(const sph::LaunchCfg& c) {
 }
 
 // Launch configuration of a handle that no autotuned entry covers (every configuration gives
-// the same bits). One thread per particle: in 2D in blocks of 128 (pressure / density
+// the same bits). Small handles, whose time is the latency of one row, share a particle among
+// four threads: in 2D below 10,000 particles (pressure / density relaxation 7 / 7 us against
+// 9 / 9 at 3,200, 8.9 / 8.4 against 8.9 / 9.1 at 16,200), in 3D below 24,000 (11 / 11 us against
+// 19 / 17 at 8,192, 13 / 13 against 19 / 17 at 16,000, 23 / 21 against 21 / 19 at 31,250).
+// Else one thread per particle: in 2D in blocks of 128 (pressure / density
 // relaxation 70 / 60 us at 980,000 particles, 77 / 62 in blocks of 256, 68 / 66 as row tasks);
 // in 3D in blocks of 256 below 300,000 particles, where blocks of 128 leave a fuller last wave
 // (62 / 59 against 69 / 61 us at 208,000), of 128 above (117 / 106 against 119 / 110 us at
@@ -531,6 +535,7 @@ std::string format_cfg(const sph::LaunchCfg& c) {
 sph::LaunchCfg default_launch(int dim, int64_t n, bool single) {
   sph::LaunchCfg c;
   c.pr_block = c.dr_block = dim == 2 || n >= 300000 ? 128 : 256;
+  if (n < (dim == 2 ? 10000 : 24000)) c.pr_tpp = c.dr_tpp = 4;
   if (dim == 3 && single && n >= 900000) c.pr_block = c.dr_block = sph::kRowBlock;
   return c;
 }
