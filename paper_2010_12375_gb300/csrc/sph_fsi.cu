@@ -93,6 +93,27 @@ __global__ void k_solid_pack_rows(int64_t ns, int cap, const int* __restrict__ c
   }
 }
 
+// After k_solid_pack_rows: the cluster blocks that read particle a's published values (those of
+// its neighbours, and its own) as a bit mask, the number of particles each block is sent, and
+// whether some neighbour's row lacks the particle (k_solid_steps_reg needs symmetric rows).
+__global__ void k_solid_readers(int64_t ns, int cap, const int* __restrict__ cnt, int P, const int* __restrict__ nb,
+                                uint32_t* __restrict__ readers, int* __restrict__ sent, int* __restrict__ lopsided) {
+  const int64_t a = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (a >= ns) return;
+  const int me = (int)((a / P) << 16 | (a % P));
+  uint32_t m = 1u << (a / P);
+  for (int t = 0; t < min(cnt[a], cap); ++t) {
+    const int pk = nb[(int64_t)t * ns + a];
+    const int64_t b = (int64_t)(pk >> 16) * P + (pk & 0xffff);
+    m |= 1u << (pk >> 16);
+    bool found = false;
+    for (int u = 0; u < min(cnt[b], cap) && !found; ++u) found = nb[(int64_t)u * ns + b] == me;
+    if (!found) *lopsided = 1;
+  }
+  readers[a] = m;
+  for (; m; m &= m - 1) atomicAdd(&sent[__ffs(m) - 1], 1);
+}
+
 // One thread per solid particle: its neighbours within 2 h_S in the reference configuration
 // (ascending index), their kernel gradients times the neighbour's volume gV_ab = V_b grad0_a
 // W_ab, the row sum c_a = sum_b gV_ab, and B0 (all in FP64, then stored in FP32).
@@ -578,6 +599,8 @@ struct SolidPtrs {
   int lanes;             // lanes per particle in the neighbour sums: 1, 2, 4, 8, 16 or 32
   int per_block;         // particles owned by each block of the cluster (the last may own fewer)
   int row;               // slots a particle in the staged rows (the longest reference row)
+  const uint32_t* readers;   // per particle, the cluster blocks that read it (k_solid_readers)
+  const int* sent;           // per block, the particles sent to it
 };
 
 // Shared-memory image of the particles one block owns during the solid steps: what the
@@ -1000,34 +1023,55 @@ k_solid_steps(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict__ ct
 // The solid's state in the caller's order (perm: internal index -> caller's), FP64.
 // The same steps for a 2D solid of which every thread group holds one particle (four lanes a
 // particle, at most kRegRow reference neighbours and kRegThreads / 4 particles a block): a
-// step is then a chain of dependent accesses, two gathers from the neighbours' shared memory
-// (about 210 cycles each) and two cluster barriers (about 600), so everything that does not
-// change over the steps (the neighbours' shared-memory addresses, V_b grad0 W, B0, c_a, the
-// fluid force) and the particle's own state stay in registers, all of a lane's neighbours are
-// fetched at once, every lane of a group carries the particle's update (no broadcasts), and
-// the sums of v and dv/dt and the position are brought up to date between a barrier's arrival
-// and its wait. A launch of about 40 steps on the 1,536-particle plate takes 60 us
-// (111 us in k_solid_steps).
+// step is then a chain of dependent accesses, two exchanges between neighbours, so everything
+// that does not change over the steps (V_b grad0 W, B0, c_a, the fluid force, where the
+// neighbours' values lie) and the particle's own state stay in registers, and every lane of a
+// group carries the particle's update (no broadcasts). Each block keeps a copy of the published
+// values of all particles it reads: a particle's lanes send its P B0, and later its v, to the
+// blocks of its neighbours (st.async), each of which counts the bytes it is due on an mbarrier
+// and then gathers from its own shared memory; the sums of v and dv/dt and the position are
+// brought up to date while the values travel. A particle overwrites a copy only after it got
+// the next value of every particle that reads it (rows are symmetric, k_solid_readers checks),
+// so one copy is enough. A launch of about 40 steps on the 1,536-particle plate takes
+// 50 us (60 us with values gathered from the other blocks' shared memory between
+// two cluster barriers a step, at about 600 cycles a barrier and 210 a gather; 111 us in
+// k_solid_steps).
 constexpr int kRegRow = 24, kRegLanes = 4, kRegThreads = 512;
+constexpr unsigned kRegWaitLimit = 1u << 21;   // polls of an exchange before the launch gives up
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 // shared-memory address of p in block `rank` of the cluster
 __device__ __forceinline__ uint32_t remote_addr(const void* p, uint32_t rank) {
   uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
   asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
-__device__ __forceinline__ float4 remote_f4(uint32_t a) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
-  return v;
+__device__ __forceinline__ void send_f4(uint32_t a, uint32_t bar, const float* v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];\n" ::"r"(a),
+               "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar)
+               : "memory");
 }
-__device__ __forceinline__ float2 remote_f2(uint32_t a) {
-  float2 v;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(a) : "memory");
-  return v;
+__device__ __forceinline__ void send_f2(uint32_t a, uint32_t bar, float2 v) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];\n" ::"r"(a),
+               "f"(v.x), "f"(v.y), "r"(bar)
+               : "memory");
+}
+// one arrival, and the bytes of the phase it begins
+__device__ __forceinline__ void expect_bytes(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"((uint32_t)__cvta_generic_to_shared(bar)),
+               "r"(bytes)
+               : "memory");
+}
+// Bounded wait of a whole warp for a phase; false in all its lanes where one gave up.
+__device__ __forceinline__ bool wait_bytes(uint64_t* bar, uint32_t parity) {
+  uint32_t done = 0;
+  for (unsigned spin = 0; spin < kRegWaitLimit && !done; ++spin)
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"((uint32_t)__cvta_generic_to_shared(bar)), "r"(parity)
+        : "memory");
+  return __all_sync(0xffffffffu, done != 0);
 }
 
 __global__ void __launch_bounds__(kRegThreads, 1)
@@ -1041,13 +1085,25 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
     if (gt_is_first() && S.g) atomicOr(&S.g->err, ERR_BOUNDS);
     return;
   }
-  __shared__ float4 sPB[kRegThreads / kRegLanes];   // published: P B0
-  __shared__ float2 sV[kRegThreads / kRegLanes];    // published: velocity
+  extern __shared__ float4 reg_smem[];
+  __shared__ uint64_t bar[2];              // P B0, v: this block's copies of the step complete
   __shared__ float red[2][kSolidThreads / 32];
   __shared__ float blk[2];
   __shared__ int s_kappa;
   const int P = S.per_block;
   const unsigned rank = cl.block_rank();
+  const int all = P * (int)cl.num_blocks();
+  float4* cPB = reg_smem;                  // [all] P B0 of particle rank * P + l
+  float2* cV = reinterpret_cast<float2*>(cPB + all);   // [all] v
+  for (int k = threadIdx.x; k < all; k += blockDim.x) {
+    cPB[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    cV[k] = make_float2(0.f, 0.f);
+  }
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < 2; ++k)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"((uint32_t)__cvta_generic_to_shared(&bar[k])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
   const int64_t first = (int64_t)rank * P;
   const int own = (int)max((int64_t)0, min((int64_t)P, S.ns - first));
   const int l = (int)threadIdx.x / L, lane = (int)threadIdx.x & (L - 1);
@@ -1059,12 +1115,12 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
   int4 q = make_int4(0, 0, 0, 0);
   float F[4] = {}, dF[4] = {}, B[4] = {};
   bool moves = false;
-  uint32_t addr[NB], addr_v[NB];
+  const int slot = (int)rank * P + min(l, P - 1);
+  int at[NB];
   float2 gv[NB];
 #pragma unroll
   for (int k = 0; k < NB; ++k) {
-    addr[k] = remote_addr(&sPB[min(l, P - 1)], rank);
-    addr_v[k] = remote_addr(&sV[min(l, P - 1)], rank);
+    at[k] = slot;
     gv[k] = make_float2(0.f, 0.f);         // no neighbour: the particle itself with weight 0
   }
   float vm = 0.f, am = 0.f;
@@ -1091,15 +1147,19 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
       if (t < nc) {
         const int pk = S.nb[(int64_t)t * S.ns + a];
         const float4 g = S.gV[(int64_t)t * S.ns + a];
-        addr[k] = remote_addr(&sPB[pk & 0xffff], (uint32_t)pk >> 16);
-        addr_v[k] = remote_addr(&sV[pk & 0xffff], (uint32_t)pk >> 16);
+        at[k] = (pk >> 16) * P + (pk & 0xffff);
         gv[k] = make_float2(g.x, g.y);
       }
     }
     vm = v4.x * v4.x + v4.y * v4.y + v4.z * v4.z;
     am = ac.x * ac.x + ac.y * ac.y + ac.z * ac.z;
   }
-  cluster_vmax(cl, vm, am, red, blk);
+  // this lane's share of the blocks that read the particle, four bits each
+  uint32_t dst = 0;
+  int n_dst = 0, bit = 0;
+  for (uint32_t m = live ? S.readers[a] : 0u; m; m &= m - 1, ++bit)
+    if ((bit & (L - 1)) == lane) dst |= (uint32_t)(__ffs(m) - 1) << (4 * n_dst++);
+  cluster_vmax(cl, vm, am, red, blk);      // also: every block's copies and mbarriers are set up
   if (threadIdx.x == 0) {
     const double dts = solid_dt(M, vm, am);
     const double r = dtF / dts;
@@ -1117,6 +1177,11 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
   if (kappa == 0) return;                  // the same decision in every block; nothing written
   const double hd = dtF / kappa;
   const float h = (float)hd, hh = 0.5f * h;
+  const uint32_t due = (uint32_t)S.sent[rank];
+  if (threadIdx.x == 0) {
+    expect_bytes(&bar[0], due * 16u);
+    expect_bytes(&bar[1], due * 8u);
+  }
   float PB[4];
   auto move = [&] {                        // half a step of the position
     if (moves) {
@@ -1124,7 +1189,7 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
       q.y += __float2int_rn(hh * v.y * I.inv_dq);
     }
   };
-  // the first half of a step: F += dt/2 dF/dt and P B0, published; the caller moves r
+  // the first half of a step: F += dt/2 dF/dt and P B0, sent; the caller moves r
   auto first_half = [&] {
     float Pk[4];
 #pragma unroll
@@ -1139,17 +1204,25 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
         for (int k = 0; k < 2; ++k) s += Pk[i * 2 + k] * B[k * 2 + j];
         PB[i * 2 + j] = s;
       }
-    if (live && lane == 0) sPB[l] = make_float4(PB[0], PB[1], PB[2], PB[3]);
+    for (int d = 0; d < n_dst; ++d) {
+      const uint32_t r = (dst >> (4 * d)) & 15u;
+      send_f4(remote_addr(&cPB[slot], r), remote_addr(&bar[0], r), PB);
+    }
   };
   first_half();
-  cluster_arrive();
   move();
-  cluster_wait();
-  for (int step = 0; step < kappa; ++step) {
+  // Warps without a particle stay out: no one waits for them, so a phase of the mbarriers could
+  // come round again unseen. A warp with one is never more than a phase behind its block's
+  // first, whose next phase needs that warp's values.
+  const int steps = __any_sync(0xffffffffu, live) ? kappa : 0;
+  bool ok = true;
+  for (int step = 0; step < steps; ++step) {
+    if (!(ok = wait_bytes(&bar[0], step & 1))) break;
+    if (threadIdx.x == 0 && step + 1 < kappa) expect_bytes(&bar[0], due * 16u);
     // A: dv/dt, v (the stress divergence as in k_solid_steps)
     float4 pb[NB];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) pb[k] = remote_f4(addr[k]);
+    for (int k = 0; k < NB; ++k) pb[k] = cPB[at[k]];
     float sx = 0.f, sy = 0.f;
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
@@ -1168,18 +1241,21 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
       v.x += h * acc.x;
       v.y += h * acc.y;
     }
-    if (live && lane == 0) sV[l] = v;
-    cluster_arrive();                      // v published; every read of P B0 done
+    for (int d = 0; d < n_dst; ++d) {
+      const uint32_t r = (dst >> (4 * d)) & 15u;
+      send_f2(remote_addr(&cV[slot], r), remote_addr(&bar[1], r), v);
+    }
     move();
     vsum.x += v.x;
     vsum.y += v.y;
     asum.x += acc.x;
     asum.y += acc.y;
-    cluster_wait();
+    if (!(ok = wait_bytes(&bar[1], step & 1))) break;
+    if (threadIdx.x == 0 && step + 1 < kappa) expect_bytes(&bar[1], due * 8u);
     // B: dF/dt from the new velocities, F the second half, then the next step's first half
     float2 vb[NB];
 #pragma unroll
-    for (int k = 0; k < NB; ++k) vb[k] = remote_f2(addr_v[k]);
+    for (int k = 0; k < NB; ++k) vb[k] = cV[at[k]];
     float G[4] = {};
 #pragma unroll
     for (int k = 0; k < NB; ++k) {
@@ -1204,12 +1280,12 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
       }
 #pragma unroll
     for (int k = 0; k < 4; ++k) F[k] = F[k] + hh * dF[k];
-    const bool more = step + 1 < kappa;
-    if (more) first_half();
-    cluster_arrive();                      // P B0 published; every read of v done
-    if (more) move();
-    cluster_wait();
+    if (step + 1 < kappa) {
+      first_half();
+      move();
+    }
   }
+  if (!ok && (threadIdx.x & 31) == 0 && S.g) atomicOr(&S.g->err, ERR_TIMEOUT);
   // the particle back to global memory, with the step averages v~ and a~, and (single time
   // stepping) the next fluid step's cap
   const float inv = 1.0f / (float)kappa;
@@ -1234,6 +1310,7 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
     cluster_vmax(cl, vm, am, red, blk);
     if (threadIdx.x == 0 && rank == 0) S.dt_cap[0] = solid_dt(M, vm, am) * (1.0 - 1e-9);
   }
+  cl.sync();                               // no block leaves while another may still send to it
 }
 
 __global__ void k_solid_export(int64_t ns, int d, const int* __restrict__ perm, const int4* __restrict__ X,
@@ -1279,6 +1356,8 @@ struct sph_solid {
   float* vol = nullptr;         // reference volumes
   int *nb = nullptr, *cnt = nullptr, *near = nullptr, *box = nullptr, *dev_err = nullptr, *kappa_last = nullptr;
   int* n_near = nullptr;        // length of the near-fluid list (device)
+  uint32_t* readers = nullptr;  // the blocks that read a particle, the particles sent to a block
+  int* sent = nullptr;          // (k_solid_readers); sent[16]: rows not symmetric
   long long* steps = nullptr;
   int* perm = nullptr;          // internal index -> the caller's (device)
   int4 *sbox = nullptr, *fbox = nullptr;   // chunk boxes: solid, near fluid list
@@ -1324,6 +1403,8 @@ sph::SolidPtrs ptrs(sph_solid* s) {
   P.acc = s->acc;
   P.vbar = s->vbar;
   P.abar = s->abar;
+  P.readers = s->readers;
+  P.sent = s->sent;
   P.steps = s->steps;
   P.kappa_last = s->kappa_last;
   P.dt_cap = s->h ? s->h->b.dt_cap : nullptr;
@@ -1407,12 +1488,17 @@ bool choose_cluster(sph_solid* s, int max_row) {
 }
 
 // Whether the chosen launch shape lets a 2D solid's steps run in registers.
+// shared memory of k_solid_steps_reg: the copies of every particle's P B0 and v
+constexpr int kRegCopies = sph::kRegThreads / sph::kRegLanes;   // particles of a block, at most
+size_t reg_copy_bytes(const sph_solid* s) { return (size_t)s->cluster * s->per_block * 24; }
+
 bool reg_steps_fit(const sph_solid* s) {
-  if (s->dim != 2 || s->lanes != sph::kRegLanes || s->row > sph::kRegRow || s->threads < s->per_block * s->lanes ||
+  if (s->dim != 2 || s->cluster > 16 || s->lanes != sph::kRegLanes || s->row > sph::kRegRow || s->threads < s->per_block * s->lanes ||
       s->per_block * s->lanes > sph::kRegThreads || s->threads > sph::kRegThreads)
     return false;
   const void* kern = (const void*)sph::k_solid_steps_reg;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * kRegCopies * 24) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -1420,6 +1506,7 @@ bool reg_steps_fit(const sph_solid* s) {
   cudaLaunchAttribute at[1];
   cfg.gridDim = dim3((unsigned)s->cluster);
   cfg.blockDim = dim3((unsigned)s->threads);
+  cfg.dynamicSmemBytes = reg_copy_bytes(s);
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)s->cluster;
   at[0].val.clusterDim.y = 1;
@@ -1435,7 +1522,7 @@ void cluster_config(const sph_solid* s, cudaStream_t st, cudaLaunchConfig_t* cfg
   *cfg = cudaLaunchConfig_t{};
   cfg->gridDim = dim3((unsigned)s->cluster);
   cfg->blockDim = dim3((unsigned)s->threads);
-  cfg->dynamicSmemBytes = s->reg ? 0 : (size_t)s->tile_bytes;
+  cfg->dynamicSmemBytes = s->reg ? reg_copy_bytes(s) : (size_t)s->tile_bytes;
   cfg->stream = st;
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)s->cluster;
@@ -1665,6 +1752,18 @@ int sph_solid_create(sph_handle* h, const sph_solid_params* p, int64_t n, const 
     return sfail(s, SPH_E_CAPACITY, "the solid does not fit the shared memory of one thread-block cluster");
   s->reg = reg_steps_fit(s);
   sph::k_solid_pack_rows<<<sph::fgrid(n), sph::kFBlock>>>(n, s->cap, s->cnt, s->per_block, s->nb);
+  if (s->reg) {
+    if (!salloc(s, &s->readers, n) || !salloc(s, &s->sent, 17)) return sfail(s, SPH_E_OOM, "device allocation failed");
+    int lopsided = 0;
+    if (cudaMemset(s->sent, 0, 17 * sizeof(int)) != cudaSuccess) cudaGetLastError();
+    sph::k_solid_readers<<<sph::fgrid(n), sph::kFBlock>>>(n, s->cap, s->cnt, s->per_block, s->nb, s->readers, s->sent,
+                                                         s->sent + 16);
+    if (cudaMemcpy(&lopsided, s->sent + 16, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) {
+      cudaGetLastError();
+      return sfail(s, SPH_E_CUDA, "solid set-up failed");
+    }
+    s->reg = lopsided == 0;
+  }
   if (cudaDeviceSynchronize() != cudaSuccess) {
     cudaGetLastError();
     return sfail(s, SPH_E_CUDA, "solid set-up failed");

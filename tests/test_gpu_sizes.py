@@ -210,3 +210,12 @@ def test_fused_edge_rounds_at_run_boundaries(sph, nx, ny):
     np.testing.assert_array_equal(y[0], y[1])
     sph.sph_learned_destroy(net)
     sim.close()
+
+
+# solid steps in registers: one block, a short last block, every block full and 16 blocks
+@pytest.mark.parametrize("ratio, L, thickness", [(1, 0.2, 0.1), (2, 0.2, 0.05), (4, 0.3, 0.0375), (4, 0.2, 0.05),
+                                                 (4, 0.825, 0.05625)])
+def test_solid_steps_over_the_blocks_of_a_cluster(sph, ratio, L, thickness):
+    from tests.test_gpu_fsi import _coupled_substep_against_oracle, _prepared
+    wl, prm = _prepared(ratio, wl=wk.water_column_on_plate(dp=1.0 / 40.0, ratio=ratio, H=0.2, L=L, thickness=thickness))
+    _coupled_substep_against_oracle(sph, wl, prm, f"ratio {ratio} L {L} thickness {thickness}")
