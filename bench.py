@@ -39,20 +39,20 @@ UNIT = "particle-substeps/s"
 # scaled to the benchmark's particle count (the traffic is per particle: state records plus
 # its neighbour row). Valid only for the kernel sources whose hash is recorded with it, in
 # the launch form it was captured in.
-TRAFFIC_BYTES_PER_PARTICLE = 389.20
-TRAFFIC_SOURCE_HASH = "5995834dfa8dd7a9"
+TRAFFIC_BYTES_PER_PARTICLE = 389.35
+TRAFFIC_SOURCE_HASH = "22697809884256d0"
 TRAFFIC_ROW_FORM = True         # captured launch form: row tasks (True) or one thread a particle
 ROW_BLOCK = 896                 # block of the row-task launch form
 # Pipe utilisation of the same kernel from the same full capture (% of peak while active):
 # the FP32 FMA pipe (scalar and packed FP32 FMA/MUL/ADD) and the L1 data pipe that bounds it
-PR_PIPES = {"fp32_fma_pipe": 0.570, "l1_data_pipe": 0.869, "issue_active": 0.605}
+PR_PIPES = {"fp32_fma_pipe": 0.569, "l1_data_pipe": 0.868, "issue_active": 0.605}
 
 
 # DRAM bytes (read + write) per particle of one diffusion stage launch, from the ncu capture
-# of k_diffusion_stage on the 120^3 block (both stages, 652.2 and 652.5 MB per launch at 1.728M
+# of k_diffusion_stage on the 120^3 block (both stages, 652.2 and 652.7 MB per launch at 1.728M
 # particles); traffic is per particle on the lattice, so it scales to the 200^3 block.
-DIFF_TRAFFIC_BYTES_PER_PARTICLE = 377.5
-DIFF_TRAFFIC_SOURCE_HASH = "36a9a20bee506b41"
+DIFF_TRAFFIC_BYTES_PER_PARTICLE = 377.6
+DIFF_TRAFFIC_SOURCE_HASH = "7450ee70e95273b3"
 # the stage kernel and its device helpers: the rest of the file (pack/unpack, the reaction
 # step, the host API) does not change the captured launches
 DIFF_SOURCES = ("sph_common.cuh", ("sph_diffusion.cu", "float2 pair_coord2(", "Per call: records of both buffers"))
