@@ -88,11 +88,13 @@ __device__ __forceinline__ void mma16816(float* c, uint32_t a0, uint32_t a1, uin
 // 128-byte shared-memory wavefront, two full global sectors per row pair of pieces), and each
 // warp stages 128 bytes of its 32 rows in shared memory (in the tile the tensor core has just
 // read, so the staging costs no shared memory of its own) to store them as whole lines.
-// A CTA mostly has one tile, so the chain of latencies counts: W comes with the first tile,
-// the mask is read in whole lines during the MMAs, and the epilogue has one staging round per
-// 128 bytes of a row. With W loaded first, 16 columns a round in 4-byte shared accesses and the
-// mask read row by row, the 28 layers of a training step of 3,200 particles (86,000 edges) took
-// 380 us and take 290. One tile buffer and more CTAs an SM instead of two buffers was no faster.
+// What bounds it at the training sizes (a few tiles an SM) is the chain of latencies of a tile:
+// W comes with the first tile, every copy is issued without a division or a wait, the MMAs are
+// issued before the next tile's copies, the mask and the sums to add to are read in whole lines
+// and all at once, and the epilogue has one staging round per 128 bytes of a row. With W loaded
+// first, 16 columns a round in 4-byte shared accesses, the mask read row by row and a CTA a
+// tile, the 28 layers of a training step of 3,200 particles (64,000 edges) took 380 us and take
+// 257 us. One tile buffer and more CTAs an SM instead of two buffers was no faster.
 // K is a multiple of 16, ldx, ldo, col0, nb_store and ldm multiples of 8, ldf and nf_store of 4
 // (checked by the host wrapper). A wait for the tensor core that runs out sets
 // ERR_TIMEOUT in *err and the CTA stops.
@@ -138,6 +140,21 @@ __device__ __forceinline__ void load_operand(unsigned char* dst, int R, int K, c
   }
 }
 
+// The same by the four warps of k_dense with the shape known when compiled: every copy of a
+// lane is issued without a division or a wait for the one before.
+template <int R, int K>
+__device__ __forceinline__ void load_tile(unsigned char* dst, const bf16* __restrict__ src, int ld, int rows_valid) {
+  constexpr int KC = K / 8, KB = (KC + 3) / 4, kBlocks = (R / 8) * KB;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = lane & 7, k0 = lane >> 3;
+#pragma unroll
+  for (int q = 0; q < (kBlocks + 3) / 4; ++q) {
+    const int blk = 4 * q + warp, r = blk / KB * 8 + r0, kc = blk % KB * 4 + k0;
+    if (blk >= kBlocks || kc >= KC) continue;
+    const bool valid = r < rows_valid;
+    cp_async16(dst + tc::core_offset(R, r, kc * 8), src + (valid ? (int64_t)r * ld : 0) + kc * 8, valid);
+  }
+}
+
 // all ones in the halves of a pair of bf16 that are > 0
 __device__ __forceinline__ uint32_t positive2(uint32_t m) {
   return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&m), __floats2bfloat162_rn(0.f, 0.f));
@@ -158,8 +175,8 @@ k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((int64_t)blockIdx.x * 128 < M) {                // the first tile and W stream in
     const int64_t m0 = (int64_t)blockIdx.x * 128;
-    load_operand<true>(sA0, 128, K, X + m0 * ldx, ldx, M - m0);
-    load_operand<true>(sB, NO, K, W, K, NO);
+    load_tile<128, K>(sA0, X + m0 * ldx, ldx, (int)min(M - m0, (int64_t)128));
+    load_tile<NO, K>(sB, W, K, NO);
   }
   cp_async_commit();
   if (threadIdx.x == 0) tc::mbar_init(&bar);
@@ -178,14 +195,16 @@ k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__
     cp_async_wait_all();
     tc::fence_to_async();
     __syncthreads();                                  // this tile in place; the other buffer free
-    const int64_t next = tile + gridDim.x;
-    if (next < tiles)                                 // the next tile streams in meanwhile
-      load_operand<true>(sA0 + (buf ^ 1) * tile_bytes, 128, K, X + next * 128 * ldx, ldx, M - next * 128);
-    cp_async_commit();
     if (threadIdx.x == 0) {
       tc::fence_after_sync();
       tc::mma_tile<NO>(tmem, tc::smem_u32(sA), b_addr, K, false, &bar);
     }
+    __syncwarp();
+    const int64_t next = tile + gridDim.x;
+    if (next < tiles)                                 // the next tile streams in meanwhile
+      load_tile<128, K>(sA0 + (buf ^ 1) * tile_bytes, X + next * 128 * ldx, ldx,
+                        (int)min(M - next * 128, (int64_t)128));
+    cp_async_commit();
     const int64_t mw = m0 + warp * 32;                // this warp's first row
     // the mask of this lane's bf16 pieces (below), in flight during the MMAs
     uint4 mk[MASK ? 8 : 1];
@@ -226,20 +245,27 @@ k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__
         }
         __syncwarp();
         const int pieces = w / 4;                     // 16-byte pieces of a row
+        float4 o[8];
+        float4* dst[8];
+        bool in[8];
 #pragma unroll
         for (int q = 0; q < pieces; ++q) {
           const int r = (q * 32 + lane) / pieces, c = (q * 32 + lane) % pieces * 4;
           const int64_t m = mw + r;
-          if (m < M && c0 + c < nf_store) {
-            float4 o = *reinterpret_cast<const float4*>(st + r * kDenseStageLd + c * 4);
-            float4* dst = reinterpret_cast<float4*>(&out_f32[m * ldf + c0 + c]);
-            if (accum) {
-              const float4 p = *dst;
-              o = make_float4(p.x + o.x, p.y + o.y, p.z + o.z, p.w + o.w);
-            }
-            *dst = o;
-          }
+          in[q] = m < M && c0 + c < nf_store;
+          dst[q] = reinterpret_cast<float4*>(&out_f32[m * ldf + c0 + c]);
+          o[q] = *reinterpret_cast<const float4*>(st + r * kDenseStageLd + c * 4);
         }
+        if (accum) {                                  // every sum read before the first is written
+          float4 p[8];
+#pragma unroll
+          for (int q = 0; q < pieces; ++q) p[q] = in[q] ? *dst[q] : o[q];
+#pragma unroll
+          for (int q = 0; q < pieces; ++q) o[q] = make_float4(p[q].x + o[q].x, p[q].y + o[q].y, p[q].z + o[q].z, p[q].w + o[q].w);
+        }
+#pragma unroll
+        for (int q = 0; q < pieces; ++q)
+          if (in[q]) *dst[q] = o[q];
         __syncwarp();                                 // the staging block is reused next
       }
     }
@@ -292,14 +318,14 @@ k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__
 // ------------------------------------------------------------------ weight gradient
 // partial[block][no][k] = sum over this block's `rows` rows m of dY[m, no] X[m, k] (tensor
 // cores, the row index is the MMA reduction dimension).
-// A layer's operands are a few MB at the training sizes (70,000 edge rows of 288 bytes), so
+// A layer's operands are a few MB at the training sizes (64,000 edge rows of 288 bytes), so
 // what bounds the kernel is how many SMs share the rows and how fast a block brings its
 // rows in: the rows are split over up to kDwBlocks blocks (two an SM) in multiples of one
 // 64-row tile, the tiles come by 16-byte cp.async into two buffers (the next one in flight
 // during the MMAs), and both operands' fragments are read with ldmatrix.trans (the rows are
 // the reduction dimension of both) from padded rows without bank conflicts. Eight warps:
 // NO/16 row tiles of the result by 8/(NO/16) column groups, the accumulators in registers.
-// A training step of a 3,200-particle 2D tank (70,000 edges) takes 1.01 ms
+// With it a training step of a 3,200-particle 2D tank (64,000 edges) took 1.01 ms
 // where blocks of 2048 rows with 2-byte loads took 14.7 ms, 15.9 ms of ncu time in this kernel.
 constexpr int kDwBlocks = 304;            // most blocks of one weight gradient (partial sums kept)
 
@@ -1706,8 +1732,12 @@ void dense(int64_t M, const bf16* X, int ldx, const bf16* W, float* of, int ldf,
     std::fprintf(stderr, "sph_learned: dense layer with unaligned shape\n");
     return;
   }
+  // One CTA an SM up to eight tiles an SM, then two: a CTA's start takes 2 us (its TMEM, its
+  // first copies), and the CTAs of an SM start one after the other, so a CTA a tile only pays
+  // where an SM has no second one (64 outputs, K = 80: 498 tiles 12.4 us with one CTA an SM, 13.6
+  // with two, 14.5 with four; 784 tiles 16.5, 16.5, 18.6; 5,000 tiles 69, 58, 62; 21,094 tiles 264, 219, 220).
   const int64_t tiles = (M + 127) / 128;
-  const unsigned grid = (unsigned)std::min<int64_t>(tiles, 152 * 8);
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, tiles <= 8 * 152 ? 152 : 2 * 152);
   k_dense<NO, K, MASK><<<grid, 128, dense_smem<NO>(K), s>>>(M, X, ldx, W, of, ldf, nf, accum, ob, ldo, col0, nb, relu,
                                                             mask, ldm, err);
 }
