@@ -764,12 +764,12 @@ void inverse_from_cholesky(const double* L, int d, double* Dinv) {
 // Whether a call runs in one launch: while every particle has a lane of its own (1024 an SM),
 // where a one-step call and a further step took, as stage launches and in one launch, 32 + 12.6
 // and 16.5 + 9.9 us on a 2D sheet of 40,000, 75 + 54 and 45 + 39 us on a 3D block of 64,000;
-// beyond that for short calls, whose packing and synchronisation it saves (44 + 15.7 against
-// 26 + 18.0 us on 160,000 in 2D, 142 + 117 against 123 + 114 us on 216,000 in 3D, but 244 + 217
-// against 252 + 240 us on 512,000).
+// beyond that in 2D for short calls, whose packing and synchronisation it saves (44 + 15.7
+// against 26 + 18.0 us on 160,000). In 3D a second, nearly empty pass of long rows costs more
+// than that (a call of two steps 39 us slower on 166,375, even on 216,000).
 bool small_diffusion(const sph::Buffers& b, int n_steps) {
   const int64_t per = (b.n + b.n_sm - 1) / b.n_sm;
-  return per <= 2 * sph::kSmallThreads || (n_steps <= 4 && per <= (b.dim == 2 ? 4096 : 1400));
+  return per <= 2 * sph::kSmallThreads || (b.dim == 2 && n_steps <= 4 && per <= 4096);
 }
 
 }  // namespace
