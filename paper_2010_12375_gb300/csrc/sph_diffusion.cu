@@ -564,9 +564,14 @@ cudaError_t launch_small(const DiffSmall& a, int n_sm, cudaStream_t s) {
   const void* kern = lpp == 4 ? (const void*)k_diffusion_small<D, PER, ISO, 4>
                               : lpp == 2 ? (const void*)k_diffusion_small<D, PER, ISO, 2>
                                          : (const void*)k_diffusion_small<D, PER, ISO, 1>;
-  const int64_t lanes = a.n * lpp;
-  const int threads = (int)std::min<int64_t>(kSmallThreads, std::max<int64_t>(128, (lanes / (2 * n_sm) + 31) / 32 * 32));
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((lanes + threads - 1) / threads, 2 * (int64_t)n_sm));
+  // two blocks an SM, as large as splits the lanes evenly over the passes that they need: a pass
+  // is a chain of dependent gathers, nearly as long with a few warps in it as with many (3D,
+  // 166,375 particles in blocks of 512 and 288: one step 126 and 98 us, a further one 111 and 83)
+  const int64_t lanes = a.n * lpp, blocks = 2 * (int64_t)n_sm;
+  const int64_t passes = (lanes + blocks * kSmallThreads - 1) / (blocks * kSmallThreads);
+  const int64_t share = (lanes + blocks * passes - 1) / (blocks * passes);
+  const int threads = (int)std::max<int64_t>(128, (share + 31) / 32 * 32);
+  const int grid = (int)std::min<int64_t>((lanes + threads - 1) / threads, blocks);
   void* args[] = {const_cast<DiffSmall*>(&a)};
   return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(threads), args, 0, s);
 }
@@ -762,14 +767,15 @@ void inverse_from_cholesky(const double* L, int d, double* Dinv) {
 }
 
 // Whether a call runs in one launch: while every particle has a lane of its own (1024 an SM),
-// where a one-step call and a further step took, as stage launches and in one launch, 32 + 12.6
-// and 16.5 + 9.9 us on a 2D sheet of 40,000, 75 + 54 and 45 + 39 us on a 3D block of 64,000;
-// beyond that in 2D for short calls, whose packing and synchronisation it saves (44 + 15.7
-// against 26 + 18.0 us on 160,000). In 3D a second, nearly empty pass of long rows costs more
-// than that (a call of two steps 39 us slower on 166,375, even on 216,000).
+// where a one-step call and a further step took, as stage launches and in one launch, 39 + 12.4
+// and 24 + 9.9 us on a 2D sheet of 40,000, 94 + 66 and 62 + 48 us on a 3D block of 97,336;
+// beyond that for calls of at most four steps, whose packing and synchronisation it saves (a
+// call of one and of four steps, stage launches and one launch: 2D 44 / 94 and 28 / 69 us on
+// 160,000, 76 / 187 and 50 / 147 on 620,944; 3D 110 / 356 and 97 / 344 us on 157,464, 122 / 402
+// and 98 / 347 on 166,375, 135 / 455 and 107 / 382 on 205,379).
 bool small_diffusion(const sph::Buffers& b, int n_steps) {
   const int64_t per = (b.n + b.n_sm - 1) / b.n_sm;
-  return per <= 2 * sph::kSmallThreads || (b.dim == 2 && n_steps <= 4 && per <= 4096);
+  return per <= 2 * sph::kSmallThreads || (n_steps <= 4 && per <= (b.dim == 2 ? 4096 : 1400));
 }
 
 }  // namespace
