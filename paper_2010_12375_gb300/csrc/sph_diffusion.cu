@@ -772,10 +772,16 @@ void inverse_from_cholesky(const double* L, int d, double* Dinv) {
 // beyond that for calls of at most four steps, whose packing and synchronisation it saves (a
 // call of one and of four steps, stage launches and one launch: 2D 44 / 94 and 28 / 69 us on
 // 160,000, 76 / 187 and 50 / 147 on 620,944; 3D 110 / 356 and 97 / 344 us on 157,464, 122 / 402
-// and 98 / 347 on 166,375, 135 / 455 and 107 / 382 on 205,379).
-bool small_diffusion(const sph::Buffers& b, int n_steps) {
-  const int64_t per = (b.n + b.n_sm - 1) / b.n_sm;
-  return per <= 2 * sph::kSmallThreads || (n_steps <= 4 && per <= (b.dim == 2 ? 4096 : 1400));
+// and 98 / 347 on 166,375, 135 / 455 and 107 / 382 on 205,379). A 2D stage with an anisotropic
+// tensor is slower in one launch past two passes, so that only a one-step call gains there: one,
+// two and four steps 62 / 95 / 161 and 46 / 78 / 140 us on 302,500 (two passes), 71 / 111 / 192
+// and 61 / 106 / 195 on 422,500, 76 / 120 / 207 and 71 / 124 / 231 on 490,000, 91 / 141 / 240 and
+// 77 / 137 / 254 on 608,400.
+bool small_diffusion(const sph::Buffers& b, int n_steps, bool iso) {
+  const int64_t per = (b.n + b.n_sm - 1) / b.n_sm, lanes = 2 * sph::kSmallThreads;
+  if (per <= lanes) return true;
+  if (b.dim == 3) return n_steps <= 4 && per <= 1400;
+  return n_steps <= (iso || per <= 2 * lanes ? 4 : 1) && per <= 4 * lanes;
 }
 
 }  // namespace
@@ -1053,7 +1059,7 @@ int sph_diffusion_step(sph_handle* h, sph_species* sp, double dt, int32_t n_step
   const float fdt = (float)dt;
   if (cudaMemsetAsync(sp->nonuniform, 0, 2 * sizeof(int), s) != cudaSuccess)
     return sfail(sp, SPH_E_CUDA, "diffusion set-up failed");
-  if (!sp->Lrow && !sp->corrected && small_diffusion(b, n_steps)) {
+  if (!sp->Lrow && !sp->corrected && small_diffusion(b, n_steps, sp->iso)) {
     const sph::DiffSmall a{b.n, n_steps, b.PS, b.id, b.inst_of, b.inst, b.mass, sp->by_row, sp->r0, sp->r1, sp->vol,
                            sp->scale_by_row, sp->sq, b.nbr, b.nbc, sp->K, fdt,
                            reinterpret_cast<unsigned*>(sp->nonuniform), b.glob};

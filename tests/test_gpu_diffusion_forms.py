@@ -46,3 +46,27 @@ def test_one_launch_diffusion_equals_the_stage_launches_in_3d(sph, n, copies, ma
     assert not np.array_equal(out[0][0], C0.astype(np.float32))
     for row in out[1]:
         np.testing.assert_array_equal(row, out[0][0])
+
+
+@pytest.mark.parametrize("n", [550, 570])
+def test_anisotropic_2d_calls_take_the_faster_form(sph, n):
+    # up to two passes (2048 particles an SM) calls of a few steps run in one launch, past that
+    # only those of one step; two calls of one step equal a call of two bit for bit
+    per = -(-n * n // torch.cuda.get_device_properties(0).multi_processor_count)
+    prob = wk.diffusion_band(n=n, ny=n)
+    sim = sph.Simulation(prob)
+    sim.build_cells()
+    sp = sph.sph_species_create(sim.handle, np.array([[2.0, 0.3], [0.3, 1.0]]), 2)
+    C0 = np.random.default_rng(3).uniform(0.0, 1.0, sim.n)
+    out, launches = [], []
+    for calls, steps in ((1, 2), (2, 1)):
+        sph.sph_species_set(sim.handle, sp, C0)
+        before = sim.kernel_launches()
+        for _ in range(calls):
+            sph.sph_diffusion_step(sim.handle, sp, 0.3 * prob.meta["dt"], steps)
+        launches.append(sim.kernel_launches() - before)
+        out.append(sph.sph_species_get(sim.handle, sp, sim.n))
+    sph.sph_species_destroy(sp)
+    sim.close()
+    assert launches[1] == 2 and (launches[0] == 1) == (per <= 2048)
+    np.testing.assert_array_equal(out[0], out[1])
