@@ -904,12 +904,14 @@ int sph_step(sph_handle* h, int32_t n_advection_steps, void* stream) {
     const int per = (h->flags & SPH_FLAG_PERSISTENT) ? n_advection_steps : 1;
     cudaError_t e = cudaSuccess;
     int done = 0;
-    for (; done < n_advection_steps && e == cudaSuccess; done += per) e = sph::launch_fused_steps(h->b, per, s);
-    if (e == cudaSuccess) {
-      h->launches += n_advection_steps / per;
+    while (done < n_advection_steps && (e = sph::launch_fused_steps(h->b, per, done > 0, s)) == cudaSuccess)
+      done += per;
+    if (done > 0) {
+      h->launches += done / per;
       h->rows_valid = false;                     // the row pieces follow the new order
       h->cells_valid = true;
-      const int r = sync_status(h, s);
+      int r = sync_status(h, s);
+      if (r == SPH_OK && e != cudaSuccess) r = cuda_fail(h, e, "advection step launch");
       if (r != SPH_OK) {                         // a failed launch may leave its counters behind
         h->step_ctl_dirty = true;
         h->counts_zero = false;
@@ -917,7 +919,6 @@ int sph_step(sph_handle* h, int32_t n_advection_steps, void* stream) {
       return r;
     }
     cudaGetLastError();                          // no room for a cooperative launch: the general paths
-    if (done > per) return cuda_fail(h, e, "advection step launch");
   }
   if ((h->flags & SPH_FLAG_PERSISTENT) && !h->timing && !debug_bounds(h) && !h->b.geo && !h->b.hrev && !h->solid) {
     // each advection step: the configuration update and the advection step's kernels, then

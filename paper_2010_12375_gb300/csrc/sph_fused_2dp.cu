@@ -3,7 +3,7 @@
 #include "sph_fused_step.cuh"
 
 namespace sph {
-cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s) {
-  return launch_d<2, true>(b, n_steps, clear_counts, s);
+cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s) {
+  return launch_d<2, true>(b, n_steps, clear_counts, follow, s);
 }
 }  // namespace sph

@@ -3,7 +3,7 @@
 #include "sph_fused_step.cuh"
 
 namespace sph {
-cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s) {
-  return launch_d<3, false>(b, n_steps, clear_counts, s);
+cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s) {
+  return launch_d<3, false>(b, n_steps, clear_counts, follow, s);
 }
 }  // namespace sph

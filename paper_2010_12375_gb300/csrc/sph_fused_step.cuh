@@ -20,6 +20,10 @@
 //  - reordered records go to the half-step arrays, the search reads them there and writes
 //    each particle's own record back, so no pass copies them;
 //  - the scan of the cell counts leaves the counts zero for the next step.
+// A step after the first (of a launch or, with `follow`, of a call) does not begin once the
+// status holds an error: not its hash, which would count on top of what a launch whose barrier
+// gave up left in the counts. Until every block has passed that test the errors of a step's own
+// hash wait in StepCtl, so that all blocks decide alike.
 // Every sum adds the terms the per-launch kernels add in their order: the state is identical
 // to theirs bit for bit, whatever the launch configuration.
 // A further step of the 2D dam break takes 55 us at 3,200 particles and 158 us at 100,352 (132
@@ -259,12 +263,13 @@ __device__ __forceinline__ uint32_t search_group_periodic(const Buffers& b, cons
 
 template <int D, bool PER, int LPP, bool TV>
 __global__ void __launch_bounds__(kStepThreads<LPP> + 32, 1)
-k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
+k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts, int follow) {
   __shared__ float4 terms_all[LPP > 1 ? kStepThreads<LPP> / 32 : 1][(1 + D + (TV ? 1 : 0)) * 32];
   __shared__ uint32_t warp_tot[kStepMaxWarps];
   __shared__ unsigned vmax_block;
   __shared__ Ctrl C;                             // the tank's control, kept alike by every block
   __shared__ int more;                           // substeps needed after the next one
+  __shared__ int failed;                         // the status before a step
   constexpr int LS = D == 3 ? 32 : 8;            // lanes of a particle in the search
   const Inst& I = b.inst0;
   StepCtl* c = b.step_ctl;
@@ -284,14 +289,24 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
   unsigned target = 0;
 
   if (threadIdx.x == 0) C = b.ctrl[0];
-  if (clear_counts) {
-    for (int64_t k = tid; k < b.n_cells; k += threads) b.count[k] = 0u;
-    if (!grid_barrier(&c->count, target, g)) return;
-  }
   for (int st = 0; st < n_steps; ++st) {
+    int4 p = tid < n ? b.PS[tid] : make_int4(0, 0, 0, 0);   // on its way while the status is read
+    if (st > 0 || follow) {
+      if (threadIdx.x == 0) failed = *(volatile int*)&g->err;
+      __syncthreads();
+      if (failed) {                              // an earlier step failed
+        if (st == 0) return;                     // every block: nothing has been touched
+        break;
+      }
+    }
+    if (st == 0 && clear_counts) {
+      for (int64_t k = tid; k < b.n_cells; k += threads) b.count[k] = 0u;
+      if (!grid_barrier(&c->count, target, g)) return;
+    }
     // ---- cells: hash, scan, sort by (cell, id)
     for (int64_t i = tid; i < n; i += threads) {
-      const uint32_t cell = hash_cell<D>(I, b.PS[i], i, g);
+      if (i != tid) p = b.PS[i];
+      const uint32_t cell = hash_cell<D>(I, p, i, &c->found);
       b.cell[i] = cell;
       b.rank[i] = atomicAdd(&b.count[cell], 1u);
     }
@@ -302,12 +317,8 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
       sum += v.x + v.y + v.z + v.w;
     }
     block_scan(sum, warp_tot, &total);
-    if (threadIdx.x == 0) {
-      c->sums[blockIdx.x] = total;
-      if (blockIdx.x == 0) c->stop = st > 0 && *(volatile int*)&g->err != 0;
-    }
+    if (threadIdx.x == 0) c->sums[blockIdx.x] = total;
     if (!grid_barrier(&c->count, target, g)) return;
-    if (c->stop) break;                          // an earlier step failed
     uint32_t before = 0, run;
     for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) before += c->sums[k];
     block_scan(before, warp_tot, &run);          // the particles of the cells before this block's
@@ -347,8 +358,13 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
     // ---- neighbours and density, a block's share of the particles at a time; Dt_ad and the
     // first dt beside them
     if (control) {
+      const int found = blockIdx.x == 0 ? *(volatile int*)&c->found.err : 0;
       dt_advection_one(I, C);
       more = dt_acoustic_one(I, C, g, 0.0);
+      if (found) {                               // the hash's errors to the status
+        raise_error(g, found, *(volatile long long*)&c->found.bad_index);
+        c->found.err = 0;
+      }
     }
     for (int64_t i0 = block0; i0 < n; i0 += step) {
       const int count = (int)min((int64_t)share, n - i0);
@@ -437,14 +453,14 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts) {
 }
 
 template <int D, bool PER, int LPP, bool TV>
-cudaError_t launch_t(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s) {
+cudaError_t launch_t(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s) {
   // the particles' lanes over all SMs, in blocks of 128 work threads or more; a few more
   // blocks where the cells would be many for them (a scan of 8192 a block)
   const int64_t lanes = b.n * LPP;
   const int work = (int)std::min<int64_t>(kStepThreads<LPP>, std::max<int64_t>(128, ((lanes + b.n_sm - 1) / b.n_sm + 31) / 32 * 32));
   const int64_t want = std::max((lanes + work - 1) / work, (b.n_cells + 8191) / 8192);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>({want, (int64_t)b.n_sm, (int64_t)kStepMaxGrid}));
-  void* args[] = {const_cast<Buffers*>(&b), &n_steps, &clear_counts};
+  void* args[] = {const_cast<Buffers*>(&b), &n_steps, &clear_counts, &follow};
   return cudaLaunchCooperativeKernel((const void*)k_fused_step<D, PER, LPP, TV>, dim3(grid), dim3(work + 32), args, 0, s);
 }
 
@@ -454,16 +470,16 @@ cudaError_t launch_t(const Buffers& b, int n_steps, int clear_counts, cudaStream
 // 20,000 and 188 / 166 / 135 / 126 at 51,200; of the 3D one 106 / 150 / 278 / 348 us at 2,662
 // and 183 / 153 / 253 / 319 at 16,000.
 template <int D, bool PER>
-cudaError_t launch_d(const Buffers& b, int n_steps, int clear, cudaStream_t s) {
+cudaError_t launch_d(const Buffers& b, int n_steps, int clear, int follow, cudaStream_t s) {
   const int64_t per = (b.n + b.n_sm - 1) / b.n_sm;         // particles of an SM
   if (b.any_transport) {
-    if (per * 4 <= kStepThreads<4>) return launch_t<D, PER, 4, true>(b, n_steps, clear, s);
-    return launch_t<D, PER, 1, true>(b, n_steps, clear, s);
+    if (per * 4 <= kStepThreads<4>) return launch_t<D, PER, 4, true>(b, n_steps, clear, follow, s);
+    return launch_t<D, PER, 1, true>(b, n_steps, clear, follow, s);
   }
-  if (per * 8 <= kStepThreads<8>) return launch_t<D, PER, 8, false>(b, n_steps, clear, s);
-  if (per * 4 <= kStepThreads<4>) return launch_t<D, PER, 4, false>(b, n_steps, clear, s);
-  if (per * 2 <= kStepThreads<2> / 2) return launch_t<D, PER, 2, false>(b, n_steps, clear, s);
-  return launch_t<D, PER, 1, false>(b, n_steps, clear, s);
+  if (per * 8 <= kStepThreads<8>) return launch_t<D, PER, 8, false>(b, n_steps, clear, follow, s);
+  if (per * 4 <= kStepThreads<4>) return launch_t<D, PER, 4, false>(b, n_steps, clear, follow, s);
+  if (per * 2 <= kStepThreads<2> / 2) return launch_t<D, PER, 2, false>(b, n_steps, clear, follow, s);
+  return launch_t<D, PER, 1, false>(b, n_steps, clear, follow, s);
 }
 
 }  // namespace

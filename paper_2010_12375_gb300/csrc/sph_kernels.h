@@ -30,7 +30,7 @@ struct StepCtl {
   unsigned count;            // arrivals of the barriers so far (zero between launches)
   unsigned exits;            // blocks that have left the launch
   unsigned vm[2];            // bits of max |v|^2 of a substep (alternating)
-  int stop;                  // an earlier step of the launch failed
+  Global found;              // errors of a step's cell hash, on their way to the handle's status
   unsigned sums[kStepMaxGrid];   // particles in each block's cells
 };
 
@@ -139,15 +139,16 @@ void launch_density_relaxation(const Buffers& b, cudaStream_t s, int64_t* launch
 cudaError_t launch_substeps_persistent(const Buffers& b, cudaStream_t s, int* grid_out);
 // n_steps whole advection steps of a handle of one tank in one cooperative launch (not with
 // the frozen-geometry or half-pair evaluation, nor a solid)
-// (clear_counts: the cell counts are not all zero yet)
-cudaError_t launch_fused_2d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
-cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);   // a periodic axis
-cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
-cudaError_t launch_fused_3dp(const Buffers& b, int n_steps, int clear_counts, cudaStream_t s);
-inline cudaError_t launch_fused_steps(const Buffers& b, int n_steps, cudaStream_t s) {
+// (clear_counts: the cell counts are not all zero yet; follow: the launch goes on with the
+// steps of the one before it, and leaves everything as it is if that one failed)
+cudaError_t launch_fused_2d(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);
+cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);   // a periodic axis
+cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);
+cudaError_t launch_fused_3dp(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);
+inline cudaError_t launch_fused_steps(const Buffers& b, int n_steps, bool follow, cudaStream_t s) {
   auto f = b.dim == 2 ? (b.any_periodic ? launch_fused_2dp : launch_fused_2d)
                       : (b.any_periodic ? launch_fused_3dp : launch_fused_3d);
-  const cudaError_t e = f(b, n_steps, *b.counts_zero ? 0 : 1, s);
+  const cudaError_t e = f(b, n_steps, *b.counts_zero ? 0 : 1, follow ? 1 : 0, s);
   if (e == cudaSuccess) *b.counts_zero = true;   // a launch leaves the cell counts zero
   return e;
 }
