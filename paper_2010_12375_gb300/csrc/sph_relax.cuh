@@ -295,7 +295,7 @@ __device__ __forceinline__ float pr_finish(const Inst& I, const PrCtx& C, int64_
 // lane a summing axis a. A particle's sums thus add the same terms in the same order as one
 // lane does: the results are identical bit for bit for every LPP, while a particle's chain of
 // dependent gathers is LPP times shorter. terms: this warp's [1 + D][32] float4 of shared
-// memory. All lanes of a group share `valid`.
+// memory, with the transport velocity [2 + D][32]. All lanes of a group share `valid`.
 //
 // Particle p of a warp's 32 / LPP has the lanes p, p + 32 / LPP, ...: neighbouring lanes hold
 // neighbouring particles at the same place of their rows, whose records lie close together
@@ -490,7 +490,7 @@ __device__ __forceinline__ float pr_group(const Inst& I, int64_t i, int sub, boo
 // FG: pair geometry from the frozen table geo ([slot][n]) instead of the positions.
 // TV: transport velocity (Eq. transport): the mid-point position written for the density
 // relaxation also takes dt^2/2 a_i, a_i = -(2 p0 / rho_i) sum_j V_j grad_i W_ij over the
-// fluid pairs (one thread per particle only).
+// fluid pairs.
 // Returns |v^{n+1}|^2 when the particle was written (*writer), else 0. The array pointers
 // carry the caller's aliasing qualifiers: the per-launch kernels pass __restrict__ ones, the
 // persistent loop plain ones (its phases read what other blocks wrote in the previous phase).
@@ -636,7 +636,8 @@ k_pressure_relaxation(const Inst Ip, const float4* __restrict__ geo, int64_t n, 
     v2 = pr_particle<D, PER, FG, TV, D == 2, const int4* __restrict__, const float4* __restrict__>(
         I, min(i, n - 1), valid, dtd, geo, n, PS, VS, PH, VH, mass, nbr, nbc, WP, WN, acc_prior, acc_keep, g, &writer);
   } else {
-    __shared__ float4 terms[TPP > 1 ? BLK / 32 : 1][(1 + D) * 32];
+    static_assert(TPP == 1 || !FG, "frozen geometry: one thread per particle");
+    __shared__ float4 terms[TPP > 1 ? BLK / 32 : 1][(1 + D + (TV ? 1 : 0)) * 32];
     RowHead head;
     head.load<TPP>(valid ? i : -1, sub, n, reinterpret_cast<const int4*>(nbr), nbc);
     v2 = pr_group<D, PER, TPP, TV>(I, i, sub, valid, dtd, n, PS, VS, PH, VH, mass,
@@ -967,6 +968,7 @@ k_density_relaxation(const Inst Ip, const float4* __restrict__ geo, int64_t n, c
     dr_particle<D, PER, FG, const int4* __restrict__, const float4* __restrict__>(
         I, i, valid, dtd, geo, n, PH, VH, PS, VS, mass, nbr, nbc, WP, WN, g);
   } else if (valid) {
+    static_assert(TPP == 1 || !FG, "frozen geometry: one thread per particle");
     __shared__ float4 terms[TPP > 1 ? BLK / 32 : 1][2 * 32];
     RowHead head;
     head.load<TPP>(i, sub, n, reinterpret_cast<const int4*>(nbr), nbc);
