@@ -469,11 +469,15 @@ int sph_species_set_tensors(sph_handle* h, sph_species* sp, const double* Dp, vo
 int sph_species_set_correction(sph_handle* h, sph_species* sp, int32_t on);
 /* n_steps RK2 steps of size dt (> 0, finite) on the current neighbour table, which
  * must be valid (sph_build_cells after the last state change; SPH_E_INVALID otherwise).
- * Positions, velocities and densities are not changed. Two kernel launches per step plus
- * a gather and a scatter of the species per call; the call synchronises stream once,
- * after the gather, to learn whether volumes and factors are uniform within each tank
- * (then the stage kernels take them out of the pair loop), and is otherwise
- * asynchronous. */
+ * Positions, velocities and densities are not changed. The plain form (no per-particle
+ * tensors, no correction) on few particles, up to 1024 an SM and for calls of few steps
+ * somewhat more, is one cooperative launch and asynchronous; a wait in it that runs out
+ * (about a second) makes sph_species_get and later diffusion steps on the handle return
+ * SPH_E_TIMEOUT until sph_clear_error, and leaves the species incomplete. Otherwise two
+ * kernel launches per step plus a gather and a scatter of the species per call; the call
+ * synchronises stream once, after the gather, to learn whether volumes and factors are
+ * uniform within each tank (then the stage kernels take them out of the pair loop), and is
+ * otherwise asynchronous. */
 int sph_diffusion_step(sph_handle* h, sph_species* sp, double dt, int32_t n_steps, void* stream);
 
 /* ---- Reaction step of reaction-diffusion (Sec. "SPH method for reaction-diffusion",

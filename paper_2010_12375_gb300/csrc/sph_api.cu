@@ -729,7 +729,9 @@ int sph_create(const sph_params* params, int32_t n_instances, const int64_t* flu
   }
   DALLOC(h, h->diag_scratch, sph::diag_scratch_elems(b));
   DALLOC(h, h->diag_out, (size_t)n_instances * sph::kDiagFields);
-  CK(h, cudaMallocHost((void**)&h->hglob, sizeof(Global)));
+  CK(h, cudaMallocHost((void**)&h->hglob, sizeof(Global) + sizeof(int)));
+  h->hstall = reinterpret_cast<int*>(h->hglob + 1);
+  *h->hstall = 0;
   {
     int r = ensure_stage(h, std::max<size_t>((size_t)n_fluid * (2 * dim + 2), (size_t)n_wall * (2 * dim + 1)));
     if (r != SPH_OK) return r;
@@ -1235,6 +1237,7 @@ int sph_clear_error(sph_handle* h, void* stream) {
   CK(h, cudaMemsetAsync(&h->b.glob->err, 0, sizeof(int), s));
   CK(h, cudaMemsetAsync(&h->b.glob->bad_index, 0, sizeof(long long), s));
   CK(h, cudaStreamSynchronize(s));
+  *h->hstall = 0;
   h->err.clear();
   return SPH_OK;
 }

@@ -466,6 +466,7 @@ struct DiffSmall {
   float dt;
   unsigned* ctl;             // [2] zero at launch: barrier arrivals, flag of unequal volumes or factors
   Global* g;
+  volatile int* stall;       // host memory: set when a barrier gave up, the species then being incomplete
 };
 constexpr int kSmallThreads = 512;
 
@@ -482,7 +483,12 @@ k_diffusion_small(const DiffSmall a) {
   unsigned target = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     pack_slot<D>(i, a.P, a.id, a.inst_of, a.inst, a.mass, a.by_row, a.r0, a.r1, a.vol, a.scale_by_row, a.sq, a.ctl + 1);
-  if (!grid_barrier(a.ctl, target, a.g)) return;
+  auto all_here = [&] {                            // bounded: a launch that gives up says so
+    const bool ok = grid_barrier(a.ctl, target, a.g);
+    if (!ok && threadIdx.x == 0) *a.stall = 1;
+    return ok;
+  };
+  if (!all_here()) return;
   const bool unif = *(volatile unsigned*)(a.ctl + 1) == 0u;
   const int4* nb4 = reinterpret_cast<const int4*>(a.nbr);
   // the stage's sum of particle i over its row, in lane 0 of the group
@@ -553,7 +559,7 @@ k_diffusion_small(const DiffSmall a) {
         if (st == 2 * a.n_steps - 1) a.by_row[a.id[i]] = out;
       }
     }
-    if (st < 2 * a.n_steps - 1 && !grid_barrier(a.ctl, target, a.g)) return;
+    if (st < 2 * a.n_steps - 1 && !all_here()) return;
   }
 }
 
@@ -707,6 +713,13 @@ namespace {
 int sfail(sph_species* sp, int code, const std::string& msg) {
   if (sp) sp->err = msg;
   return code;
+}
+
+// Whether a diffusion call on the handle that has run so far gave up at a barrier: the call
+// itself returns before it has run.
+int stalled(sph_handle* h, sph_species* sp) {
+  return *(volatile int*)h->hstall ? sfail(sp, SPH_E_TIMEOUT, "a diffusion step gave up waiting and left the species incomplete")
+                                   : SPH_OK;
 }
 
 // Where a caller array lives: host memory (copied through the staging buffer), memory
@@ -902,7 +915,8 @@ int sph_species_set(sph_handle* h, sph_species* sp, const double* C, void* strea
 }
 
 int sph_species_get(sph_handle* h, sph_species* sp, double* C, void* stream) {
-  return species_download(h, sp, sp ? sp->by_row : nullptr, C, stream);
+  const int r = species_download(h, sp, sp ? sp->by_row : nullptr, C, stream);
+  return r == SPH_OK ? stalled(h, sp) : r;
 }
 
 int sph_species_set_gate(sph_handle* h, sph_species* sp, const double* w, void* stream) {
@@ -1054,6 +1068,7 @@ int sph_diffusion_step(sph_handle* h, sph_species* sp, double dt, int32_t n_step
   }
   const sph::Buffers& b = h->b;
   if (b.n == 0 || n_steps == 0) return SPH_OK;
+  if (const int r = stalled(h, sp)) return r;
   cudaStream_t s = (cudaStream_t)stream;
   const unsigned grid = sph::diff_grid(b.n);
   const float fdt = (float)dt;
@@ -1062,7 +1077,7 @@ int sph_diffusion_step(sph_handle* h, sph_species* sp, double dt, int32_t n_step
   if (!sp->Lrow && !sp->corrected && small_diffusion(b, n_steps, sp->iso)) {
     const sph::DiffSmall a{b.n, n_steps, b.PS, b.id, b.inst_of, b.inst, b.mass, sp->by_row, sp->r0, sp->r1, sp->vol,
                            sp->scale_by_row, sp->sq, b.nbr, b.nbc, sp->K, fdt,
-                           reinterpret_cast<unsigned*>(sp->nonuniform), b.glob};
+                           reinterpret_cast<unsigned*>(sp->nonuniform), b.glob, h->hstall};
     using Launch = cudaError_t (*)(const sph::DiffSmall&, int, cudaStream_t);
     const Launch f = b.dim == 2
         ? (b.any_periodic ? (sp->iso ? sph::launch_small<2, true, true> : sph::launch_small<2, true, false>)

@@ -29,6 +29,7 @@ struct sph_handle {
   double* diag_scratch = nullptr;
   double* diag_out = nullptr;
   sph::Global* hglob = nullptr;         // pinned host mirror of the device status
+  int* hstall = nullptr;                // behind it: a one-launch diffusion call gave up (written by the device)
   // kernel timing
   bool timing = false;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
