@@ -327,7 +327,9 @@ k_dense(int64_t M, const bf16* __restrict__ X, int ldx, const bf16* __restrict__
 // NO/16 row tiles of the result by 8/(NO/16) column groups, the accumulators in registers.
 // With it a training step of a 3,200-particle 2D tank (64,000 edges) took 1.01 ms
 // where blocks of 2048 rows with 2-byte loads took 14.7 ms, 15.9 ms of ncu time in this kernel.
-constexpr int kDwBlocks = 304;            // most blocks of one weight gradient (partial sums kept)
+// Most blocks of one weight gradient (their partial sums are kept): two for each of GB300's 152
+// SMs, fixed, since a gradient's rounding follows the split.
+constexpr int kDwBlocks = 304;
 
 inline int64_t dw_rows(int64_t M) {       // rows per block
   const int64_t r = (M + kDwBlocks - 1) / kDwBlocks;
@@ -1609,6 +1611,7 @@ struct sph_learned {
   int64_t adam_t = 0;
   int fused = 1;                             // inference rounds: 0 layer by layer, 1 warp MMA, 2 tcgen05 pipeline
   int* tc_err = nullptr;                     // the handle's device error word (tensor-core waits)
+  int n_sm = 1;                              // SMs of the device
   // workspace
   int64_t cap_n = 0, cap_e = 0;
   uint32_t* cnt = nullptr;
@@ -1722,7 +1725,7 @@ int ensure_workspace(sph_learned* L, int64_t n, int64_t E) {
 
 template <int NO, int K, bool MASK = false>
 void dense(int64_t M, const bf16* X, int ldx, const bf16* W, float* of, int ldf, int nf, int accum,
-           bf16* ob, int ldo, int col0, int nb, int relu, const bf16* mask, int ldm, int* err, cudaStream_t s) {
+           bf16* ob, int ldo, int col0, int nb, int relu, const bf16* mask, int ldm, const sph_learned* L, cudaStream_t s) {
   static_assert(K % 16 == 0, "K in MMA steps of 16");
   if (M == 0) return;
   // rows move as 16-byte pieces, results as 16-byte pieces: strides and column ranges must
@@ -1737,9 +1740,10 @@ void dense(int64_t M, const bf16* X, int ldx, const bf16* W, float* of, int ldf,
   // where an SM has no second one (64 outputs, K = 80: 498 tiles 12.4 us with one CTA an SM, 13.6
   // with two, 14.5 with four; 784 tiles 16.5, 16.5, 18.6; 5,000 tiles 69, 58, 62; 21,094 tiles 264, 219, 220).
   const int64_t tiles = (M + 127) / 128;
-  const unsigned grid = (unsigned)std::min<int64_t>(tiles, tiles <= 8 * 152 ? 152 : 2 * 152);
+  const int64_t sms = L->n_sm;
+  const unsigned grid = (unsigned)std::min<int64_t>(tiles, tiles <= 8 * sms ? sms : 2 * sms);
   k_dense<NO, K, MASK><<<grid, 128, dense_smem<NO>(K), s>>>(M, X, ldx, W, of, ldf, nf, accum, ob, ldo, col0, nb, relu,
-                                                            mask, ldm, err);
+                                                            mask, ldm, L->tc_err);
 }
 
 // The weight gradients pending for one launch of k_reduce_partials
@@ -1809,20 +1813,17 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
   const bool fused = L->fused == 1 && !train;
   const bool piped = L->fused == 2 && !train;
   // encoder: H = relu(U W_enc^T); H0 keeps h0 for the encoder's backward
-  dense<64, 16>(n, L->U, 16, Wl(L, L_ENC), L->H, F, F, 0, nullptr, 0, 0, 0, 1, nullptr, 0, L->tc_err, s);
+  dense<64, 16>(n, L->U, 16, Wl(L, L_ENC), L->H, F, F, 0, nullptr, 0, 0, 0, 1, nullptr, 0, L, s);
   if (train) cudaMemcpyAsync(L->H0, L->H, sizeof(float) * n * F, cudaMemcpyDeviceToDevice, s);
   for (int r = 0; r < ROUNDS; ++r) {
     if (fused) {
       if (n == 0) continue;
-      int sms = 1, dev = 0;
-      cudaGetDevice(&dev);
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
       // runs of equal node counts, a whole number of them per warp where possible; short runs
       // where the warps would outnumber them, down to a half tile of edges
-      const int64_t slots = (int64_t)sms * kFuseWarps;
+      const int64_t slots = (int64_t)L->n_sm * kFuseWarps;
       const int64_t per = (n + slots * kFuseRun - 1) / (slots * kFuseRun);
       const int run = (int)std::max<int64_t>(kFuseRunMin, (n + slots * per - 1) / (slots * per));
-      const unsigned grid = (unsigned)std::min<int64_t>((n + run - 1) / run, sms);
+      const unsigned grid = (unsigned)std::min<int64_t>((n + run - 1) / run, L->n_sm);
       // node states ping-pong between H and H0 (H0 is only kept for training's backward), the
       // templates between T and T2; the last round leaves the decoder's input rows instead
       const float* hin = (r & 1) ? L->H0 : L->H;
@@ -1842,11 +1843,8 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
       auto tmpl = d == 2 ? k_node_templates<7> : k_node_templates<9>;
       tmpl<<<blocks_for((n + 1) * 10 + n * 8), 256, 0, s>>>(n, L->H, L->T, L->XN[r]);
       if (n > 0) {
-        int sms = 1, dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         // runs of equal node counts, a whole number of them per CTA where possible
-        const int64_t slots = 2 * (int64_t)sms;
+        const int64_t slots = 2 * (int64_t)L->n_sm;
         const int64_t per = (n + slots * kWsRun - 1) / (slots * kWsRun);
         const int run = (int)std::max<int64_t>(1, (n + slots * per - 1) / (slots * per));
         const int64_t runs = (n + run - 1) / run;
@@ -1855,21 +1853,21 @@ void forward(sph_handle* h, sph_learned* L, cudaStream_t s, bool train) {
         kern<<<grid, kWsThreads, ws_smem(), s>>>(n, run, L->off, L->XS, L->enbr, L->T, Wl(L, L_E1), Wl(L, L_E2),
                                                  inv_nbar, L->XN[r], L->tc_err);
       }
-      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L, s);
+      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
     } else {
       if (E > 0) k_edge_rows<<<blocks_for(E * 10), 256, 0, s>>>(E, fe, L->XS, L->enbr, L->H, L->XE[r]);
-      dense<64, 80>(E, L->XE[r], 80, Wl(L, L_E1), nullptr, 0, 0, 0, L->A1[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64, 80>(E, L->A1[r], 80, Wl(L, L_E2), L->Mbuf, F, F, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 80>(E, L->XE[r], 80, Wl(L, L_E1), nullptr, 0, 0, 0, L->A1[r], 80, 0, F, 1, nullptr, 0, L, s);
+      dense<64, 80>(E, L->A1[r], 80, Wl(L, L_E2), L->Mbuf, F, F, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
       k_segsum<<<blocks_for(n * F), 256, 0, s>>>(n, L->off, L->Mbuf, L->H, inv_nbar, L->XN[r]);
-      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+      dense<64, 144>(n, L->XN[r], 144, Wl(L, L_N1), nullptr, 0, 0, 0, L->A2[r], 80, 0, F, 1, nullptr, 0, L, s);
+      dense<64, 80>(n, L->A2[r], 80, Wl(L, L_N2), L->H, F, F, 1, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
     }
   }
   // the fused rounds leave the decoder's input rows
   if (!fused) k_rows_bf16<<<blocks_for(n * F), 256, 0, s>>>(n, F, L->H, F, L->XD, 80);
-  dense<64, 80>(n, L->XD, 80, Wl(L, L_D1), nullptr, 0, 0, 0, L->A3, 80, 0, F, 1, nullptr, 0, L->tc_err, s);
-  dense<16, 80>(n, L->A3, 80, Wl(L, L_D2), L->Y, 16, 16, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+  dense<64, 80>(n, L->XD, 80, Wl(L, L_D1), nullptr, 0, 0, 0, L->A3, 80, 0, F, 1, nullptr, 0, L, s);
+  dense<16, 80>(n, L->A3, 80, Wl(L, L_D2), L->Y, 16, 16, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
 }
 
 void backward(sph_handle* h, sph_learned* L, cudaStream_t s) {
@@ -1882,21 +1880,21 @@ void backward(sph_handle* h, sph_learned* L, cudaStream_t s) {
   DwPending p;
   // decoder; dZe is the edge buffer (at least n rows)
   dense_dw<16, 80>(L, p, L_D2, n, L->dYb, 16, L->A3, 80, s);
-  dense<80, 16, true>(n, L->dYb, 16, WTl(L, L_D2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A3, 80, L->tc_err, s);
+  dense<80, 16, true>(n, L->dYb, 16, WTl(L, L_D2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A3, 80, L, s);
   dense_dw<64, 80>(L, p, L_D1, n, L->dZe, F, L->XD, 80, s);
-  dense<80, 64>(n, L->dZe, F, WTl(L, L_D1), L->dH, F, F, 0, L->dZn, F, 0, F, 0, nullptr, 0, L->tc_err, s);
+  dense<80, 64>(n, L->dZe, F, WTl(L, L_D1), L->dH, F, F, 0, L->dZn, F, 0, F, 0, nullptr, 0, L, s);
   for (int r = ROUNDS - 1; r >= 0; --r) {
     // h_new = h + W_n2 [relu(W_n1 XN), 1]; dZn = bf16(dh)
     dense_dw<64, 80>(L, p, L_N2, n, L->dZn, F, L->A2[r], 80, s);
     bf16* dZ2 = L->dZe;
-    dense<80, 64, true>(n, L->dZn, F, WTl(L, L_N2), nullptr, 0, 0, 0, dZ2, F, 0, F, 0, L->A2[r], 80, L->tc_err, s);
+    dense<80, 64, true>(n, L->dZn, F, WTl(L, L_N2), nullptr, 0, 0, 0, dZ2, F, 0, F, 0, L->A2[r], 80, L, s);
     dense_dw<64, 144>(L, p, L_N1, n, dZ2, F, L->XN[r], 144, s);
-    dense<144, 64>(n, dZ2, F, WTl(L, L_N1), L->dXN, 144, 144, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+    dense<144, 64>(n, dZ2, F, WTl(L, L_N1), L->dXN, 144, 144, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
     if (E > 0) k_edge_back<<<blocks_for(E * (F / 8)), 256, 0, s>>>(E, L->esrc, L->dXN, inv_nbar, L->dM);
     dense_dw<64, 80>(L, p, L_E2, E, L->dM, F, L->A1[r], 80, s);
-    dense<80, 64, true>(E, L->dM, F, WTl(L, L_E2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A1[r], 80, L->tc_err, s);
+    dense<80, 64, true>(E, L->dM, F, WTl(L, L_E2), nullptr, 0, 0, 0, L->dZe, F, 0, F, 0, L->A1[r], 80, L, s);
     dense_dw<64, 80>(L, p, L_E1, E, L->dZe, F, L->XE[r], 80, s);
-    dense<80, 64>(E, L->dZe, F, WTl(L, L_E1), L->dXE, 80, 80, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L->tc_err, s);
+    dense<80, 64>(E, L->dZe, F, WTl(L, L_E1), L->dXE, 80, 80, 0, nullptr, 0, 0, 0, 0, nullptr, 0, L, s);
     k_gather_dh<<<blocks_for(n * 32), 256, 0, s>>>(n, fe, L->off, L->enbr, L->erev, L->dXE, L->dXN,
                                                    r == 0 ? L->H0 : nullptr, L->dH, L->dZn);
     if (r > 0) flush_dw(L, p, s);
@@ -1992,6 +1990,12 @@ int sph_learned_create(int32_t dim, const float* weights, sph_learned** out) {
   sph_learned* L = new sph_learned();
   *out = L;
   L->dim = dim;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&L->n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return lfail(L, SPH_E_CUDA, "no CUDA device");
+  }
   if (!nalloc(L, &L->w32, kWeights) || !nalloc(L, &L->m, kWeights) || !nalloc(L, &L->v, kWeights) ||
       !nalloc(L, &L->grad, kWeights) || !nalloc(L, &L->wb, kWeights) || !nalloc(L, &L->wbt, kWeights))
     return lfail(L, SPH_E_OOM, "device allocation of the weights failed");
