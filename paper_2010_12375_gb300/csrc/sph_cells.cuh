@@ -1,5 +1,5 @@
 // Device helpers of the configuration update shared by the per-launch kernels
-// (sph_cells.cu) and the one-launch step (sph_fused_step.cu).
+// (sph_cells.cu) and the one-launch step (sph_fused_step.cuh).
 #pragma once
 #include "sph_kernels.h"
 

@@ -1,5 +1,5 @@
 // Per-particle density summation and viscous acceleration (once per advection step), shared
-// by the per-launch kernels (sph_physics.cu) and the one-launch step (sph_fused_step.cu).
+// by the per-launch kernels (sph_physics.cu) and the one-launch step (sph_fused_step.cuh).
 //
 // LPP lanes share one particle: lane `sub` evaluates quads sub, sub + LPP, ... of its row and
 // the terms are added in row order through shared memory, so the sums are those of one lane

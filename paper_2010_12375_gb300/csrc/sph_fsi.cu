@@ -1020,7 +1020,6 @@ k_solid_steps(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict__ ct
   }
 }
 
-// The solid's state in the caller's order (perm: internal index -> caller's), FP64.
 // The same steps for a 2D solid of which every thread group holds one particle (four lanes a
 // particle, at most kRegRow reference neighbours and kRegThreads / 4 particles a block): a
 // step is then a chain of dependent accesses, two exchanges between neighbours, so everything
@@ -1313,6 +1312,7 @@ k_solid_steps_reg(const Inst I, SolidMat M, SolidPtrs S, const Ctrl* __restrict_
   cl.sync();                               // no block leaves while another may still send to it
 }
 
+// The solid's state in the caller's order (perm: internal index -> caller's), FP64.
 __global__ void k_solid_export(int64_t ns, int d, const int* __restrict__ perm, const int4* __restrict__ X,
                                const float4* __restrict__ V, const float4* __restrict__ force,
                                const float* __restrict__ F, double lo0, double lo1, double lo2, double dq,
@@ -1487,11 +1487,11 @@ bool choose_cluster(sph_solid* s, int max_row) {
   return false;
 }
 
-// Whether the chosen launch shape lets a 2D solid's steps run in registers.
-// shared memory of k_solid_steps_reg: the copies of every particle's P B0 and v
+// Shared memory of k_solid_steps_reg: the copies of every particle's P B0 and v.
 constexpr int kRegCopies = sph::kRegThreads / sph::kRegLanes;   // particles of a block, at most
 size_t reg_copy_bytes(const sph_solid* s) { return (size_t)s->cluster * s->per_block * 24; }
 
+// Whether the chosen launch shape lets a 2D solid's steps run in registers.
 bool reg_steps_fit(const sph_solid* s) {
   if (s->dim != 2 || s->cluster > 16 || s->lanes != sph::kRegLanes || s->row > sph::kRegRow || s->threads < s->per_block * s->lanes ||
       s->per_block * s->lanes > sph::kRegThreads || s->threads > sph::kRegThreads)

@@ -117,9 +117,7 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 
 // 16-byte pieces of an R-row operand, [R x K] row-major in global memory (row stride ld
 // elements), into the core-matrix layout: piece (row, kc) by lane (row % 8) + 8 (kc % 4) of a
-// warp-sized block of 8 rows x 4 pieces. Rows at or past rows_valid are zero. ASYNC: by
-// cp.async (zero-filled past rows_valid), completed by the caller's cp_async_wait_all.
-template <bool ASYNC>
+// warp-sized block of 8 rows x 4 pieces. Rows at or past rows_valid are zero.
 __device__ __forceinline__ void load_operand(unsigned char* dst, int R, int K, const bf16* __restrict__ src,
                                              int64_t ld, int64_t rows_valid) {
   const int KC = K / 8, KB = (KC + 3) / 4;           // pieces per row, 4-piece groups
@@ -128,20 +126,15 @@ __device__ __forceinline__ void load_operand(unsigned char* dst, int R, int K, c
   for (int blk = threadIdx.x >> 5; blk < blocks; blk += blockDim.x >> 5) {
     const int r = (blk / KB) * 8 + (lane & 7), kc = (blk % KB) * 4 + (lane >> 3);
     if (kc >= KC) continue;
-    const bool valid = r < rows_valid;
-    unsigned char* d = dst + tc::core_offset(R, r, kc * 8);
-    if (ASYNC) {
-      cp_async16(d, src + (valid ? (int64_t)r * ld : 0) + kc * 8, valid);
-    } else {
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (valid) v = *reinterpret_cast<const uint4*>(src + (int64_t)r * ld + kc * 8);
-      *reinterpret_cast<uint4*>(d) = v;
-    }
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r < rows_valid) v = *reinterpret_cast<const uint4*>(src + (int64_t)r * ld + kc * 8);
+    *reinterpret_cast<uint4*>(dst + tc::core_offset(R, r, kc * 8)) = v;
   }
 }
 
-// The same by the four warps of k_dense with the shape known when compiled: every copy of a
-// lane is issued without a division or a wait for the one before.
+// The same by the four warps of k_dense with the shape known when compiled, by cp.async
+// (completed by the caller's cp_async_wait_all): every copy of a lane is issued without a
+// division or a wait for the one before.
 template <int R, int K>
 __device__ __forceinline__ void load_tile(unsigned char* dst, const bf16* __restrict__ src, int ld, int rows_valid) {
   constexpr int KC = K / 8, KB = (KC + 3) / 4, kBlocks = (R / 8) * KB;
@@ -1115,8 +1108,8 @@ k_edge_round_ws(int64_t n, int run, const uint32_t* __restrict__ off, const bf16
   float* carry_out = carry_in + 64;                   // ... and of the node it leaves open
   uint32_t* soff = reinterpret_cast<uint32_t*>(carry_out + 64);   // the run's edge offsets
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
-  load_operand<false>(sW1, 64, 80, W1, 80, 64);
-  load_operand<false>(sW2, 64, 80, W2, 80, 64);
+  load_operand(sW1, 64, 80, W1, 80, 64);
+  load_operand(sW2, 64, 80, W2, 80, 64);
   if (tid == 0) {
     for (int s = 0; s < kWsStages; ++s) {
       ws_bar_init(&S.full[s], 1);
