@@ -20,10 +20,12 @@
 //  - reordered records go to the half-step arrays, the search reads them there and writes
 //    each particle's own record back, so no pass copies them;
 //  - the scan of the cell counts leaves the counts zero for the next step.
-// A step after the first (of a launch or, with `follow`, of a call) does not begin once the
-// status holds an error: not its hash, which would count on top of what a launch whose barrier
-// gave up left in the counts. Until every block has passed that test the errors of a step's own
-// hash wait in StepCtl, so that all blocks decide alike.
+// A step after the first (of a launch or, with `follow`, of a call) goes no further than its hash
+// once the status holds an error: the scan and the scatter would build on counts that a launch
+// whose barrier gave up has left half filled, and on barriers whose arrivals it has left counted.
+// The status is read beside the hash and looked at behind its barrier, where it costs nothing (a
+// test before the hash took 2 us a step). The errors of a step's own hash wait in StepCtl until
+// then, so that all blocks see the same status.
 // Every sum adds the terms the per-launch kernels add in their order: the state is identical
 // to theirs bit for bit, whatever the launch configuration.
 // A further step of the 2D dam break takes 55 us at 3,200 particles and 158 us at 100,352 (132
@@ -289,28 +291,23 @@ k_fused_step(const __grid_constant__ Buffers b, int n_steps, int clear_counts, i
   unsigned target = 0;
 
   if (threadIdx.x == 0) C = b.ctrl[0];
+  if (clear_counts) {
+    for (int64_t k = tid; k < b.n_cells; k += threads) b.count[k] = 0u;
+    if (!grid_barrier(&c->count, target, g)) return;
+  }
   for (int st = 0; st < n_steps; ++st) {
-    int4 p = tid < n ? b.PS[tid] : make_int4(0, 0, 0, 0);   // on its way while the status is read
-    if (st > 0 || follow) {
-      if (threadIdx.x == 0) failed = *(volatile int*)&g->err;
-      __syncthreads();
-      if (failed) {                              // an earlier step failed
-        if (st == 0) return;                     // every block: nothing has been touched
-        break;
-      }
-    }
-    if (st == 0 && clear_counts) {
-      for (int64_t k = tid; k < b.n_cells; k += threads) b.count[k] = 0u;
-      if (!grid_barrier(&c->count, target, g)) return;
-    }
     // ---- cells: hash, scan, sort by (cell, id)
+    if (threadIdx.x == 0) failed = st > 0 || follow ? *(volatile int*)&g->err : 0;
     for (int64_t i = tid; i < n; i += threads) {
-      if (i != tid) p = b.PS[i];
-      const uint32_t cell = hash_cell<D>(I, p, i, &c->found);
+      const uint32_t cell = hash_cell<D>(I, b.PS[i], i, &c->found);
       b.cell[i] = cell;
       b.rank[i] = atomicAdd(&b.count[cell], 1u);
     }
     if (!grid_barrier(&c->count, target, g)) return;
+    if (failed) {                                // an earlier step failed: every block leaves, its
+      if (st == 0) return;                       // counters to the host (this barrier may not have held
+      break;                                     // the blocks together, after a launch that gave up)
+    }
     uint32_t sum = 0, total;
     for (int64_t k = c0 + 4 * threadIdx.x; k < c1; k += 4 * blockDim.x) {
       const uint4 v = load4(b.count, k, c1);

@@ -140,7 +140,7 @@ cudaError_t launch_substeps_persistent(const Buffers& b, cudaStream_t s, int* gr
 // n_steps whole advection steps of a handle of one tank in one cooperative launch (not with
 // the frozen-geometry or half-pair evaluation, nor a solid)
 // (clear_counts: the cell counts are not all zero yet; follow: the launch goes on with the
-// steps of the one before it, and leaves everything as it is if that one failed)
+// steps of the one before it, and leaves the state as it is if that one failed)
 cudaError_t launch_fused_2d(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);
 cudaError_t launch_fused_2dp(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);   // a periodic axis
 cudaError_t launch_fused_3d(const Buffers& b, int n_steps, int clear_counts, int follow, cudaStream_t s);
