@@ -39,13 +39,13 @@ UNIT = "particle-substeps/s"
 # scaled to the benchmark's particle count (the traffic is per particle: state records plus
 # its neighbour row). Valid only for the kernel sources whose hash is recorded with it, in
 # the launch form it was captured in.
-TRAFFIC_BYTES_PER_PARTICLE = 389.35
-TRAFFIC_SOURCE_HASH = "22697809884256d0"
+TRAFFIC_BYTES_PER_PARTICLE = 389.30
+TRAFFIC_SOURCE_HASH = "071e23d5ec3ffb1c"
 TRAFFIC_ROW_FORM = True         # captured launch form: row tasks (True) or one thread a particle
 ROW_BLOCK = 896                 # block of the row-task launch form
 # Pipe utilisation of the same kernel from the same full capture (% of peak while active):
 # the FP32 FMA pipe (scalar and packed FP32 FMA/MUL/ADD) and the L1 data pipe that bounds it
-PR_PIPES = {"fp32_fma_pipe": 0.569, "l1_data_pipe": 0.868, "issue_active": 0.605}
+PR_PIPES = {"fp32_fma_pipe": 0.567, "l1_data_pipe": 0.864, "issue_active": 0.60}
 
 
 # DRAM bytes (read + write) per particle of one diffusion stage launch, from the ncu capture
